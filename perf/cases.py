@@ -279,3 +279,128 @@ def tolerance(case):
     # one of them may be a tie within the rounding of its logits: another expert of the same weight then stands in.
     many = case["seqs"] * case["branches"] * case["block"] >= TILE_MIN_ROWS
     return {"rel": 7e-3, "max": 0.9 if many else 0.06}
+
+
+# ---- what run returns, in 64 bits -----------------------------------------------------------------------------------
+def _classes(c, states, conf):
+    """True for rows that are computed, and for those among them that choose in the first round, [S, B, L] each: Eq. 4 with
+    make_config's defaults (threshold 0.7, a distance of at most L_hot, the position in front of the block decoded)."""
+    S, nb, L = states.shape
+    decoded = np.concatenate([np.ones((S, nb, 1), bool), states != W.TOK_MASKED], axis=2)
+    near_by = np.abs(np.arange(L)[:, None] - np.arange(-1, L)[None, :]) <= c["L_hot"]
+    near = (decoded[:, :, None, :] & near_by).any(axis=3)
+    computed = (states != W.TOK_CACHED) | (not c["flags"] & B.TEAM_F_DCD)
+    first = computed & ((states != W.TOK_MASKED) | (conf > np.float32(0.7)) | near | (not c["flags"] & B.TEAM_F_LAC))
+    empty = ~first.any(axis=(1, 2))
+    first[empty] = computed[empty]
+    return computed, first
+
+
+def _layer64(c, weights, x, states, conf, y):
+    """The layer on x [T, H]; rows that are not computed keep what y holds.  Experts are chosen on the 64-bit logits."""
+    wr, wg, wu, wd = weights
+    computed, first = _classes(c, states.reshape(c["seqs"], -1, c["block"]), conf.reshape(c["seqs"], -1, c["block"]))
+    S, T = c["seqs"], x.shape[0]
+    computed, first = (torch.as_tensor(a.reshape(S, -1)).cuda() for a in (computed, first))
+    x64 = x.double()
+    logits = x64 @ wr.double().T
+    own = torch.zeros(logits.shape, dtype=torch.bool, device="cuda").scatter_(1, logits.topk(c["k"], dim=1).indices, True).view(S, -1, c["E"])
+    allowed = (own & first[:, :, None]).any(dim=1, keepdim=True) | first[:, :, None]
+    z, idx = logits.masked_fill(~allowed.expand_as(own).reshape(T, -1), -float("inf")).topk(c["k"], dim=1)
+    w = torch.softmax(z, dim=1)          # the softmax over all experts, renormalised over the chosen ones
+    rows = computed.reshape(-1)
+    y[rows] = 0
+    for e in range(c["E"] + c["ns"]):
+        if e < c["E"]:
+            t, j = torch.nonzero((idx == e) & rows[:, None], as_tuple=True)
+            share = w[t, j]
+        else:
+            t = torch.nonzero(rows)[:, 0]
+            share = torch.ones(t.numel(), dtype=torch.float64, device="cuda")
+        if t.numel():
+            a = torch.nn.functional.silu(x64[t] @ wg[e].double().T) * (x64[t] @ wu[e].double().T)
+            y.index_add_(0, t, share[:, None] * (a @ wd[e].double().T))
+    return y
+
+
+def _accept(c, seq, pred, conf):
+    """One acceptance step of a sequence (threshold 0.95): seq holds token, state and the speculated (position, token)
+    pairs; pred and conf are [branches, L].  Returns the states and the confidences of the next pass's rows."""
+    token, state, spec = seq["token"], seq["state"], seq["spec"]
+    carries = {0: (), 1: (0,), 2: (1,), 3: (0, 1)}
+
+    def sure(b, i):
+        return i < len(spec) and pred[b, spec[i][0]] == spec[i][1] and conf[b, spec[i][0]] > np.float32(0.95)
+
+    chain = [0]
+    if sure(0, 0):
+        chain += [1, 3] if sure(1, 1) else [1]
+    elif sure(0, 1):
+        chain += [2, 3] if sure(2, 0) else [2]
+    new = {}
+    for b in chain:
+        held = [spec[i][0] for i in carries[b] if i < len(spec)]
+        for i in carries[b]:
+            if i < len(spec):
+                new.setdefault(*spec[i])
+        for p in range(c["block"]):
+            if state[p] == W.TOK_MASKED and p not in held and conf[b, p] > np.float32(0.95):
+                new.setdefault(p, int(pred[b, p]))
+    state[state == W.TOK_NEW] = W.TOK_CACHED
+    for p, t in new.items():
+        token[p], state[p] = t, W.TOK_NEW
+    last = chain[-1]
+    masked = sorted(np.flatnonzero(state == W.TOK_MASKED), key=lambda p: (-conf[last, p], p))
+    seq["spec"] = [(int(p), int(pred[last, p])) for p in masked[:2]] if c["branches"] == 4 else []
+    states = np.tile(state, (c["branches"], 1))
+    for b in range(c["branches"]):
+        for i in carries[b]:
+            if i < len(seq["spec"]):
+                states[b, seq["spec"][i][0]] = W.TOK_NEW
+    return states, np.where(states == W.TOK_MASKED, conf[last], np.float32(1))
+
+
+def _attn64(c, s):
+    """Every layer of an attention state: the outputs and the in-block caches after the insertion."""
+    S, L, rep, d = c["seqs"], c["block"], c["n_heads"] // c["n_kv"], c["head_dim"]
+    states = s["st"]["tok_state"].view(S, -1, L)
+    computed = (states != W.TOK_CACHED) | (not c["flags"] & B.TEAM_F_DCD)
+    out = torch.zeros(s["out"].shape, dtype=torch.float64, device="cuda")
+    caches = [s["k_block"].double(), s["v_block"].double()]
+    for n in range(c["layers"]):
+        fresh = [s[f][n].double().view(S, -1, L, c["n_kv"], d) for f in ("k_new", "v_new")]
+        for q in range(S):
+            length = int(s["prefix_len"][q])
+            for b in range(states.shape[1]):
+                use = computed[q, b]
+                k, v = (torch.cat([s[p][n, q, :length].double(), torch.where(use[:, None, None], f[q, b], cache[n, q])])
+                        for p, f, cache in zip(("k_prefix", "v_prefix"), fresh, caches))
+                rows = (q * states.shape[1] + b) * L + torch.nonzero(use)[:, 0]
+                query = s["q"][n][rows].double().view(-1, c["n_kv"], rep, d)
+                p = torch.softmax(torch.einsum("tgrd,jgd->tgrj", query, k) / d ** 0.5, dim=-1)
+                out[n, rows] = torch.einsum("tgrj,jgd->tgrd", p, v).reshape(-1, c["n_heads"], d)
+        keep = (computed[:, 0] & (states[:, 0] != W.TOK_MASKED))[:, :, None, None]
+        for cache, f in zip(caches, fresh):
+            cache[n] = torch.where(keep, f[:, 0], cache[n])
+    return out, caches[0], caches[1]
+
+
+def exact(case, seed):
+    c = dict(case)
+    s = prepare(case, seed)
+    if c["kind"] == "attn":
+        return _attn64(c, s)
+    weights = W.device_layer_weights(_shape(c), seed, "cuda")
+    y = torch.zeros(s["y"].shape, dtype=torch.float64, device="cuda")
+    if c["kind"] != "decode":
+        st = _step_host(c, seed)
+        return _layer64(c, weights, s["x"].cuda(), st["tok_state"], st["conf"], y)
+    S, nb, L = c["seqs"], c["branches"], c["block"]
+    seqs = [dict(token=np.full(L, -1, np.int32), state=np.zeros(L, np.uint8), spec=[]) for _ in range(S)]
+    states, conf = np.zeros((S, nb, L), np.uint8), np.zeros((S, nb, L), np.float32)
+    for p in range(c["passes"]):
+        y = _layer64(c, weights, s["x"][p], states, conf, y)
+        pred, seen = s["pred"][p].cpu().numpy(), s["conf"][p].cpu().numpy()
+        for i, q in enumerate(seqs):
+            states[i], conf[i] = _accept(c, q, pred[i], seen[i])
+    return (y, np.stack([q["token"] for q in seqs]), np.stack([q["state"] for q in seqs]), states.reshape(-1), conf.reshape(-1))
