@@ -1,10 +1,11 @@
 // Router kernels (Algorithm 1 "Router"; Sec. 4.1 for which rows are computed).
 //
-//  k_router_logits : logits[t,e] = sum_h x[t,h] * W_r[e,h] in fp32.  The work is split over
-//                    experts (one warp per expert, 128-bit loads of the expert's row) and over
-//                    tiles of 8 rows whose activations sit in shared memory, so that with a
-//                    handful of rows the 4*E*H bytes of router weights are still pulled by many SMs.
-//                    The same launch zeroes the output rows the expert kernel will accumulate into.
+//  k_router_logits_small : up to 8 rows: logits[t,e] = sum_h x[t,h] * W_r[e,h] in fp32, spread as widely as possible.
+//  k_router_logits_mma   : more rows, bf16 activations: the same sums on the tensor cores, weights as three bf16 parts.
+//  k_router_logits : more rows, fp32 activations (and hidden sizes the small kernel does not hold).  The work is split
+//                    over experts (one warp per expert, 128-bit loads of the expert's row) and over tiles of 8 rows
+//                    whose activations sit in shared memory.
+//                    Each of them also zeroes the output rows the expert kernel will accumulate into.
 //  k_router_topk   : one warp per row: softmax over all experts, plain top-k by warp shuffles,
 //                    renormalised weights, decision margin (team_route's outputs).
 #include <mutex>
@@ -17,9 +18,8 @@ namespace team {
 constexpr int kRowTile = 8;       // rows per CTA in the logits kernel
 constexpr int kExpertsPerCta = 8; // one warp each
 
-template <typename XT>
 __global__ void __launch_bounds__(kExpertsPerCta * 32)
-k_router_logits(const XT* __restrict__ x, const float* __restrict__ w_router, const uint8_t* __restrict__ tok_state,
+k_router_logits(const float* __restrict__ x, const float* __restrict__ w_router, const uint8_t* __restrict__ tok_state,
                 float* __restrict__ logits, float* __restrict__ y_zero, Dims d, int flags) {
   extern __shared__ __align__(16) float s_x[];   // [kRowTile][H]
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the selection kernel may stage its inputs meanwhile
@@ -38,18 +38,8 @@ k_router_logits(const XT* __restrict__ x, const float* __restrict__ w_router, co
   for (int i = 0; i < kBatch; ++i)
     wv[i] = lane + 32 * i < n4 ? __ldg(wrow + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
 
-  if constexpr (sizeof(XT) == 2) {
-    const uint2* src = reinterpret_cast<const uint2*>(x + (size_t)t0 * H);
-    for (int i = tid; i < nt * H / 4; i += blockDim.x) {
-      const uint2 v = __ldg(src + i);
-      const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.x));
-      const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.y));
-      reinterpret_cast<float4*>(s_x)[i] = make_float4(a.x, a.y, b.x, b.y);
-    }
-  } else {
-    const float4* src = reinterpret_cast<const float4*>(x + (size_t)t0 * H);
-    for (int i = tid; i < nt * H / 4; i += blockDim.x) reinterpret_cast<float4*>(s_x)[i] = __ldg(src + i);
-  }
+  const float4* src = reinterpret_cast<const float4*>(x + (size_t)t0 * H);
+  for (int i = tid; i < nt * H / 4; i += blockDim.x) reinterpret_cast<float4*>(s_x)[i] = __ldg(src + i);
   for (int i = nt * H + tid; i < kRowTile * H; i += blockDim.x) s_x[i] = 0.f;
 
   // Output rows of computed tokens start from zero (the expert kernel adds partial sums into them);
@@ -102,93 +92,148 @@ k_router_logits(const XT* __restrict__ x, const float* __restrict__ w_router, co
 }
 
 
-// Many rows (bf16 activations): a register-tiled fp32 FMA kernel.  A CTA takes 16 rows x 32 experts; the rows sit in
-// shared memory as bf16 (widened exactly on use); warp w takes experts 4w .. 4w+3 of the tile, its lanes stride
-// the hidden dimension four elements at a time (128-bit weight loads, 512 contiguous bytes per warp and expert)
-// and keep 4 x 16 accumulators each, so that one weight load feeds 16 rows and one row load feeds 4 experts.  The
-// 64 per-lane partial sums of a warp are reduced with a transposing butterfly (62 shuffles instead of 320).
-constexpr int kTiledRows = 16;
-constexpr int kTiledExperts = 32;      // per CTA: 8 warps x 4
+// More than eight rows of bf16 activations: x W_r^T on the tensor cores, with the accuracy of fp32.
+//
+// An fp32 weight is exactly the sum of three bf16 numbers (8 + 8 + 8 mantissa bits, split by truncation) and a product
+// of two bf16 numbers is exact in fp32.  The tensor core truncates while it accumulates (chains over the whole hidden
+// dimension were off by 1.05e-6 against 64 bits), so a chain is the three parts of one fragment of 16 elements, the
+// smallest first, and the fragments are added with rounded fp32 additions: 1.08e-7, against 1.57e-7 of the fp32 FMA
+// kernels that this one replaced (2-norm, 16 to 2048 rows, hidden 2048).  Measured at hidden 2048 x 128 experts, in the
+// call, end to end: 2048 rows 48 -> 29 us, 1024 rows 26 -> 17, 128 rows 11 -> 6; the mma.sync rate and the reads of x
+// and W from L2 are what is left.  mma.sync and not tcgen05: a tcgen05 chain cannot be cut every 16 elements.
+//
+// A warp owns MT x 16 rows by NT x 8 experts and every eighth block of 32 hidden elements.  Lane (g, c) of a fragment
+// takes elements 8c .. 8c+7 of its row's block -- 16 contiguous bytes of x, 32 of W -- which is a permutation of the
+// k index common to both operands, so fragments come straight from global memory: no staging, no barrier before the
+// first mma, the next blocks are in flight while the current ones are multiplied.  The eight warps' partial tiles meet
+// in shared memory and are summed in warp order.
+constexpr int kMmaWarps = 8;
 
-__device__ __forceinline__ void butterfly32(float (&v)[32], int lane) {
-  // after the five steps lane l holds the warp-wide sum of entry l
-#pragma unroll
-  for (int half = 16; half >= 1; half >>= 1) {
-    const bool upper = (lane & half) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const float keep = upper ? v[i + half] : v[i];
-      const float send = upper ? v[i] : v[i + half];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-    }
-  }
+// The two truncated bf16 halves of a pair (low half = a), and the pair's exact remainders.
+__device__ __forceinline__ uint32_t split_pair(float& a, float& b) {
+  const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+  a -= __uint_as_float(ua & 0xffff0000u);
+  b -= __uint_as_float(ub & 0xffff0000u);
+  return __byte_perm(ua, ub, 0x7632);
 }
 
-__global__ void __launch_bounds__(256)
-k_router_logits_tiled(const __nv_bfloat16* __restrict__ x, const float* __restrict__ w_router,
-                      const uint8_t* __restrict__ tok_state, float* __restrict__ logits, float* __restrict__ y_zero,
-                      Dims d, int flags) {
-  extern __shared__ __align__(16) unsigned char s_xb[];   // [kTiledRows][H] bf16
+__device__ __forceinline__ void router_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int MT, int NT>
+__global__ void __launch_bounds__(kMmaWarps * 32, 1)
+k_router_logits_mma(const __nv_bfloat16* __restrict__ x, const float* __restrict__ w_router,
+                    const uint8_t* __restrict__ tok_state, float* __restrict__ logits, float* __restrict__ y_zero,
+                    Dims d, int flags) {
+  constexpr int R = MT * 16, N = NT * 8;
+  constexpr int U = MT * NT == 1 ? 4 : (MT * NT == 2 ? 2 : 1);      // blocks of 32 in flight beside the current ones
+  extern __shared__ __align__(16) float s_part[];                   // [warps][R][N]
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int H = d.H, T = d.T, E = d.E;
-  const int t0 = blockIdx.y * kTiledRows, nt = min(kTiledRows, T - t0);
-  const int e0 = blockIdx.x * kTiledExperts + warp * 4;
-  // stage the rows (16-byte pieces; rows beyond T are zero)
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)t0 * H);
-    uint4* dst = reinterpret_cast<uint4*>(s_xb);
-    const int n16 = nt * H / 8, all16 = kTiledRows * H / 8;
-    for (int i = tid; i < all16; i += 256) dst[i] = i < n16 ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
-  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
+  const int H = d.H, T = d.T, E = d.E, nb = H >> 5;
+  const int t0 = blockIdx.x * R, e0 = blockIdx.y * N;
+  const uint4* xr[MT][2];                                           // rows and experts past the end repeat the last one
+  const float4* wr[NT];
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) xr[m][h] = reinterpret_cast<const uint4*>(x + (size_t)min(t0 + m * 16 + h * 8 + g, T - 1) * H) + c;
+#pragma unroll
+  for (int n = 0; n < NT; ++n) wr[n] = reinterpret_cast<const float4*>(w_router + (size_t)min(e0 + n * 8 + g, E - 1) * H) + 2 * c;
+  uint4 xc[U][MT][2], xn[U][MT][2];
+  float4 wc[U][NT][2], wn[U][NT][2];
+  auto load = [&](int b0, uint4 (&xv)[U][MT][2], float4 (&wv)[U][NT][2]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int b = b0 + u * kMmaWarps;
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) wv[u][n][h] = b < nb ? __ldg(wr[n] + b * 8 + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) xv[u][m][h] = b < nb ? __ldg(xr[m][h] + b * 4) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  load(warp, xc, wc);
+  // output rows of computed tokens start from zero (the expert kernel adds partial sums into them); the CTAs of one
+  // row tile share the job
   if (y_zero != nullptr) {
+    const int nt = min(R, T - t0);
     for (int r = 0; r < nt; ++r) {
       const bool skip = (flags & TEAM_F_DCD) && tok_state[t0 + r] == TEAM_TOK_CACHED;
       if (!skip)
-        for (int i = blockIdx.x * 256 + tid; i < H; i += gridDim.x * 256) y_zero[(size_t)(t0 + r) * H + i] = 0.f;
+        for (int i = blockIdx.y * blockDim.x + tid; i < H / 4; i += gridDim.y * blockDim.x)
+          reinterpret_cast<float4*>(y_zero + (size_t)(t0 + r) * H)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+#pragma unroll 1
+  for (int b = warp; b < nb; b += kMmaWarps * U) {
+    load(b + kMmaWarps * U, xn, wn);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)                                   // elements 0-3, then 4-7 of the lane's eight
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          float4 w = wc[u][n][h];
+          uint32_t b0[3], b1[3];
+#pragma unroll
+          for (int part = 0; part < 3; ++part) {
+            b0[part] = split_pair(w.x, w.y);
+            b1[part] = split_pair(w.z, w.w);
+          }
+#pragma unroll
+          for (int m = 0; m < MT; ++m) {
+            const uint4 lo = xc[u][m][0], hi = xc[u][m][1];
+            const uint32_t a0 = h ? lo.z : lo.x, a1 = h ? hi.z : hi.x, a2 = h ? lo.w : lo.y, a3 = h ? hi.w : hi.y;
+            float t[4] = {0.f, 0.f, 0.f, 0.f};
+            router_mma(t, a0, a1, a2, a3, b0[2], b1[2]);
+            router_mma(t, a0, a1, a2, a3, b0[1], b1[1]);
+            router_mma(t, a0, a1, a2, a3, b0[0], b1[0]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[m][n][q] += t[q];
+          }
+        }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int m = 0; m < MT; ++m) { xc[u][m][0] = xn[u][m][0]; xc[u][m][1] = xn[u][m][1]; }
+#pragma unroll
+      for (int n = 0; n < NT; ++n) { wc[u][n][0] = wn[u][n][0]; wc[u][n][1] = wn[u][n][1]; }
+    }
+  }
+  float* mine = s_part + warp * R * N;
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      *reinterpret_cast<float2*>(mine + (m * 16 + g) * N + n * 8 + 2 * c) = make_float2(acc[m][n][0], acc[m][n][1]);
+      *reinterpret_cast<float2*>(mine + (m * 16 + g + 8) * N + n * 8 + 2 * c) = make_float2(acc[m][n][2], acc[m][n][3]);
+    }
   __syncthreads();
-  float acc[2][32];                    // [pair of experts][expert-in-pair * 16 + row]
+  for (int i = tid; i < R * N; i += kMmaWarps * 32) {
+    const int t = t0 + i / N, e = e0 + i % N;
+    if (t >= T || e >= E) continue;
+    float sum = 0.f;
 #pragma unroll
-  for (int g = 0; g < 2; ++g)
-#pragma unroll
-    for (int i = 0; i < 32; ++i) acc[g][i] = 0.f;
-  const float4* wrow[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) wrow[q] = reinterpret_cast<const float4*>(w_router + (size_t)min(e0 + q, E - 1) * H);
-  const int n4 = H >> 2;
-  float4 wv[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) wv[q] = __ldg(wrow[q] + lane);
-  for (int c = lane; c < n4; c += 32) {
-    float4 wn[4];
-    const int cn = c + 32 < n4 ? c + 32 : c;             // next step's weights are requested before this step's math
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wn[q] = __ldg(wrow[q] + cn);
-#pragma unroll
-    for (int r = 0; r < kTiledRows; ++r) {
-      const uint2 xb = *reinterpret_cast<const uint2*>(s_xb + ((size_t)r * H + c * 4) * 2);
-      const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&xb.x));
-      const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&xb.y));
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float a = acc[q >> 1][(q & 1) * 16 + r];
-        a = fmaf(wv[q].x, lo.x, a);
-        a = fmaf(wv[q].y, lo.y, a);
-        a = fmaf(wv[q].z, hi.x, a);
-        a = fmaf(wv[q].w, hi.y, a);
-        acc[q >> 1][(q & 1) * 16 + r] = a;
-      }
+    for (int w = 0; w < kMmaWarps; ++w) sum += s_part[w * R * N + i];
+    if (!isfinite(sum)) {
+      // an infinity or NaN among the operands (or an overflow): the remainders of an infinity are NaN, so the
+      // logit is formed again without splitting
+      sum = 0.f;
+      for (int k = 0; k < H; ++k) sum = fmaf(__ldg(w_router + (size_t)e * H + k), __bfloat162float(x[(size_t)t * H + k]), sum);
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wv[q] = wn[q];
-  }
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    butterfly32(acc[g], lane);
-    const int e = e0 + g * 2 + (lane >> 4), r = lane & 15;
-    if (e < E && r < nt) logits[(size_t)(t0 + r) * E + e] = acc[g][0];
+    logits[(size_t)t * E + e] = sum;
   }
 }
 
@@ -324,6 +369,22 @@ k_router_topk(const float* __restrict__ logits, const uint8_t* __restrict__ tok_
   if (lane == 0 && out.margin) out.margin[t] = r.margin;
 }
 
+// Tiles of the tensor-core router, largest first.  A call takes the largest one that still gives about two thirds of the
+// SMs a CTA: larger tiles split every weight fewer times and read x and W fewer times from L2, smaller ones keep more
+// SMs loading.
+struct MmaTile {
+  int rows, experts;
+  void (*kernel)(const __nv_bfloat16*, const float*, const uint8_t*, float*, float*, Dims, int);
+};
+static const MmaTile kMmaTiles[] = {{64, 32, k_router_logits_mma<4, 4>}, {32, 32, k_router_logits_mma<2, 4>},
+                                    {32, 16, k_router_logits_mma<2, 2>}, {16, 16, k_router_logits_mma<1, 2>},
+                                    {16, 8, k_router_logits_mma<1, 1>}};
+static MmaTile mma_tile(const Dims& d) {
+  for (const MmaTile& t : kMmaTiles)
+    if (((d.T + t.rows - 1) / t.rows) * ((d.E + t.experts - 1) / t.experts) >= 96) return t;
+  return kMmaTiles[4];
+}
+
 // Opt in to the dynamic shared memory the kernels need (done once per context, outside any stream capture).
 static bool small_router_ok(const Dims& d) {
   return d.T <= kRowTile && d.H % (4 * kSmallSplit) == 0 && d.H / (4 * kSmallSplit) <= 32 * kSmallMaxVec;
@@ -355,12 +416,12 @@ cudaError_t configure_router(int dtype, int hidden) {
   std::lock_guard<std::mutex> lock(mu);
   if (dev >= 0 && dev < 64 && prepared[dev][di] >= smem) return cudaSuccess;
   if (dtype == TEAM_DTYPE_F32) {
-    e = prepare_kernel(k_router_logits<float>, smem);
+    e = prepare_kernel(k_router_logits, smem);
     if (e == cudaSuccess) e = prepare_kernel(k_router_logits_small<float>, smem);
   } else {
-    e = prepare_kernel(k_router_logits<__nv_bfloat16>, smem);
-    if (e == cudaSuccess) e = prepare_kernel(k_router_logits_small<__nv_bfloat16>, smem);
-    if (e == cudaSuccess) e = prepare_kernel(k_router_logits_tiled, smem);
+    e = prepare_kernel(k_router_logits_small<__nv_bfloat16>, smem);
+    for (const MmaTile& t : kMmaTiles)
+      if (e == cudaSuccess) e = prepare_kernel(t.kernel, kMmaWarps * t.rows * t.experts * (int)sizeof(float));
   }
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_router_topk, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -381,24 +442,24 @@ cudaError_t launch_router_logits(const void* x, int dtype, const float* w_router
                                                                      tok_state, logits, y_zero, d, flags);
     return cudaGetLastError();
   }
-  // the register-tiled kernel pays off once its 16-row x 32-expert tiles fill the SMs; smaller calls keep more,
-  // smaller CTAs in flight with the 8 x 8 kernel below
-  if (dtype == TEAM_DTYPE_BF16 && ((d.T + kTiledRows - 1) / kTiledRows) * ((d.E + kTiledExperts - 1) / kTiledExperts) >= 128) {
-    dim3 grid((d.E + kTiledExperts - 1) / kTiledExperts, (d.T + kTiledRows - 1) / kTiledRows);
-    k_router_logits_tiled<<<grid, 256, (size_t)kTiledRows * d.H * 2, s>>>(static_cast<const __nv_bfloat16*>(x), w_router,
-                                                                        tok_state, logits, y_zero, d, flags);
-    return cudaGetLastError();
+  if (dtype == TEAM_DTYPE_BF16) {
+    const MmaTile t = mma_tile(d);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((d.T + t.rows - 1) / t.rows, (d.E + t.experts - 1) / t.experts);
+    cfg.blockDim = dim3(kMmaWarps * 32);
+    cfg.dynamicSmemBytes = (size_t)kMmaWarps * t.rows * t.experts * sizeof(float);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;      // the launch latency hides behind the preceding kernel
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, t.kernel, static_cast<const __nv_bfloat16*>(x), w_router, tok_state, logits, y_zero, d, flags);
   }
   dim3 grid((d.E + kExpertsPerCta - 1) / kExpertsPerCta, (d.T + kRowTile - 1) / kRowTile);
   dim3 block(kExpertsPerCta * 32);
   const size_t smem = (size_t)kRowTile * d.H * sizeof(float);
-  if (dtype == TEAM_DTYPE_F32) {
-    k_router_logits<float><<<grid, block, smem, s>>>(static_cast<const float*>(x), w_router, tok_state, logits,
-                                                     y_zero, d, flags);
-  } else {
-    k_router_logits<__nv_bfloat16><<<grid, block, smem, s>>>(static_cast<const __nv_bfloat16*>(x), w_router,
-                                                             tok_state, logits, y_zero, d, flags);
-  }
+  k_router_logits<<<grid, block, smem, s>>>(static_cast<const float*>(x), w_router, tok_state, logits, y_zero, d, flags);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,65 @@
+"""The tensor-core router (bf16 activations, more than 8 rows) against the oracle's fp64 dot products, at the edges of its
+tiles: ragged rows and experts, hidden sizes that leave warps without a block, every tile size of its dispatch."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import team_oracle as O
+from paper_2602_08404_b200 import binding as B
+from tests import _parity as P
+
+pytestmark = pytest.mark.gpu
+
+
+def _route(x, w_router, k):
+    T, H = x.shape
+    E = w_router.shape[0]
+    cfg = B.make_config(H, E, k, 64, max_rows=T, max_groups=1, dtype=B.TEAM_DTYPE_BF16)
+    ctx = B.team_create(cfg)
+    gu, dn = (torch.zeros(m * E * 64 * H, dtype=torch.bfloat16, device="cuda") for m in (2, 1))
+    B.team_set_weights(ctx, w_router, w_gu_tiles=gu, w_down_tiles=dn)
+    st = dict(tok_state=torch.zeros(T, dtype=torch.uint8, device="cuda"), conf=torch.zeros(T, device="cuda"),
+              **{n: torch.zeros(T, dtype=torch.int32, device="cuda") for n in ("pos", "group", "branch")})
+    out = {n: v for n, v in B.alloc_routing(cfg, T).items() if n in ("probs", "topk_idx", "topk_w", "margin")}
+    B.team_route(ctx, x, st, out)
+    got = B.routing_to_host(out)
+    B.team_destroy(ctx)
+    return got
+
+
+@pytest.mark.parametrize("T,H,E", [(9, 128, 9), (16, 2048, 128), (17, 1536, 97), (65, 1024, 33), (185, 1536, 96), (256, 2176, 129),
+                                   (300, 640, 250), (1000, 384, 100), (2048, 256, 128), (2047, 128, 256)])
+def test_logits_of_every_tile_size(T, H, E):
+    g = torch.Generator().manual_seed(T + H)
+    x = torch.randn((T, H), generator=g).to(torch.bfloat16)
+    w = torch.randn((E, H), generator=g) / H ** 0.5
+    k = min(8, E - 1)
+    got = _route(x.cuda(), w.cuda(), k)
+    logits, probs = O.router(x.float().numpy(), w.numpy())
+    # a logit is off by at most a few roundings of its partial sums (2^-24 each): PROBS_ATOL holds with room to spare
+    np.testing.assert_allclose(got["probs"], probs, rtol=0, atol=P.PROBS_ATOL)
+    clear = 0
+    for t in range(T):
+        take, _ = O.topk_row(logits[t], k)
+        if P.ordering_margin(logits[t], take, range(E)) > P.MARGIN:
+            assert got["topk_idx"][t].tolist() == list(take), t
+            clear += 1
+    assert clear > 0.9 * T
+
+
+def test_infinite_and_large_weights_keep_their_sums():
+    """The remainder of an infinity is not a number: such logits are formed without splitting, as plain fp32 sums."""
+    T, H, E = 20, 256, 24
+    g = torch.Generator().manual_seed(3)
+    x = torch.randn((T, H), generator=g).to(torch.bfloat16)
+    x[:, 5] = x[:, 5].abs() + 0.5
+    w = torch.randn((E, H), generator=g) / H ** 0.5
+    w[11, 5] = float("inf")
+    w[12, 5] = -float("inf")
+    w[13, 5] = 3.4e38                     # rounds up to infinity in bf16, is cut to a finite number in two parts
+    x[0, 5] = 0.5
+    got = _route(x.cuda(), w.cuda(), 2)
+    assert (got["topk_idx"][:, 0] == 11).all()
+    assert not (got["topk_idx"] == 12).any()
+    assert (got["topk_idx"][:, 1] == 13).all()
+    assert got["margin"][0] > 1e37        # row 0: 0.5 * 3.4e38 is finite and above the third choice by that much
