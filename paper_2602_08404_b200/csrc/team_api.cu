@@ -244,7 +244,7 @@ int team_create(const team_config* cfg, team_ctx** out) {
   choose_expert_kernel(ctx);
   e = team::configure_router(cfg->dtype, cfg->hidden);
   if (e == cudaSuccess) e = team::configure_select(dims_of(*cfg, cfg->max_rows));
-  if (e == cudaSuccess && ctx->can_tile) e = team::configure_experts_tile();
+  if (e == cudaSuccess && ctx->can_tile) e = team::configure_experts_tile(dims_of(*cfg, cfg->max_rows));
   if (e == cudaSuccess && ctx->can_stream) e = team::configure_experts_stream(cfg->hidden, cfg->max_rows);
   if (e != cudaSuccess) {
     delete ctx;
@@ -266,10 +266,10 @@ int team_create(const team_config* cfg, team_ctx** out) {
   const size_t o_scal = take(64), o_items = take((EN + S / 8 + 2) * sizeof(team::WorkItem));
   const size_t o_act = take(cfg->dtype == TEAM_DTYPE_F32 ? S * cfg->inter * 4 : 256);
   // the tensor-memory kernels' gathered token tiles, activation tiles and per-slot tables
-  const size_t tile_items = EN + S / ctx->tile_item_tile + 2;
-  const size_t tile_rows = ctx->can_tile ? team::experts_tile_rows(S, tile_items) : 0;
+  const size_t tile_rows = ctx->can_tile ? team::experts_tile_rows(S, EN) : 0;
   const size_t o_trow = take(tile_rows * 4 + 4), o_tw = take(tile_rows * 4 + 4);
   const size_t o_tx = take(tile_rows * cfg->hidden * 2 + 256), o_tact = take(tile_rows * cfg->inter * 2 + 256);
+  const size_t o_work = take(EN * sizeof(int4)), o_begin = take((size_t)(ctx->n_sms + 1) * sizeof(int4));
   ctx->ws_bytes = off;
   e = cudaMalloc(&ctx->ws_base, ctx->ws_bytes);
   if (e != cudaSuccess) {
@@ -302,6 +302,8 @@ int team_create(const team_config* cfg, team_ctx** out) {
   ws.tile_w = reinterpret_cast<float*>(b + o_tw);
   ws.tile_x = reinterpret_cast<__nv_bfloat16*>(b + o_tx);
   ws.tile_act = reinterpret_cast<__nv_bfloat16*>(b + o_tact);
+  ws.plan.work = reinterpret_cast<int4*>(b + o_work);
+  ws.plan.begin = reinterpret_cast<int4*>(b + o_begin);
   *out = ctx;
   return TEAM_OK;
 }
@@ -390,7 +392,7 @@ int team_select_experts(team_ctx* ctx, const team_step_state* st, team_routing* 
   cudaError_t e = team::launch_select(ctx->ws.logits, step_ptrs(st), ctx->ws, export_ptrs(out), d,
                                       policy_of(ctx->cfg, st), ctx->item_tile, true, s);
   if (e != cudaSuccess) return fail_cuda(ctx, e, "select");
-  ctx->last_launches += team::select_launches(d);
+  ctx->last_launches += team::select_launches(d, true);
   return TEAM_OK;
 }
 
@@ -408,11 +410,12 @@ int team_moe_forward(team_ctx* ctx, const void* x, const team_step_state* st, te
   if (tc && ctx->stream_path && !ctx->w.w_gate) return TEAM_ERR_ARG;
   if (tc && !ctx->stream_path && !ctx->w.w_gu_tiles) return TEAM_ERR_ARG;
   if (!tc && !ctx->w.w_gate) return TEAM_ERR_ARG;
-  // The resident few-rows expert kernel reads the rows' choices directly; the dispatch tables are built only
-  // when the caller asked for one of them.
+  // The resident few-rows expert kernel and the tensor-memory kernels work from the rows' choices; the dispatch tables
+  // are built only when the caller asked for one of them.
   const bool wants_tables = out != nullptr && (out->expert_count || out->expert_offset || out->perm || out->active ||
                                                out->n_active || out->n_rows_active);
   const bool resident = tc && ctx->stream_path && !team::experts_stream_gathers(ctx->cfg.max_rows);
+  const bool need_tables = wants_tables || !(resident || (tc && !ctx->stream_path));
   cudaError_t e = cudaSuccess;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (resident && !wants_tables && ctx->fused_ok && !ctx->no_fuse) {
@@ -433,9 +436,9 @@ int team_moe_forward(team_ctx* ctx, const void* x, const team_step_state* st, te
   if (e != cudaSuccess) return fail_cuda(ctx, e, "router logits");
   ++ctx->last_launches;
   e = team::launch_select(ctx->ws.logits, step_ptrs(st), ctx->ws, export_ptrs(out), d, policy_of(ctx->cfg, st),
-                          ctx->item_tile, wants_tables || !resident, s);
+                          ctx->item_tile, need_tables, s);
   if (e != cudaSuccess) return fail_cuda(ctx, e, "select");
-  ctx->last_launches += team::select_launches(d);
+  ctx->last_launches += team::select_launches(d, need_tables);
   if (ctx->timing) {
     if ((e = timing_events(ctx, &ev0, &ev1)) != cudaSuccess) return fail_cuda(ctx, e, "event create");
     cudaEventRecord(ev0, s);

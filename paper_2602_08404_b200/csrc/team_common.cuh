@@ -64,6 +64,12 @@ struct WorkItem {
   int32_t pad;
 };
 
+// Tensor-memory expert kernels: the experts with work, in ascending order, and where each CTA's share begins.
+struct TilePlan {
+  int4* work;           // [experts] expert, first gathered row, token-slots
+  int4* begin;          // [CTAs + 1] index into work, first unit of the gate/up pass, first unit of the down pass
+};
+
 struct Workspace {
   float* logits;        // [max_rows, E]
   RoutePtrs r;          // context-owned routing tables (probs is null here)
@@ -76,6 +82,7 @@ struct Workspace {
   __nv_bfloat16* tile_act;  // [padded slot rows][I] likewise
   int32_t* tile_row;        // [padded slot rows]
   float* tile_w;            // [padded slot rows]
+  TilePlan plan;
   unsigned long long* arrivals;   // fused step: CTA arrivals at the grid barrier, counted over all launches
 };
 
@@ -103,8 +110,8 @@ int router_smem_bytes(int hidden);   // dynamic shared memory the logits kernels
 cudaError_t configure_select(Dims max_dims);
 bool experts_tile_supported(int hidden, int inter);
 int experts_tile_chunk();
-size_t experts_tile_rows(size_t slots, size_t max_items);
-cudaError_t configure_experts_tile();
+size_t experts_tile_rows(size_t slots, size_t n_experts);
+cudaError_t configure_experts_tile(Dims max_dims);
 cudaError_t launch_experts_tile(const void* x, const void* gu_tiles, const void* d_tiles, Workspace ws, float* y, Dims d,
                                 int grid, cudaStream_t s);
 cudaError_t launch_pack_w_tiles(const void* w_gate, const void* w_up, const void* w_down, void* gu, void* dt, int n_exp,
@@ -125,7 +132,7 @@ cudaError_t launch_router_topk(const float* logits, const uint8_t* tok_state, Ro
                                cudaStream_t s);
 cudaError_t launch_select(const float* logits, StepPtrs st, Workspace ws, RoutePtrs ex, Dims d, Policy p,
                           int item_tile, bool need_tables, cudaStream_t s);
-int select_launches(Dims d);   // kernels launch_select issues for these sizes
+int select_launches(Dims d, bool need_tables);   // kernels launch_select issues for these sizes
 size_t select_smem_bytes(Dims d);
 cudaError_t launch_experts_simt(const void* x, int dtype, const void* w_gate, const void* w_up, const void* w_down,
                                 Workspace ws, float* y, Dims d, cudaStream_t s);

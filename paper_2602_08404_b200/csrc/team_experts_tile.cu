@@ -10,44 +10,52 @@
 //   kernel B   D[128, N] = Wd_tile[128 hidden rows, I] * A[N, I]^T, scaled by the slot's routing weight and
 //              added into y[row, :] with fp32 reductions (a row's k experts meet there).
 //
-// Both are the same pipeline with a different epilogue.  A unit of work is (chunk, tile): a chunk is a run of
-// up to 128 token-slots of one activated expert (a work item of the selection kernel), a tile is 64
-// intermediate columns (A) or 128 hidden rows (B).  The global list of units is cut into one contiguous range
-// per CTA (grid = number of SMs): every unit of a kernel moves the same weight bytes, no CTA ever waits for
-// another one, nothing is exchanged between CTAs inside a kernel.
+// Both are the same pipeline with a different epilogue.  A unit of work is (tile, chunk): a tile is 64 intermediate
+// columns (A) or 128 hidden rows (B) of an activated expert, a chunk up to 128 of its token-slots.  The list of units
+// is cut into one contiguous range per CTA (grid = number of SMs) of equal cost, no CTA ever waits for another one,
+// nothing is exchanged between CTAs inside a kernel.
 //
 // Operands.  Weights are read from a tile-major copy made once per layer (team_pack_w_tiles): every
 // [128 rows x 64 k] bf16 tile is 16 KB contiguous and already in the 128-byte-swizzled K-major layout the
-// tensor core reads, so a pipeline stage is two one-dimensional bulk copies (weight tile from HBM with an
-// evict-first hint, token tile from L2) that complete on the stage's mbarrier.  The token tiles of kernel A
-// are gathered per chunk by a small kernel (k_gather_tiles) into the same layout; those of kernel B are what
-// kernel A wrote.
+// tensor core reads, so a pipeline stage is three one-dimensional bulk copies (weight tiles from HBM with an
+// evict-first hint, token tiles from L2) that complete on the stage's mbarrier.  The token tiles of kernel A
+// are gathered per chunk by k_dispatch_gather into the same layout; those of kernel B are what kernel A wrote.
 //
-// Warp roles (192 threads): warp 0 = producer (one lane issues the bulk copies), warp 1 = MMA issuer and
-// owner of the tensor memory (converged warp, one elected lane issues), warps 2-5 = epilogue (one lane
-// quarter of the accumulator each).  Two accumulators of 128 columns: the tensor core works on the next unit
-// while the epilogue drains the previous one.  Every wait is bounded; on expiry the kernel records
+// Warp roles (320 threads): warp 0 = producer (one lane issues the bulk copies), warp 1 = MMA issuer and
+// owner of the tensor memory (converged warp, one elected lane issues), warps 2-9 = epilogue (one lane
+// quarter of one accumulator each).  Two buffers of two accumulators of 128 columns: the tensor core works on the next
+// step while the epilogue drains the previous one.  Every wait is bounded; on expiry the kernel records
 // TEAM_ERR_TIMEOUT, leaves its loops, lets its copies land, frees its tensor memory and returns.
+#include <mutex>
+
 #include "team_common.cuh"
 #include "team_tc_ptx.cuh"
 
 namespace team {
 
-constexpr int kTileThreads = 192;
+constexpr int kTileThreads = 320;
 constexpr int kTileBytes = 128 * 128;          // one [128 rows x 64 bf16] tile
 constexpr int kTileElems = kTileBytes / 2;
-constexpr int kTileStages = 6;                 // pipeline stages: weight tile + token tile each
-constexpr int kStageBytes = 2 * kTileBytes;
+constexpr int kTileStages = 4;                 // pipeline stages: three operand tiles each
+constexpr int kStageBytes = 3 * kTileBytes;
 constexpr int kTileChunk = 128;                // token-slots per chunk at most (N of the MMA)
-constexpr int kTmemCols = 256;                 // two accumulators of 128 columns
-constexpr int kTileSmemBytes = 1024 + kTileStages * kStageBytes + 4 * kTileChunk * 8 + 256;
+constexpr int kTmemCols = 512;                 // two buffers of two accumulators of 128 columns
+constexpr int kEpiWarps = 8;                   // two warpgroups, one per accumulator of a step
+constexpr int kTileSmemBytes = 1024 + kTileStages * kStageBytes + kEpiWarps * kTileChunk * 8 + 256;
 
 enum { kEpiSwiglu = 0, kEpiCombine = 1 };
 
 __host__ __device__ inline int pad16(int n) { return (n + 15) & ~15; }
-// First padded row of chunk c in the gathered tables: chunks follow each other in dispatch order, each padded
-// to a multiple of 16 rows (at most 15 rows of padding, so 16 rows of slack per chunk keep them apart).
-__host__ __device__ inline int chunk_row0(const WorkItem& it, int c) { return it.begin + 16 * c; }
+// Rows of an expert with n token-slots in the gathered tables: all its chunks but the last are full.
+__host__ __device__ inline int padded_rows(int n) { return n / kTileChunk * kTileChunk + pad16(n % kTileChunk); }
+
+// What an expert with n token-slots costs per weight tile: the bytes a k-block brings into shared memory, in 128-byte
+// rows.  One chunk: a weight tile and half a token tile (two weight tiles share it); more: half a weight tile per
+// chunk (two chunks share it) and all token tiles.
+__device__ __forceinline__ int tile_cost(int n) {
+  const int chunks = (n + kTileChunk - 1) / kTileChunk;
+  return chunks <= 1 ? chunks * 128 + padded_rows(n) / 2 : (chunks + 1) / 2 * 128 + padded_rows(n);
+}
 
 // ---------------------------------------------------------------------------------------------------------
 // Weight layout: row-major -> tile-major, pre-swizzled (once per layer)
@@ -92,46 +100,189 @@ cudaError_t launch_pack_w_tiles(const void* w_gate, const void* w_up, const void
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Token rows of every chunk, gathered into B tiles: [chunk rows padded to 16][H] as [kb][np rows][64 k] swizzled,
-// and the chunk's (output row, routing weight) table.  One warp per padded row.
+// Dispatch: who chose which expert, the experts' places in the gathered tables, the GEMM CTAs' shares of the work, and
+// the token rows themselves as B tiles: [chunk rows padded to 16][H] as [kb][np rows][64 k] swizzled.
+//
+// One CTA doing this alone (a counting sort of T * k slots) is a serial 22 us at 1024 rows and 28 us at 2048, followed
+// by a gather that has to wait for it (13 / 37 us).  Here every CTA forms the tables for itself from the rows' choices,
+// as a bit matrix [expert][row] in shared memory: the rank of row t inside expert e is a population count (slots
+// ascend inside an expert as rows do), so nothing is sorted and no CTA waits for another one, and then copies its own
+// rows to the places their slots have.  Measured, end of the routing rounds to end of the gather: 35 -> 19 us at 1024 rows, 65 -> 36 us at 2048.
+// Padding rows stay what they are: they only reach accumulator columns that nobody reads.
 // ---------------------------------------------------------------------------------------------------------
-struct GatherArgs {
+constexpr int kDispThreads = 512;
+
+struct DispatchArgs {
   const __nv_bfloat16* x;       // [T, H]
-  const int32_t* perm;
+  const int32_t* topk_idx;      // [T, k] (-1: row skipped)
   const float* topk_w;
-  const WorkItem* items;
-  const int32_t* n_items;
+  const uint8_t* tok_class;     // [T]
   __nv_bfloat16* xg;            // gathered tiles
-  int32_t* row_of;              // [padded rows] output row of the slot (-1: padding)
+  int32_t* row_of;              // [padded rows] output row of the slot
   float* w_of;                  // [padded rows] its routing weight
+  TilePlan plan;
+  int gemm_ctas;
   Dims d;
 };
 
-__global__ void __launch_bounds__(256) k_gather_tiles(GatherArgs a) {
+// shared memory: bits[EN][W1] | pre[EN][W1] (u16) | n[EN] | row0[EN] | cost[EN + 1] | work index of the expert [EN]
+__host__ __device__ inline int disp_words(int T) { return ((T + 31) >> 5) | 1; }      // odd: no bank conflicts over experts
+static size_t disp_smem_bytes(const Dims& d) {
+  const size_t EN = d.E + d.ns, W1 = disp_words(d.T);
+  return EN * W1 * 4 + ((EN * W1 * 2 + 15) & ~size_t(15)) + (4 * EN + 4) * 4;
+}
+
+__global__ void __launch_bounds__(kDispThreads) k_dispatch_gather(DispatchArgs a) {
+  extern __shared__ __align__(16) uint32_t disp_smem[];
+  const int T = a.d.T, k = a.d.k, E = a.d.E, EN = E + a.d.ns, H = a.d.H;
+  const int W = (T + 31) >> 5, W1 = disp_words(T);
+  uint32_t* bits = disp_smem;
+  uint16_t* pre = reinterpret_cast<uint16_t*>(bits + EN * W1);
+  int32_t* s_n = reinterpret_cast<int32_t*>(reinterpret_cast<unsigned char*>(pre) + ((EN * W1 * 2 + 15) & ~15));
+  int32_t* s_row0 = s_n + EN;
+  int32_t* s_cost = s_row0 + EN;          // [EN + 1] cost of the experts in front of this one
+  int32_t* s_widx = s_cost + EN + 1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");            // the selection kernel's tables are complete
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int H = a.d.H, n_items = *a.n_items;
-  const int pieces = H / 8;                                      // 16-byte pieces per row
-  // four CTAs share a chunk: CTA slice s takes the rows n with (n / 8) % 4 == s, its warp w those with n % 8 == w
-  const int slice = blockIdx.x & 3;
-  for (int c = blockIdx.x >> 2; c < n_items; c += gridDim.x >> 2) {
-    const WorkItem it = a.items[c];
-    const int np = pad16(it.n), r0 = chunk_row0(it, c);
-    __nv_bfloat16* base = a.xg + (size_t)r0 * H;
-    for (int n = slice * 8 + warp; n < np; n += 32) {
-      int row = -1;
-      float wt = 0.f;
-      if (n < it.n) slot_row_weight(a.perm[it.begin + n], a.d.T, a.d.k, a.topk_w, row, wt);
-      if (lane == 0) {
-        a.row_of[r0 + n] = row;
-        a.w_of[r0 + n] = wt;
+  asm volatile("griddepcontrol.wait;" ::: "memory");            // the rows' choices are complete
+  // 32 rows per warp: lane = row collects its choices as a bit string over the experts, then 32 x 32 bit transposes turn
+  // rows into experts (shared-memory atomics per slot took 10 us at 2048 rows)
+  for (int w = warp; w < W; w += kDispThreads / 32) {
+    const int t = w * 32 + lane;
+    uint32_t m[8] = {};
+    for (int j0 = 0; j0 < k; j0 += 4) {
+      int ee[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) ee[q] = t < T && j0 + q < k ? a.topk_idx[t * k + j0 + q] : -1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (ee[q] >= a.d.elo && ee[q] < a.d.ehi) {              // this rank's own experts
+#pragma unroll
+          for (int i = 0; i < 8; ++i) m[i] |= (ee[q] >> 5) == i ? 1u << (ee[q] & 31) : 0u;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (i * 32 >= E) break;
+      uint32_t v = m[i], keep = 0x0000ffffu;
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        const uint32_t x = __shfl_xor_sync(0xffffffffu, v, o);
+        v = (lane & o) ? (v & ~keep) | ((x & ~keep) >> o) : (v & keep) | ((x & keep) << o);
+        keep ^= keep << (o >> 1);
       }
-      const uint4* src = reinterpret_cast<const uint4*>(a.x + (size_t)max(row, 0) * H);
-      for (int p = lane; p < pieces; p += 32) {
-        const uint4 v = row >= 0 ? __ldg(src + p) : make_uint4(0u, 0u, 0u, 0u);
-        const int kb = p >> 3, pc = (p & 7) ^ (n & 7);
-        *reinterpret_cast<uint4*>(base + (size_t)kb * np * 64 + n * 64 + pc * 8) = v;
+      if (i * 32 + lane < E) bits[(i * 32 + lane) * W1 + w] = v;
+    }
+  }
+  if (a.d.ns > 0) {                                             // shared experts take every computed row
+    for (int w = warp; w < W; w += kDispThreads / 32) {
+      const int t = w * 32 + lane;
+      const uint32_t m = __ballot_sync(0xffffffffu, t < T && a.tok_class[t] != TEAM_CLS_SKIP);
+      if (lane < a.d.ns) bits[(E + lane) * W1 + w] = m;
+    }
+  }
+  __syncthreads();
+  for (int e = warp; e < EN; e += kDispThreads / 32) {          // slots of the expert in front of each word (W <= 64)
+    int run = 0;
+    for (int w0 = 0; w0 < W; w0 += 32) {
+      const int w = w0 + lane, c = w < W ? __popc(bits[e * W1 + w]) : 0;
+      int incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+      }
+      if (w < W) pre[e * W1 + w] = (uint16_t)(run + incl - c);
+      run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) s_n[e] = run;
+  }
+  __syncthreads();
+  if (warp == 0) {                                              // places of the experts, costs in front of them
+    int rows = 0, cost = 0, used = 0;
+    for (int e0 = 0; e0 < EN; e0 += 32) {
+      const int e = e0 + lane, n = e < EN ? s_n[e] : 0;
+      const int pr = padded_rows(n), cs = tile_cost(n);
+      int ir = pr, ic = cs;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int r1 = __shfl_up_sync(0xffffffffu, ir, o), c1 = __shfl_up_sync(0xffffffffu, ic, o);
+        if (lane >= o) { ir += r1; ic += c1; }
+      }
+      const uint32_t act = __ballot_sync(0xffffffffu, n > 0);
+      if (e < EN) {
+        s_row0[e] = rows + ir - pr;
+        s_cost[e] = cost + ic - cs;
+        s_widx[e] = used + __popc(act & ((1u << lane) - 1u));
+      }
+      rows += __shfl_sync(0xffffffffu, ir, 31);
+      cost += __shfl_sync(0xffffffffu, ic, 31);
+      used += __popc(act);
+    }
+    if (lane == 0) s_cost[EN] = cost;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (int e = tid; e < EN; e += kDispThreads)
+      if (s_n[e] > 0) a.plan.work[s_widx[e]] = make_int4(e, s_row0[e], s_n[e], 0);
+    // where CTA b of the GEMMs begins: the expert that holds cost total * b / gemm_ctas, and the unit inside it
+    const long long total = s_cost[EN];
+    for (int b = tid; b <= a.gemm_ctas; b += kDispThreads) {
+      const int at = (int)(total * b / a.gemm_ctas);
+      int lo = 0, hi = EN;                                      // the last expert with s_cost[e] <= at (empty ones: cost 0)
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (s_cost[mid] <= at) lo = mid; else hi = mid;
+      }
+      int units_a = 0, units_b = 0;
+      const int cost = s_cost[lo + 1] - s_cost[lo], chunks = (s_n[lo] + kTileChunk - 1) / kTileChunk;
+      if (cost > 0) {                                           // 0: behind the last expert
+        units_a = (int)((long long)(at - s_cost[lo]) * (a.d.I / 64) * chunks / cost);
+        units_b = (int)((long long)(at - s_cost[lo]) * (a.d.H / 128) * chunks / cost);
+      }
+      a.plan.begin[b] = make_int4(s_widx[lo], units_a, units_b, 0);
+    }
+  }
+  // the CTA's rows: a row's pieces are read once and written to all places of the row; with fewer rows than warps several
+  // warps share a row
+  const int rows_per = (T + gridDim.x - 1) / gridDim.x, t0 = blockIdx.x * rows_per, t1 = min(T, t0 + rows_per);
+  const int per_row = k + a.d.ns, pieces = H / 8;               // 16-byte pieces per row
+  const int share = max(1, (kDispThreads / 32) / rows_per), sub = warp % share;
+  if (warp / share * share + share > kDispThreads / 32) return; // warps left over when share does not divide their number
+  for (int t = t0 + warp / share; t < t1; t += (kDispThreads / 32) / share) {
+    // lane j: place of the row's j-th slot (per_row <= 20)
+    int at = 0, base_row = -1, np = 0;
+    const int e = lane < k ? a.topk_idx[t * k + lane] : (lane < per_row ? E + lane - k : -1);
+    if (e >= 0) {
+      const uint32_t word = bits[e * W1 + (t >> 5)];
+      if ((word >> (t & 31)) & 1u) {
+        const int rank = pre[e * W1 + (t >> 5)] + __popc(word & ((1u << (t & 31)) - 1u));
+        at = rank % kTileChunk;
+        base_row = s_row0[e] + rank - at;
+        np = pad16(min(kTileChunk, s_n[e] - (rank - at)));
+        if (sub == 0) {
+          a.row_of[base_row + at] = t;
+          a.w_of[base_row + at] = lane < k ? a.topk_w[t * k + lane] : 1.f;
+        }
+      }
+    }
+    const uint4* src = reinterpret_cast<const uint4*>(a.x + (size_t)t * H);
+    for (int p0 = sub * 32; p0 < pieces; p0 += share * 128) {
+      uint4 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int p = p0 + q * share * 32 + lane;
+        v[q] = p < pieces ? __ldg(src + p) : make_uint4(0u, 0u, 0u, 0u);
+      }
+      for (int j = 0; j < per_row; ++j) {
+        const int br = __shfl_sync(0xffffffffu, base_row, j), n = __shfl_sync(0xffffffffu, at, j), pn = __shfl_sync(0xffffffffu, np, j);
+        if (br < 0) continue;
+        __nv_bfloat16* base = a.xg + (size_t)br * H + n * 64;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int p = p0 + q * share * 32 + lane;
+          if (p < pieces) *reinterpret_cast<uint4*>(base + (size_t)(p >> 3) * pn * 64 + (((p & 7) ^ (n & 7)) << 3)) = v[q];
+        }
       }
     }
   }
@@ -142,17 +293,74 @@ __global__ void __launch_bounds__(256) k_gather_tiles(GatherArgs a) {
 // ---------------------------------------------------------------------------------------------------------
 struct TileArgs {
   const __nv_bfloat16* w_tiles;   // [e][tile][kb][16 KB]
-  const __nv_bfloat16* b_tiles;   // per chunk: [kb][np rows][64 k], chunk c at row chunk_row0(c) * (n_k * 64) elements
-  const WorkItem* items;
-  const int32_t* n_items;
+  const __nv_bfloat16* b_tiles;   // per chunk: [kb][np rows][64 k], from the chunk's first row * (n_k * 64) elements
+  TilePlan plan;
   const int32_t* row_of;
   const float* w_of;
   __nv_bfloat16* act;             // kEpiSwiglu: output, per chunk [u][np rows][64 columns] swizzled
   float* y;                       // kEpiCombine: [T, H]
   int32_t* status;
   int n_k;                        // k-blocks of 64: H/64 (A) or I/64 (B)
-  int tiles_per_chunk;            // I/64 (A) or H/128 (B)
+  int tiles;                      // weight tiles per expert: I/64 (A) or H/128 (B)
   int H, I;
+};
+
+// The walk over a CTA's range of (tile, chunk) units, tile by tile and inside a tile chunk by chunk.  A step computes up
+// to two accumulators from three operand tiles: two neighbouring weight tiles for an expert of one chunk (the token
+// tile is fetched once for both), or one weight tile for two chunks of a larger expert (its weights cross HBM once up to
+// 256 token-slots; read again one chunk later they would come from HBM again, because the other CTAs stream more than L2
+// holds in between: gate/up pass of 2048 rows of the SDAR shape 255 us that way, 168 us this way).
+struct TileWalk {
+  const int4* work;
+  int x, u, x_end, u_end, tiles;
+  int e, row0, n, chunks, limit;
+  int j, nt, nc, first;           // current step: tiles j .. j + nt - 1, chunks of rows first, first + 128 (nc of them)
+  int slots[2];                   // token-slots of the two chunks
+  __device__ __forceinline__ void load() {
+    const int4 w = work[x];
+    e = w.x;
+    row0 = w.y;
+    n = w.z;
+    chunks = (n + kTileChunk - 1) / kTileChunk;
+    limit = x == x_end ? u_end : chunks * tiles;
+  }
+  __device__ __forceinline__ TileWalk(const TilePlan& p, int t, bool phase_b) : work(p.work), tiles(t) {
+    const int4 lo = p.begin[blockIdx.x], hi = p.begin[blockIdx.x + 1];
+    x = lo.x;
+    x_end = hi.x;
+    u = phase_b ? lo.z : lo.y;
+    u_end = phase_b ? hi.z : hi.y;
+    if (x < x_end || u < u_end) load();
+  }
+  __device__ __forceinline__ bool next() {
+    if (x == x_end && u >= u_end) return false;
+    if (u >= limit) {
+      ++x;
+      u = 0;
+      if (x == x_end && u >= u_end) return false;
+      load();
+    }
+    int c = 0;
+    nt = nc = 1;
+    if (chunks == 1) {
+      j = u;
+      if ((u & 1) == 0 && u + 1 < limit) nt = 2;
+    } else {
+      j = u / chunks;
+      c = u - j * chunks;
+      if ((c & 1) == 0 && c + 1 < chunks && u + 1 < limit) nc = 2;
+    }
+    u += nt * nc;
+    first = row0 + c * kTileChunk;
+    slots[0] = min(kTileChunk, n - c * kTileChunk);
+    slots[1] = min(kTileChunk, n - (c + 1) * kTileChunk);
+    return true;
+  }
+  __device__ __forceinline__ int accs() const { return nt * nc; }
+  // of accumulator i: its tile, its chunk's first gathered row and token-slots
+  __device__ __forceinline__ int tile(int i) const { return nt == 2 ? j + i : j; }
+  __device__ __forceinline__ int row(int i) const { return nc == 2 ? first + i * kTileChunk : first; }
+  __device__ __forceinline__ int n_of(int i) const { return nc == 2 && i ? slots[1] : slots[0]; }
 };
 
 template <int EPI>
@@ -161,13 +369,13 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
   // 1024-byte alignment for the swizzled tiles
   unsigned char* smem = tile_smem_raw + ((1024u - (smem_u32(tile_smem_raw) & 1023u)) & 1023u);
   unsigned char* stages = smem;
-  int32_t* tab_row = reinterpret_cast<int32_t*>(smem + kTileStages * kStageBytes);      // [4 epilogue warps][128]
-  float* tab_w = reinterpret_cast<float*>(tab_row + 4 * kTileChunk);                    // [4][128]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tab_w + 4 * kTileChunk);
+  int32_t* tab_row = reinterpret_cast<int32_t*>(smem + kTileStages * kStageBytes);      // [8 epilogue warps][128]
+  float* tab_w = reinterpret_cast<float*>(tab_row + kEpiWarps * kTileChunk);            // [8][128]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tab_w + kEpiWarps * kTileChunk);
   uint64_t* bar_full = bars;                       // [stages] bytes of the stage have landed
   uint64_t* bar_empty = bars + kTileStages;        // [stages] the MMAs reading the stage are done
-  uint64_t* bar_dfull = bars + 2 * kTileStages;    // [2] accumulator complete
-  uint64_t* bar_dempty = bar_dfull + 2;            // [2] accumulator drained by the epilogue
+  uint64_t* bar_dfull = bars + 2 * kTileStages;    // [2] accumulators complete
+  uint64_t* bar_dempty = bar_dfull + 2;            // [2] accumulators drained by the epilogue
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_dempty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -179,7 +387,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(bar_dfull + i), 1);
-      mbar_init(smem_u32(bar_dempty + i), 4);
+      mbar_init(smem_u32(bar_dempty + i), kEpiWarps);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -195,32 +403,32 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // Everything above overlaps the preceding kernel; its outputs (work items, token tiles) are complete from here.
+  // Everything above overlaps the preceding kernel; its outputs (plan, token tiles) are complete from here.
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  const int TPC = a.tiles_per_chunk, NK = a.n_k;
-  const long long n_units = (long long)(*a.n_items) * TPC;
-  const int u_lo = (int)(n_units * blockIdx.x / gridDim.x), u_hi = (int)(n_units * (blockIdx.x + 1) / gridDim.x);
+  const int NK = a.n_k;
+  TileWalk wk(a.plan, a.tiles, EPI == kEpiCombine);
 
   if (warp == 0) {
     // ------------------------------ producer ------------------------------
     const uint64_t pol = stream_policy();
     uint32_t it = 0;
     bool ok = true;
-    for (int unit = u_lo; unit < u_hi && ok; ++unit) {
-      const int c = unit / TPC, j = unit - c * TPC;
-      const WorkItem item = a.items[c];
-      const int np = pad16(item.n);
-      const __nv_bfloat16* wsrc = a.w_tiles + ((size_t)item.e * TPC + j) * NK * kTileElems;
-      const __nv_bfloat16* bsrc = a.b_tiles + (size_t)chunk_row0(item, c) * NK * 64;
+    while (ok && wk.next()) {
+      const __nv_bfloat16* wsrc = a.w_tiles + ((size_t)wk.e * a.tiles + wk.j) * NK * kTileElems;
+      const __nv_bfloat16* bsrc = a.b_tiles + (size_t)wk.first * NK * 64;
+      const int np0 = pad16(wk.slots[0]), np1 = wk.nc == 2 ? pad16(wk.slots[1]) : 0;
       for (int kb = 0; kb < NK; ++kb, ++it) {
         const uint32_t s = it % kTileStages;
         if (!(ok = mbar_wait_warp<32>(smem_u32(bar_empty + s), ((it / kTileStages) & 1) ^ 1, abort_flag, a.status, 31))) break;
         if (lane == 0) {
+          // stage: weight tile | second weight tile or second token tile | token tile
           const uint32_t full = smem_u32(bar_full + s), dst = smem_u32(stages + (size_t)s * kStageBytes);
-          mbar_expect_tx(full, (uint32_t)(kTileBytes + np * 128));
+          mbar_expect_tx(full, (uint32_t)(wk.nt * kTileBytes + (np0 + np1) * 128));
           bulk_g2s_stream(dst, wsrc + (size_t)kb * kTileElems, kTileBytes, full, pol);
-          bulk_g2s(dst + kTileBytes, bsrc + (size_t)kb * np * 64, (uint32_t)(np * 128), full);
+          if (wk.nt == 2) bulk_g2s_stream(dst + kTileBytes, wsrc + (size_t)(NK + kb) * kTileElems, kTileBytes, full, pol);
+          bulk_g2s(dst + 2 * kTileBytes, bsrc + (size_t)kb * np0 * 64, (uint32_t)np0 * 128, full);
+          if (np1 > 0) bulk_g2s(dst + kTileBytes, bsrc + (size_t)NK * (kTileChunk * 64) + (size_t)kb * np1 * 64, (uint32_t)np1 * 128, full);
         }
         __syncwarp();
       }
@@ -233,84 +441,87 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
     // ------------------------------ MMA issuer ------------------------------
     uint32_t it = 0, un = 0;
     bool ok = true;
-    for (int unit = u_lo; unit < u_hi && ok; ++unit, ++un) {
-      const int c = unit / TPC;
-      const uint32_t idesc = make_idesc_bf16(pad16(a.items[c].n));
+    for (; ok && wk.next(); ++un) {
+      const uint32_t idesc0 = make_idesc_bf16(pad16(wk.n_of(0))), idesc1 = make_idesc_bf16(pad16(wk.n_of(1)));
+      const int accs = wk.accs();
       const uint32_t buf = un & 1;
       if (!(ok = mbar_wait_warp(smem_u32(bar_dempty + buf), ((un >> 1) & 1) ^ 1, abort_flag, a.status, 32))) break;
       tc_fence_after();
-      const uint32_t acc = tmem_base + buf * kTileChunk;
+      const uint32_t acc = tmem_base + buf * 2 * kTileChunk;
       for (int kb = 0; kb < NK; ++kb, ++it) {
         const uint32_t s = it % kTileStages;
         if (!(ok = mbar_wait_warp(smem_u32(bar_full + s), (it / kTileStages) & 1, abort_flag, a.status, 33))) break;
         tc_fence_after();
         const uint32_t base = smem_u32(stages + (size_t)s * kStageBytes);
-        const uint64_t da = make_kmajor_sw128_desc(base), db = make_kmajor_sw128_desc(base + kTileBytes);
+        const uint64_t d0 = make_kmajor_sw128_desc(base), d1 = make_kmajor_sw128_desc(base + kTileBytes),
+                       d2 = make_kmajor_sw128_desc(base + 2 * kTileBytes);
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) tc_mma(acc, da + 2 * k4, db + 2 * k4, idesc, (kb | k4) != 0);
+        for (int k4 = 0; k4 < 4; ++k4) tc_mma(acc, d0 + 2 * k4, d2 + 2 * k4, idesc0, (kb | k4) != 0);
+        if (accs == 2) {
+          const uint64_t da = wk.nt == 2 ? d1 : d0, db = wk.nt == 2 ? d2 : d1;
+#pragma unroll
+          for (int k4 = 0; k4 < 4; ++k4) tc_mma(acc + kTileChunk, da + 2 * k4, db + 2 * k4, idesc1, (kb | k4) != 0);
+        }
         tc_commit(smem_u32(bar_empty + s));
       }
       if (ok) tc_commit(smem_u32(bar_dfull + buf));
     }
   } else {
-    // ------------------------------ epilogue ------------------------------
-    const int q = warp & 3;                          // this warp's lane quarter of the accumulator
+    // ------------------------------ epilogue: warps 2-5 accumulator 0 of a step, warps 6-9 accumulator 1 ------------------------------
+    const int ew = warp - 2, half = ew >> 2;
+    const int q = warp & 3;                          // this warp's lane quarter of the accumulators
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     uint32_t un = 0;
-    int tab_chunk = -1;
+    int tab_first = -1;
     bool ok = true;
-    for (int unit = u_lo; unit < u_hi && ok; ++unit, ++un) {
-      const int c = unit / TPC, j = unit - c * TPC;
-      const WorkItem item = a.items[c];
-      const int np = pad16(item.n), r0 = chunk_row0(item, c);
+    for (; ok && wk.next(); ++un) {
       const uint32_t buf = un & 1;
-      if (EPI == kEpiCombine && c != tab_chunk) {
+      const bool mine = half < wk.accs();
+      const int j = wk.tile(half), first = wk.row(half), n_c = wk.n_of(half), np = pad16(n_c);
+      if (EPI == kEpiCombine && mine && first != tab_first) {
         // (output row, weight) of the chunk's slots: every epilogue warp keeps a copy of its own, refilled at its own pace
         __syncwarp();
-        for (int n = lane; n < np; n += 32) {
-          tab_row[q * kTileChunk + n] = a.row_of[r0 + n];
-          tab_w[q * kTileChunk + n] = a.w_of[r0 + n];
+        for (int n = lane; n < n_c; n += 32) {
+          tab_row[ew * kTileChunk + n] = a.row_of[first + n];
+          tab_w[ew * kTileChunk + n] = a.w_of[first + n];
         }
-        tab_chunk = c;
+        tab_first = first;
         __syncwarp();
       }
       if (!(ok = mbar_wait_warp<32>(smem_u32(bar_dfull + buf), (un >> 1) & 1, abort_flag, a.status, 34))) break;
       tc_fence_after();
-      const uint32_t acc = tmem_base + buf * kTileChunk + lane_off;
-      if (EPI == kEpiSwiglu) {
-        // rows of this warp: [16 gate | 16 up] of intermediate columns j*64 + q*16 + (lane & 15)
-        const bool is_gate = lane < 16;
-        const int i = q * 16 + (lane & 15);                                   // column inside the tile
-        __nv_bfloat16* dst = a.act + (size_t)r0 * a.I + (size_t)j * np * 64;   // this unit's [np][64] tile
-        for (int c0 = 0; c0 < np; c0 += 8) {
-          float v[8];
-          tmem_ld8(acc + c0, v);
+      const uint32_t acc = tmem_base + buf * 2 * kTileChunk + half * kTileChunk + lane_off;
+      if (mine) {
+        if (EPI == kEpiSwiglu) {
+          // lanes 0-15 hold gate rows, lanes 16-31 the up rows of the same intermediate columns j*64 + q*16 + (lane & 15):
+          // the lower half finishes slots c0 .. c0+3, the upper half c0+4 .. c0+7
+          const bool is_gate = lane < 16;
+          const int i = q * 16 + (lane & 15), tb = is_gate ? 0 : 4;
+          __nv_bfloat16* dst = a.act + (size_t)first * a.I + (size_t)j * np * 64;   // this unit's [np][64] tile
+          for (int c0 = 0; c0 < np; c0 += 8) {
+            float v[8];
+            tmem_ld8(acc + c0, v);
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const float o = __shfl_xor_sync(0xffffffffu, v[t], 16);
-            const float g = is_gate ? v[t] : o;
-            const float u = is_gate ? o : v[t];
-            v[t] = g / (1.f + expf(-g)) * u;
+            for (int t = 0; t < 4; ++t) {
+              const float o = __shfl_xor_sync(0xffffffffu, is_gate ? v[t + 4] : v[t], 16);
+              const float g = is_gate ? v[t] : o;
+              const float u = is_gate ? o : v[t + 4];
+              const int n = c0 + tb + t;
+              dst[(size_t)n * 64 + (((i >> 3) ^ (n & 7)) << 3) + (i & 7)] = __float2bfloat16_rn(g / (1.f + expf(-g)) * u);
+            }
           }
-          // lanes 0-15 store slots c0 .. c0+3, lanes 16-31 store c0+4 .. c0+7 (padding slots are zero rows: silu(0) * 0 = 0)
-          const int tb = is_gate ? 0 : 4;
+        } else {
+          const int32_t* rows = tab_row + ew * kTileChunk;
+          const float* wts = tab_w + ew * kTileChunk;
+          float* ycol = a.y + (size_t)j * 128 + q * 32 + lane;
+          for (int c0 = 0; c0 < n_c; c0 += 8) {
+            float v[8];
+            tmem_ld8(acc + c0, v);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int n = c0 + tb + t;
-            dst[(size_t)n * 64 + (((i >> 3) ^ (n & 7)) << 3) + (i & 7)] = __float2bfloat16_rn(v[tb + t]);
-          }
-        }
-      } else {
-        const int32_t* rows = tab_row + q * kTileChunk;
-        const float* wts = tab_w + q * kTileChunk;
-        float* ycol = a.y + (size_t)j * 128 + q * 32 + lane;
-        for (int c0 = 0; c0 < item.n; c0 += 8) {
-          float v[8];
-          tmem_ld8(acc + c0, v);
-#pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const int n = c0 + t;
-            if (n < item.n) atomicAdd(ycol + (size_t)rows[n] * a.H, wts[n] * v[t]);
+            for (int t = 0; t < 8; ++t) {
+              const int n = c0 + t;
+              if (n < n_c) atomicAdd(ycol + (size_t)rows[n] * a.H, wts[n] * v[t]);
+            }
           }
         }
       }
@@ -334,23 +545,26 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
 // ---------------------------------------------------------------------------------------------------------
 bool experts_tile_supported(int hidden, int inter) { return hidden % 128 == 0 && inter % 64 == 0; }
 int experts_tile_chunk() { return kTileChunk; }
-// Rows of the gathered tables: every slot, plus 16 rows of padding slack per chunk.
-size_t experts_tile_rows(size_t slots, size_t max_items) { return slots + 16 * max_items + 16; }
+// Rows of the gathered tables: every slot, plus the padding of each expert's last chunk.
+size_t experts_tile_rows(size_t slots, size_t n_experts) { return slots + 16 * n_experts; }
 
-cudaError_t configure_experts_tile() {
-  static bool done[64] = {};
+// The opt-in is per device and shared by all contexts: the dispatch kernel's is only ever raised.
+cudaError_t configure_experts_tile(Dims max_dims) {
+  static std::mutex mu;
+  static int prepared[64] = {};      // dispatch kernel's shared memory opted in so far
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_grouped_gemm<kEpiSwiglu>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_grouped_gemm<kEpiCombine>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_grouped_gemm<kEpiSwiglu>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_grouped_gemm<kEpiCombine>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+  const int disp = (int)disp_smem_bytes(max_dims);
+  std::lock_guard<std::mutex> lock(mu);
+  if (dev >= 0 && dev < 64 && prepared[dev] >= disp) return cudaSuccess;
+  for (const void* fn : {reinterpret_cast<const void*>(&k_dispatch_gather), reinterpret_cast<const void*>(&k_grouped_gemm<kEpiSwiglu>),
+                         reinterpret_cast<const void*>(&k_grouped_gemm<kEpiCombine>)}) {
+    const int smem = fn == reinterpret_cast<const void*>(&k_dispatch_gather) ? disp : kTileSmemBytes;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  }
+  if (e == cudaSuccess && dev >= 0 && dev < 64) prepared[dev] = disp;
   return e;
 }
 
@@ -369,24 +583,25 @@ static cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem
   return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
-// gather, gate/up + SwiGLU, down + combine: three launches chained with programmatic dependent launch
+// dispatch + gather, gate/up + SwiGLU, down + combine: three launches chained with programmatic dependent launch
 cudaError_t launch_experts_tile(const void* x, const void* gu_tiles, const void* d_tiles, Workspace ws, float* y, Dims d,
                                 int grid, cudaStream_t s) {
-  GatherArgs g;
+  DispatchArgs g;
   g.x = static_cast<const __nv_bfloat16*>(x);
-  g.perm = ws.r.perm;
+  g.topk_idx = ws.r.topk_idx;
   g.topk_w = ws.r.topk_w;
-  g.items = ws.items;
-  g.n_items = ws.n_items;
+  g.tok_class = ws.r.tok_class;
   g.xg = ws.tile_x;
   g.row_of = ws.tile_row;
   g.w_of = ws.tile_w;
+  g.plan = ws.plan;
+  g.gemm_ctas = grid;
   g.d = d;
-  cudaError_t e = launch_pdl(reinterpret_cast<const void*>(&k_gather_tiles), dim3(4 * grid), dim3(256), 0, s, &g);
+  cudaError_t e = launch_pdl(reinterpret_cast<const void*>(&k_dispatch_gather), dim3(d.T < grid ? d.T : grid), dim3(kDispThreads),
+                             disp_smem_bytes(d), s, &g);
   if (e != cudaSuccess) return e;
   TileArgs a = {};
-  a.items = ws.items;
-  a.n_items = ws.n_items;
+  a.plan = ws.plan;
   a.row_of = ws.tile_row;
   a.w_of = ws.tile_w;
   a.act = ws.tile_act;
@@ -397,13 +612,13 @@ cudaError_t launch_experts_tile(const void* x, const void* gu_tiles, const void*
   a.w_tiles = static_cast<const __nv_bfloat16*>(gu_tiles);
   a.b_tiles = ws.tile_x;
   a.n_k = d.H / 64;
-  a.tiles_per_chunk = d.I / 64;
+  a.tiles = d.I / 64;
   e = launch_pdl(reinterpret_cast<const void*>(&k_grouped_gemm<kEpiSwiglu>), dim3(grid), dim3(kTileThreads), kTileSmemBytes, s, &a);
   if (e != cudaSuccess) return e;
   a.w_tiles = static_cast<const __nv_bfloat16*>(d_tiles);
   a.b_tiles = ws.tile_act;
   a.n_k = d.I / 64;
-  a.tiles_per_chunk = d.H / 128;
+  a.tiles = d.H / 128;
   return launch_pdl(reinterpret_cast<const void*>(&k_grouped_gemm<kEpiCombine>), dim3(grid), dim3(kTileThreads), kTileSmemBytes, s, &a);
 }
 

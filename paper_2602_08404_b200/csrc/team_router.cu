@@ -130,8 +130,10 @@ k_router_logits_mma(const __nv_bfloat16* __restrict__ x, const float* __restrict
   constexpr int R = MT * 16, N = NT * 8;
   constexpr int U = MT * NT == 1 ? 4 : (MT * NT == 2 ? 2 : 1);      // blocks of 32 in flight beside the current ones
   extern __shared__ __align__(16) float s_part[];                   // [warps][R][N]
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // in this order: the selection kernel stages the step state ahead of its own wait, and that state may come from the
+  // kernel in front of this one
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
   const int H = d.H, T = d.T, E = d.E, nb = H >> 5;
   const int t0 = blockIdx.x * R, e0 = blockIdx.y * N;

@@ -566,22 +566,22 @@ cudaError_t launch_select(const float* logits, StepPtrs st, Workspace ws, RouteP
     attrs[1].val.clusterDim.z = 1;
     cfg.attrs = attrs;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_select, logits, st, ws, ex, d, p, item_tile, 1, (int)kSelCluster, 0);
+    return cudaLaunchKernelEx(&cfg, k_select, logits, st, ws, ex, d, p, item_tile, 1, (int)kSelCluster, need_tables ? 0 : 1);
   }
   if (d.G > 1 && d.T > kSelWarps) {
     cfg.gridDim = dim3(group_ctas);
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_select, logits, st, ws, ex, d, p, item_tile, 1, (int)kSelRounds, 0);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !need_tables) return e;
     cfg.gridDim = dim3(1);
     return cudaLaunchKernelEx(&cfg, k_select, logits, st, ws, ex, d, p, item_tile, 1, (int)kSelDispatch, 0);
   }
   return cudaLaunchKernelEx(&cfg, k_select, logits, st, ws, ex, d, p, item_tile, 1, (int)kSelAll, need_tables ? 0 : 1);
 }
 
-int select_launches(Dims d) {
+int select_launches(Dims d, bool need_tables) {
   const int group_ctas = d.G < 128 ? d.G : 128;
   if (d.T > kSelWarps && (d.G == 1 || d.T / group_ctas > kSelWarps)) return 1;
-  return d.G > 1 && d.T > kSelWarps ? 2 : 1;
+  return d.G > 1 && d.T > kSelWarps && need_tables ? 2 : 1;
 }
 
 }  // namespace team
