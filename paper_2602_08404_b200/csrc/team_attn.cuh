@@ -1,4 +1,4 @@
-// Shared by the two attention kernels (Sec. 4.1, the attention half of delayed caching): argument block and
+// Shared by the attention kernel and the insertion (Sec. 4.1, the attention half of delayed caching): argument block and
 // the test for "this row is computed".
 #pragma once
 
@@ -6,7 +6,6 @@
 
 namespace team {
 
-constexpr int kAttnPairs = 128;        // (row, head) pairs per CTA
 constexpr int kAttnMaxSplits = 8;      // portable cluster size
 
 struct AttnArgs {
@@ -29,8 +28,7 @@ struct AttnArgs {
 
 __device__ __forceinline__ bool attn_computed(int state, int flags) { return !((flags & TEAM_F_DCD) && state == TEAM_TOK_CACHED); }
 
-// head size 128 on the tensor-memory path (team_attn_tc.cu): launch and one-time set-up
-cudaError_t configure_attention_tc();
-cudaError_t launch_attention_tc(const AttnArgs& a, int m_tiles, int n_splits, cudaStream_t s);
+// the attention itself (team_attn_tc.cu); one-time set-up on a device's first call
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s);
 
 }  // namespace team

@@ -1,22 +1,24 @@
-// The attention half of delayed caching (Sec. 4.1; block diffusion, Sec. 2) for head size 128 on the fifth-generation
-// tensor cores: S = Q K^T and O += P V are tcgen05.mma instructions with their accumulators in tensor memory.
+// The attention half of delayed caching (Sec. 4.1; block diffusion, Sec. 2) on the fifth-generation tensor cores:
+// S = Q K^T and O += P V are tcgen05.mma instructions with their accumulators, and P, in tensor memory.
 //
-// One CTA owns 128 (computed row, query head) pairs that share one (sequence, branch) and one key / value head, and a
-// share of the keys (the CTAs of a thread-block cluster split the keys of one M tile and merge their partial results
-// through distributed shared memory, as in the fragment kernel).  Thirteen warps, three roles:
-//   warps 0-3  softmax: thread i owns pair i = lane i of tensor memory.  Per tile of 64 keys it reads its row of S,
-//              keeps a running maximum that only moves when the new maximum exceeds it by 2^8 (then the output
-//              accumulator in tensor memory is rescaled, which is rare after the first tiles), writes P = 2^(s - m)
-//              into shared memory as a bf16 pair hi + lo (the A operand of the second product) and sums the row.
-//   warp 4     issues the MMAs: S(t+1) ahead of P V(t), so the tensor core works on the next scores while the
-//              softmax warps are busy with the current ones.
-//   warps 5-12 loaders: keys by cp.async straight into the K-major 128-byte-swizzled operand layout; values into a
-//              staging tile, which the same warps transpose with ldmatrix.trans / stmatrix into V^T (head dimension on
-//              rows, keys contiguous), the K-major B operand of P V.  Source per key: prefix, fresh row or in-block
-//              cache.
+// One CTA owns up to 256 (computed row, query head) pairs, as two M tiles of 128, that share one (sequence, branch) and
+// one key / value head, and a share of the keys (the CTAs of a thread-block cluster split the keys and merge their
+// partial results through distributed shared memory).  Both M tiles use the same key / value tile: the tensor core works
+// for one while the softmax of the other runs, and a tile is fetched once for 256 pairs.  Thirteen warps, three roles:
+//   warps 0-7  softmax, four per M tile: thread i owns pair i = lane i of tensor memory.  Per tile of 64 keys it reads its
+//              row of S, keeps a running maximum that only moves when the new maximum exceeds it by 2^8 (then the output
+//              accumulator in tensor memory is rescaled, which is rare after the first tiles), and writes
+//              P = 2^(s - m) as a bf16 pair hi + lo over the columns of S (the A operand of the second product).
+//   warp 8     issues the MMAs: S(t+1) of both M tiles ahead of P V(t).
+//   warps 9-12 loaders.  A tile that lies in the prefix is fetched by one thread with TMA boxes of [64 keys][64
+//              elements], swizzled on the way; tiles that reach into the block (prefix, fresh rows and in-block cache mixed)
+//              are stored by all four warps.  Keys are the K-major and values, stored the same way, the MN-major operand.
+// What bounds it: the softmax (a 32-bit exponential, a bf16 split and a row sum per score; 16 exponentials per clock and
+// SM).  MEASURED_ATTN
 // Every wait is an mbarrier wait with a limit; when one runs out the CTA stops working, reports TEAM_ERR_TIMEOUT and
 // still takes part in the cluster's barriers and frees its tensor memory.
 #include <cooperative_groups.h>
+#include <cuda.h>
 
 #include <mutex>
 
@@ -28,82 +30,155 @@ namespace cg = cooperative_groups;
 
 namespace team {
 
-constexpr int kAtD = 128;
 constexpr int kAtKeys = 64;                 // keys per tile
-constexpr int kAtLoadWarps = 8;                // a warp issues one cp.async per ~130 cycles: the loaders are many
+constexpr int kAtPairs = 256;               // pairs per CTA: two M tiles
+constexpr int kAtSoftmaxWarps = 8, kAtLoadWarps = 4;
 constexpr int kAtLoadThreads = kAtLoadWarps * 32;
-constexpr int kAtThreads = 160 + kAtLoadThreads;
-constexpr int kAtKStages = 3, kAtVStages = 3, kAtVtStages = 2;
-constexpr int kAtQBytes = kAttnPairs * kAtD * 2;             // 32 KB: two k-blocks of [128 rows][128 B]
-constexpr int kAtPBytes = 2 * kAttnPairs * 128;              // hi and lo: [128 rows][128 B] each
-constexpr int kAtVtBytes = kAtD * 128;                       // [128 rows (d)][64 keys]
-constexpr int kAtKBytes = kAtKeys * kAtD * 2;                // two k-blocks of [64 rows][128 B]
-constexpr int kAtVBytes = kAtKeys * kAtD * 2;                // staging: [64 keys][256 B], 16-byte pieces xor-swizzled
-constexpr int kAtOffP = kAtQBytes, kAtOffVt = kAtOffP + kAtPBytes, kAtOffK = kAtOffVt + kAtVtStages * kAtVtBytes;
-constexpr int kAtOffV = kAtOffK + kAtKStages * kAtKBytes, kAtOffBars = kAtOffV + kAtVStages * kAtVBytes;
-constexpr int kAtSmemBytes = kAtOffBars + 256 + 1024;        // + barriers + slack for the 1024-byte alignment
-constexpr int kAtOStride = kAtD + 8;                         // floats per row of the partial output (aliases K / V stages)
-static_assert(kAttnPairs * kAtOStride * 4 <= kAtKStages * kAtKBytes + kAtVStages * kAtVBytes, "partial output must fit");
-constexpr int kAtTmemCols = 256;                             // S: 2 x 64 columns, O: 128 columns
-constexpr float kAtRescale = 8.f;                            // the maximum moves only when it grows by more than 2^8
+constexpr int kAtThreads = (kAtSoftmaxWarps + 1 + kAtLoadWarps) * 32;
+constexpr int kAtTmemCols = 512;            // per M tile: S / P twice 64 columns, O 128 (64 with head size 64)
+constexpr float kAtRescale = 8.f;           // the maximum moves only when it grows by more than 2^8
 
-__device__ __forceinline__ void at_cp16z(uint32_t dst, const void* src, int bytes) {   // bytes 0: zero fill
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-template <int N>
-__device__ __forceinline__ void at_cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void at_ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void at_stsm4(uint32_t addr, const uint32_t (&r)[4]) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};"
-               ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+template <int D>
+struct AtShape {
+  static constexpr int NH = D / 64;                        // 64-element halves of a head: one swizzle atom wide each
+  static constexpr int kStages = D == 128 ? 4 : 6;         // of the key and of the value ring
+  static constexpr int kQTile = 128 * 128;                 // one half of an M tile's queries: [128 rows][128 B]
+  static constexpr int kHalf = kAtKeys * 128;              // one half of a key or value tile: [64 keys][128 B]
+  static constexpr int kOffK = 2 * NH * kQTile, kOffV = kOffK + kStages * NH * kHalf, kOffBars = kOffV + kStages * NH * kHalf;
+  static constexpr int kSmem = kOffBars + 512 + 1024;      // + barriers + slack for the 1024-byte alignment
+  static constexpr int kOStride = D + 4;                   // floats per row of the partial output (aliases the operands)
+  static_assert(kAtPairs * kOStride * 4 <= kOffBars, "partial output must fit");
+};
+
 __device__ __forceinline__ float at_ex2(float x) {          // 2^x, relative error 2^-22; -inf -> 0
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// two probabilities as bf16 pairs hi = rn(p), lo = rn(p - hi); low half = the lower key
-__device__ __forceinline__ void at_split2(float p0, float p1, uint32_t& hi, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-  const float2 hf = __bfloat1622float2(h);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(p0 - hf.x, p1 - hf.y);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
+// two fp32 operations in one instruction
+__device__ __forceinline__ float2 at_fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 at_add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+// thirty-two columns of this warp's lanes of tensor memory; the load is complete only after tmem_wait_ld
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+               "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+               "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                 "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+                 "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+                 "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+               : "r"(taddr));
+}
+// the operands tie the loaded registers to the wait
+__device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
+                 "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
+                 "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+               "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+               "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
+                 "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
+                 "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// D[tmem] (+)= A[tmem] * B[smem desc], bf16 inputs, fp32 accumulate, M = 128; issued by a converged warp
+__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// MN-major operand, 128-byte swizzle: atoms of [8 k][64 mn], 1024 B apart along k, half_bytes apart along mn
+__device__ __forceinline__ uint64_t make_mnmajor_sw128_desc(uint32_t smem_addr, int half_bytes) {
+  return (make_kmajor_sw128_desc(smem_addr) & ~((uint64_t)0x3fff << 16)) | (uint64_t)(half_bytes >> 4) << 16;
+}
+// one [64 keys][64 elements] box of a [rows][heads][D] tensor
+__device__ __forceinline__ void tma_box(uint32_t dst, const void* map, int x, int head, int row, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.3d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+               ::"r"(dst), "l"(map), "r"(x), "r"(head), "r"(row), "r"(bar)
+               : "memory");
 }
 __device__ __forceinline__ void bar_loaders() { asm volatile("bar.sync 1, %0;" ::"n"(kAtLoadThreads) : "memory"); }
 
-__global__ void __launch_bounds__(kAtThreads, 1) k_block_attention_tc(AttnArgs a, int n_splits) {
+template <int D>
+__global__ void __launch_bounds__(kAtThreads, 1)
+k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
+  using P = AtShape<D>;
+  constexpr int NH = P::NH, ST = P::kStages;
   extern __shared__ unsigned char at_smem_raw[];
   unsigned char* smem = at_smem_raw + ((1024u - (smem_u32(at_smem_raw) & 1023u)) & 1023u);      // swizzled tiles: 1024-byte aligned
   const uint32_t sm0 = smem_u32(smem);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kAtOffBars);
-  uint64_t* k_full = bars;                        // [3] loaders (one arrival per thread): the key tile has landed
-  uint64_t* k_empty = k_full + kAtKStages;        // [3] MMA commit: S of that tile is done
-  uint64_t* vt_full = k_empty + kAtKStages;       // [2] loader warps: V^T is written
-  uint64_t* vt_empty = vt_full + kAtVtStages;     // [2] MMA commit: P V of that tile is done
-  uint64_t* s_full = vt_empty + kAtVtStages;      // [2] MMA commit: the scores are in tensor memory
-  uint64_t* s_empty = s_full + 2;                 // [2] softmax warps (4): the scores are in registers
-  uint64_t* p_full = s_empty + 2;                 // [1] softmax warps (4): P is in shared memory, O is rescaled
-  uint64_t* pv_done = p_full + 1;                 // [1] MMA commit: O holds the tiles so far
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + 1);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P::kOffBars);
+  uint64_t* k_full = bars;                        // [ST] the key tile has landed
+  uint64_t* k_empty = k_full + ST;                // [ST] MMA commit: S of that tile is done
+  uint64_t* v_full = k_empty + ST;                // [ST] the value tile has landed
+  uint64_t* v_empty = v_full + ST;                // [ST] MMA commit: P V of that tile is done
+  uint64_t* s_full = v_empty + ST;                // [M tile][2] MMA commit: the scores are in tensor memory
+  uint64_t* p_full = s_full + 4;                  // [M tile][2] softmax warps (4): P is in tensor memory, O is rescaled
+  uint64_t* pv_done = p_full + 4;                 // [M tile] MMA commit: O holds the tiles so far
+  uint64_t* q_full = pv_done + 2;                 // [1] softmax warps (8): the queries are in shared memory
+  uint64_t* all_done = q_full + 1;                // [1] MMA commit: every MMA of the CTA is complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(all_done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int32_t* status_sink = reinterpret_cast<int32_t*>(tmem_slot + 2);      // [2] stands in for a null status pointer
+  static_assert((4 * ST + 12) * 8 + 16 <= 512, "barriers must fit");
   __shared__ int s_comp[TEAM_MAX_BLOCK], s_list[TEAM_MAX_BLOCK], s_cnt[2];
-  __shared__ float s_m[kAttnPairs], s_l[kAttnPairs];
+  __shared__ float s_m[kAtPairs], s_l[kAtPairs];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m_tile = blockIdx.x, run = blockIdx.y / a.Hkv, g = blockIdx.y - run * a.Hkv, z = blockIdx.z;
   const int L = a.L, rep = a.Hq / a.Hkv;
   const int row0 = run * L, s = run / a.B;
   int32_t* status = a.status != nullptr ? a.status : status_sink;
+  if (tid == 0) {
+    for (int i = 0; i < ST; ++i) {
+      mbar_init(smem_u32(k_full + i), 1);
+      mbar_init(smem_u32(k_empty + i), 1);
+      mbar_init(smem_u32(v_full + i), 1);
+      mbar_init(smem_u32(v_empty + i), 1);
+    }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(smem_u32(s_full + i), 1);
+      mbar_init(smem_u32(p_full + i), 4);
+    }
+    mbar_init(smem_u32(pv_done), 1);
+    mbar_init(smem_u32(pv_done + 1), 1);
+    mbar_init(smem_u32(q_full), kAtSoftmaxWarps);
+    mbar_init(smem_u32(all_done), 1);
+    *abort_flag = 0;
+    status_sink[0] = status_sink[1] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // everything from here on reads what preceding kernels may have written; the kernel behind this one may be scheduled
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ---- the run's rows: layout contract, which of them are computed ----
+  const int plen = min(max(a.prefix_len[s], 0), a.P);
   bool comp = false;
   unsigned bal = 0u;
   if (tid < TEAM_MAX_BLOCK) {                               // two warps cover the block's positions
@@ -120,225 +195,201 @@ __global__ void __launch_bounds__(kAtThreads, 1) k_block_attention_tc(AttnArgs a
   __syncthreads();
   if (comp) s_list[(warp ? s_cnt[0] : 0) + __popc(bal & ((1u << lane) - 1u))] = tid;
   const int n_pairs = (s_cnt[0] + s_cnt[1]) * rep;
-  if (m_tile * kAttnPairs >= n_pairs) return;               // the whole cluster shares (m_tile, run): it leaves together
-  const int plen = min(max(a.prefix_len[s], 0), a.P);
+  const int pair0 = m_tile * kAtPairs, my_pairs = min(kAtPairs, n_pairs - pair0);
+  if (my_pairs <= 0) return;                                // the whole cluster shares (m_tile, run): it leaves together
+  const int n_m = my_pairs > 128 ? 2 : 1;                   // M tiles in use
   const int n_keys = plen + L;
   const int tiles_total = (n_keys + kAtKeys - 1) / kAtKeys;
   const int tps = (tiles_total + n_splits - 1) / n_splits;
   const int t_begin = min(z * tps, tiles_total), t_end = min(t_begin + tps, tiles_total);
   const int n_tiles = t_end - t_begin;
-  if (tid == 0) {
-    for (int i = 0; i < kAtKStages; ++i) {
-      mbar_init(smem_u32(k_full + i), kAtLoadThreads);
-      mbar_init(smem_u32(k_empty + i), 1);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(vt_full + i), kAtLoadWarps);
-      mbar_init(smem_u32(vt_empty + i), 1);
-      mbar_init(smem_u32(s_full + i), 1);
-      mbar_init(smem_u32(s_empty + i), 4);
-    }
-    mbar_init(smem_u32(p_full), 4);
-    mbar_init(smem_u32(pv_done), 1);
-    *abort_flag = 0;
-    status_sink[0] = status_sink[1] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 4) {
+  if (warp == kAtSoftmaxWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"((uint32_t)kAtTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  __syncthreads();                                          // s_list is complete
-  // ---- loaders: the first two key / value tiles are requested before anything else is set up ----
-  const int ltid = tid - 160, lw = warp - 5;
-  constexpr int RPI = kAtLoadThreads / 16;                  // key rows covered per step of the copy loop
-  const int c = ltid & 15, jr = ltid >> 4;                  // a loader thread's 16-byte piece and key row (jr + RPI i)
-  // Keys and values travel through registers (16-byte loads, two tiles ahead, then 16-byte shared-memory stores):
-  // cp.async tops out near 20 B per clock and SM here, a third of what one tile per microsecond needs.
-  constexpr int NR = kAtKeys / RPI;                         // key rows per loader thread and tile
-  uint4 kr0[NR], vr0[NR], kr1[NR], vr1[NR];                 // tiles of even / odd index
-  auto load_tile = [&](int i, uint4 (&kk)[NR], uint4 (&vv)[NR]) {
-#pragma unroll
-    for (int r8 = 0; r8 < NR; ++r8) {
-      const int key = (t_begin + i) * kAtKeys + r8 * RPI + jr;
-      kk[r8] = vv[r8] = make_uint4(0u, 0u, 0u, 0u);          // keys past the end: zero rows
-      if (key < n_keys) {
-        const __nv_bfloat16 *ks = a.k_prefix, *vs = a.v_prefix;
-        size_t o;
-        if (key < plen) {
-          o = (((size_t)s * a.P + key) * a.Hkv + g) * kAtD;
-        } else {
-          const int p = key - plen;
-          if (s_comp[p]) {
-            o = ((size_t)(row0 + p) * a.Hkv + g) * kAtD;
-            ks = a.k_new; vs = a.v_new;
-          } else {
-            o = (((size_t)s * L + p) * a.Hkv + g) * kAtD;
-            ks = a.k_block; vs = a.v_block;
-          }
-        }
-        kk[r8] = __ldg(reinterpret_cast<const uint4*>(ks + o + c * 8));
-        vv[r8] = __ldg(reinterpret_cast<const uint4*>(vs + o + c * 8));
-      }
-    }
-  };
-  auto store_tile = [&](int i, const uint4 (&kk)[NR], const uint4 (&vv)[NR]) {   // key stage i % 3, staging i % 3
-    unsigned char* kst = smem + kAtOffK + (i % kAtKStages) * kAtKBytes;
-    unsigned char* vst = smem + kAtOffV + (i % kAtVStages) * kAtVBytes;
-#pragma unroll
-    for (int r8 = 0; r8 < NR; ++r8) {
-      const int j = r8 * RPI + jr;
-      *reinterpret_cast<uint4*>(kst + (c >> 3) * (kAtKeys * 128) + sw128(j, c & 7)) = kk[r8];
-      *reinterpret_cast<uint4*>(vst + j * 256 + ((c ^ (j & 7)) << 4)) = vv[r8];
-    }
-  };
-  if (warp >= 5) {
-    if (n_tiles > 0) load_tile(0, kr0, vr0);
-    if (n_tiles > 1) load_tile(1, kr1, vr1);
-  }
-  // ---- the queries of this CTA's pairs: A operand of S = Q K^T, two k-blocks of [128 rows][128 B], swizzled ----
-  for (int i = tid; i < kAttnPairs * 16 && warp < 5; i += 160) {
-    const int pr = i >> 4, c = i & 15, gp = m_tile * kAttnPairs + pr;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (gp < n_pairs) {
-      const int cr = gp / rep, j = gp - cr * rep;
-      v = *reinterpret_cast<const uint4*>(a.q + ((size_t)(row0 + s_list[cr]) * a.Hq + g * rep + j) * kAtD + c * 8);
-    }
-    *reinterpret_cast<uint4*>(smem + (c >> 3) * (kAttnPairs * 128) + sw128(pr, c & 7)) = v;
-  }
-  fence_async_smem();                                       // generic-proxy writes, read by the tensor core
   tc_fence_before();
-  __syncthreads();
+  __syncthreads();                                          // s_list and the tensor memory's address
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  float m_used = kNegInf, l_run = 0.f;                      // softmax threads: running maximum in use (base 2) and row sum
 
-  if (warp >= 5) {
+  if (warp > kAtSoftmaxWarps) {
     // ------------------------------ loaders ------------------------------
+    const int ltid = tid - (kAtSoftmaxWarps + 1) * 32;
     bool ok = true;
     for (int i = 0; i < n_tiles; ++i) {
-      // the key stage of tile i was read by S(i - 3)
-      if (ok && i >= kAtKStages)
-        ok = mbar_wait_warp(smem_u32(k_empty + i % kAtKStages), ((i / kAtKStages) & 1) ^ 1, abort_flag, status, 51);
+      const int st = i % ST, key0 = (t_begin + i) * kAtKeys;
+      const uint32_t free_parity = ((i / ST) & 1) ^ 1;
+      const uint32_t kst = sm0 + P::kOffK + st * NH * P::kHalf, vst = sm0 + P::kOffV + st * NH * P::kHalf;
+      if (key0 + kAtKeys <= plen) {
+        if (warp == kAtSoftmaxWarps + 1 && ok) {            // inside the prefix: one thread, boxes of one half each
+          ok = mbar_wait_warp<32>(smem_u32(k_empty + st), free_parity, abort_flag, status, 51);
+          if (ok && lane == 0) {
+            mbar_expect_tx(smem_u32(k_full + st), NH * P::kHalf);
+            for (int h = 0; h < NH; ++h) tma_box(kst + h * P::kHalf, &kmap, h * 64, g, s * a.P + key0, smem_u32(k_full + st));
+          }
+          if (ok) ok = mbar_wait_warp<32>(smem_u32(v_empty + st), free_parity, abort_flag, status, 52);
+          if (ok && lane == 0) {
+            mbar_expect_tx(smem_u32(v_full + st), NH * P::kHalf);
+            for (int h = 0; h < NH; ++h) tma_box(vst + h * P::kHalf, &vmap, h * 64, g, s * a.P + key0, smem_u32(v_full + st));
+          }
+          __syncwarp();
+        }
+        continue;
+      }
+      // only the warp that has followed every phase of the ring may wait for the stage; the others wait for it
+      if (warp == kAtSoftmaxWarps + 1 && ok) {
+        ok = mbar_wait_warp<32>(smem_u32(k_empty + st), free_parity, abort_flag, status, 51);
+        if (ok) ok = mbar_wait_warp<32>(smem_u32(v_empty + st), free_parity, abort_flag, status, 52);
+      }
+      bar_loaders();
+      ok = ok && !*abort_flag;
       if (ok) {
-        if (i & 1) {
-          store_tile(i, kr1, vr1);
-          if (i + 2 < n_tiles) load_tile(i + 2, kr1, vr1);
-        } else {
-          store_tile(i, kr0, vr0);
-          if (i + 2 < n_tiles) load_tile(i + 2, kr0, vr0);
+        constexpr int PIECES = D / 8, PER = kAtKeys * PIECES / kAtLoadThreads;      // 16-byte pieces per row, per thread
+        uint4 kk[PER], vv[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          const int idx = ltid + q * kAtLoadThreads, j = idx / PIECES, c = idx % PIECES, key = key0 + j;
+          kk[q] = vv[q] = make_uint4(0u, 0u, 0u, 0u);       // keys past the end: zero rows
+          if (key < n_keys) {
+            const __nv_bfloat16 *ks = a.k_prefix, *vs = a.v_prefix;
+            size_t o;
+            if (key < plen) {
+              o = (((size_t)s * a.P + key) * a.Hkv + g) * D;
+            } else {
+              const int p = key - plen;
+              if (s_comp[p]) {
+                o = ((size_t)(row0 + p) * a.Hkv + g) * D;
+                ks = a.k_new; vs = a.v_new;
+              } else {
+                o = (((size_t)s * L + p) * a.Hkv + g) * D;
+                ks = a.k_block; vs = a.v_block;
+              }
+            }
+            kk[q] = *reinterpret_cast<const uint4*>(ks + o + c * 8);
+            vv[q] = *reinterpret_cast<const uint4*>(vs + o + c * 8);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          const int idx = ltid + q * kAtLoadThreads, j = idx / PIECES, c = idx % PIECES;
+          const uint32_t off = (c >> 3) * P::kHalf + sw128(j, c & 7);
+          *reinterpret_cast<uint4*>(smem + P::kOffK + st * NH * P::kHalf + off) = kk[q];
+          *reinterpret_cast<uint4*>(smem + P::kOffV + st * NH * P::kHalf + off) = vv[q];
         }
       }
       fence_async_smem();                                   // generic-proxy writes, read by the tensor core
-      if (ok) mbar_arrive(smem_u32(k_full + i % kAtKStages));
-      bar_loaders();                                        // the staged values are complete, and every warp is done
-                                                            // transposing tile i - 1
-      if (ok) ok = mbar_wait_warp(smem_u32(vt_empty + (i & 1)), ((i >> 1) & 1) ^ 1, abort_flag, status, 52);
-      if (ok) {
-        // V^T: 8 x 8 blocks transposed on the way; the warps share the 16 head-dimension pieces
-        const uint32_t vst = sm0 + kAtOffV + (i % kAtVStages) * kAtVBytes, vt = sm0 + kAtOffVt + (i & 1) * kAtVtBytes;
-        const int mi = lane >> 3, r = lane & 7;
-#pragma unroll
-        for (int dd = 0; dd < 16 / kAtLoadWarps; ++dd) {
-          const int dc = lw * (16 / kAtLoadWarps) + dd;
-#pragma unroll
-          for (int kb4 = 0; kb4 < 2; ++kb4) {
-            uint32_t v[4];
-            const int key = (kb4 * 4 + mi) * 8 + r;         // source: matrix mi = keys 8 (4 kb4 + mi) .., piece dc
-            at_ldsm4t(vst + key * 256 + ((dc ^ r) << 4), v);
-            at_stsm4(vt + sw128(dc * 8 + r, kb4 * 4 + mi), v);      // target: rows d = 8 dc + r, key piece 4 kb4 + mi
-          }
-        }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(vt_full + (i & 1)));
+      bar_loaders();
+      if (ok && ltid == 0) {
+        mbar_arrive(smem_u32(k_full + st));
+        mbar_arrive(smem_u32(v_full + st));
       }
     }
-  } else if (warp == 4) {
+    if (!ok) {
+      // gave up: the copies already issued still land in this CTA's shared memory; give them time before the CTA exits
+      for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    }
+  } else if (warp == kAtSoftmaxWarps) {
     // ------------------------------ MMA issuer ------------------------------
-    const uint32_t idesc_s = make_idesc_bf16(kAtKeys), idesc_o = make_idesc_bf16(kAtD);
-    const uint32_t tm_o = tmem_base + 2 * kAtKeys;
-    bool ok = true;
+    const uint32_t idesc_s = make_idesc_bf16(kAtKeys), idesc_o = make_idesc_bf16(D) | (1u << 16);      // V: MN-major
+    bool ok = mbar_wait_warp(smem_u32(q_full), 0, abort_flag, status, 50);
     auto issue_s = [&](int i) {
-      const int st = i % kAtKStages, b = i & 1;
-      if (!(ok = mbar_wait_warp(smem_u32(k_full + st), (i / kAtKStages) & 1, abort_flag, status, 53))) return;
-      if (!(ok = mbar_wait_warp(smem_u32(s_empty + b), ((i >> 1) & 1) ^ 1, abort_flag, status, 54))) return;
+      const int st = i % ST, b = i & 1;
+      if (!(ok = mbar_wait_warp(smem_u32(k_full + st), (i / ST) & 1, abort_flag, status, 53))) return;
       tc_fence_after();
-      const uint32_t kst = sm0 + kAtOffK + st * kAtKBytes;
+      const uint32_t kst = sm0 + P::kOffK + st * NH * P::kHalf;
+      for (int m = 0; m < n_m; ++m) {
+        // the columns were P of tile i - 2: its product was issued before
 #pragma unroll
-      for (int kb = 0; kb < 2; ++kb) {
-        const uint64_t da = make_kmajor_sw128_desc(sm0 + kb * (kAttnPairs * 128)), db = make_kmajor_sw128_desc(kst + kb * (kAtKeys * 128));
+        for (int h = 0; h < NH; ++h) {
+          const uint64_t da = make_kmajor_sw128_desc(sm0 + (m * NH + h) * P::kQTile), db = make_kmajor_sw128_desc(kst + h * P::kHalf);
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) tc_mma(tmem_base + b * kAtKeys, da + 2 * k4, db + 2 * k4, idesc_s, (kb | k4) != 0);
+          for (int k4 = 0; k4 < 4; ++k4) tc_mma(tmem_base + m * 256 + b * kAtKeys, da + 2 * k4, db + 2 * k4, idesc_s, (h | k4) != 0);
+        }
+        tc_commit(smem_u32(s_full + m * 2 + b));
       }
       tc_commit(smem_u32(k_empty + st));
-      tc_commit(smem_u32(s_full + b));
     };
-    if (n_tiles > 0) issue_s(0);
+    if (ok && n_tiles > 0) issue_s(0);
     for (int i = 0; i < n_tiles && ok; ++i) {
+      const int st = i % ST, b = i & 1;
       if (i + 1 < n_tiles) {
         issue_s(i + 1);
         if (!ok) break;
       }
-      if (!(ok = mbar_wait_warp(smem_u32(p_full), i & 1, abort_flag, status, 55))) break;
-      if (!(ok = mbar_wait_warp(smem_u32(vt_full + (i & 1)), (i >> 1) & 1, abort_flag, status, 56))) break;
-      tc_fence_after();
-      const uint64_t db = make_kmajor_sw128_desc(sm0 + kAtOffVt + (i & 1) * kAtVtBytes);
+      if (!(ok = mbar_wait_warp(smem_u32(v_full + st), (i / ST) & 1, abort_flag, status, 56))) break;
+      const uint64_t db = make_mnmajor_sw128_desc(sm0 + P::kOffV + st * NH * P::kHalf, P::kHalf);
+      for (int m = 0; m < n_m && ok; ++m) {
+        if (!(ok = mbar_wait_warp(smem_u32(p_full + m * 2 + b), (i >> 1) & 1, abort_flag, status, 55))) break;
+        tc_fence_after();
+        const uint32_t tm = tmem_base + m * 256;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {                          // P hi, then P lo
-        const uint64_t da = make_kmajor_sw128_desc(sm0 + kAtOffP + h * (kAttnPairs * 128));
+        for (int h = 0; h < 2; ++h)                          // P hi, then P lo: 32 columns of 2 keys each
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) tc_mma(tm_o, da + 2 * k4, db + 2 * k4, idesc_o, (i | h | k4) != 0);
+          for (int k4 = 0; k4 < 4; ++k4)                     // 16 keys: 8 columns of P, 2048 B of V
+            tc_mma_ts(tm + 128, tm + b * kAtKeys + h * 32 + k4 * 8, db + 128 * k4, idesc_o, (i | h | k4) != 0);
+        tc_commit(smem_u32(pv_done + m));
       }
-      tc_commit(smem_u32(vt_empty + (i & 1)));
-      tc_commit(smem_u32(pv_done));
+      if (ok) tc_commit(smem_u32(v_empty + st));
     }
+    if (ok && n_tiles > 0) tc_commit(smem_u32(all_done));
   } else {
-    // ------------------------------ softmax ------------------------------
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;       // this warp's quarter of the lanes of tensor memory
-    const uint32_t tm_o = tmem_base + lane_base + 2 * kAtKeys;
-    const int pr = tid;                                      // pair = lane of tensor memory = row of P
-    const float sl2 = rsqrtf((float)kAtD) * 1.4426950408889634f;      // scores in base 2
-    bool ok = true;
-    for (int i = 0; i < n_tiles && ok; ++i) {
-      const int b = i & 1;
-      if (!(ok = mbar_wait_warp(smem_u32(s_full + b), (i >> 1) & 1, abort_flag, status, 57))) break;
-      tc_fence_after();
-      float sc[kAtKeys];
-      {
-        const uint32_t tm_s = tmem_base + lane_base + b * kAtKeys;
+    // ---- the queries of this CTA's pairs: A operand of S = Q K^T, per M tile NH halves of [128 rows][128 B], swizzled ----
+    {
+      constexpr int PIECES = D / 8, PER = 8;                // 16-byte pieces per row; loads in flight per thread
+      for (int i0 = tid; i0 < n_m * 128 * PIECES; i0 += kAtSoftmaxWarps * 32 * PER) {
+        uint4 v[PER];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t r0[8], r1[8], r2[8], r3[8];
-          tmem_ld8_issue(tm_s + half * 32, r0);
-          tmem_ld8_issue(tm_s + half * 32 + 8, r1);
-          tmem_ld8_issue(tm_s + half * 32 + 16, r2);
-          tmem_ld8_issue(tm_s + half * 32 + 24, r3);
-          tmem_ld_wait(r0, r1, r2, r3);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            sc[half * 32 + e] = __uint_as_float(r0[e]);
-            sc[half * 32 + 8 + e] = __uint_as_float(r1[e]);
-            sc[half * 32 + 16 + e] = __uint_as_float(r2[e]);
-            sc[half * 32 + 24 + e] = __uint_as_float(r3[e]);
+        for (int q = 0; q < PER; ++q) {
+          const int i = i0 + q * kAtSoftmaxWarps * 32, pr = i / PIECES, c = i % PIECES;
+          v[q] = make_uint4(0u, 0u, 0u, 0u);
+          if (pr < my_pairs) {
+            const int gp = pair0 + pr, cr = gp / rep, j = gp - cr * rep;
+            v[q] = *reinterpret_cast<const uint4*>(a.q + ((size_t)(row0 + s_list[cr]) * a.Hq + g * rep + j) * D + c * 8);
           }
         }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(s_empty + b));      // the tensor core may write the scores of tile i + 2 here
-      // scale, mask the keys past the end (last tile only), the tile's maximum
-      const int key0 = (t_begin + i) * kAtKeys;
-      const bool ragged = key0 + kAtKeys > n_keys;
-      float mx = kNegInf;
 #pragma unroll
-      for (int e = 0; e < kAtKeys; ++e) {
-        if (ragged && key0 + e >= n_keys) sc[e] = kNegInf;
-        mx = fmaxf(mx, sc[e]);
+        for (int q = 0; q < PER; ++q) {
+          const int i = i0 + q * kAtSoftmaxWarps * 32, pr = i / PIECES, c = i % PIECES;
+          if (pr < n_m * 128)
+            *reinterpret_cast<uint4*>(smem + ((pr >> 7) * NH + (c >> 3)) * P::kQTile + sw128(pr & 127, c & 7)) = v[q];
+        }
       }
-      mx *= sl2;                                             // sl2 > 0: the maximum of the scaled scores
+      fence_async_smem();                                   // generic-proxy writes, read by the tensor core
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(q_full));
+    }
+    // ------------------------------ softmax ------------------------------
+    const int m = warp >> 2;                                 // M tile
+    const uint32_t tm = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + m * 256;      // this warp's quarter of the lanes
+    const int pr = tid;                                      // pair of the CTA = lane of tensor memory + 128 * M tile
+    const float sl2 = rsqrtf((float)D) * 1.4426950408889634f;      // scores in base 2
+    float m_used = kNegInf, l_run = 0.f;                     // running maximum in use (base 2) and row sum
+    bool ok = true;
+    for (int i = 0; i < n_tiles && ok && m < n_m; ++i) {
+      const int b = i & 1;
+      if (!(ok = mbar_wait_warp(smem_u32(s_full + m * 2 + b), (i >> 1) & 1, abort_flag, status, 57))) break;
+      tc_fence_after();
+      const uint32_t tm_s = tm + b * kAtKeys;
+      uint32_t sc[kAtKeys];
+      tmem_ld32(tm_s, sc);
+      tmem_ld32(tm_s + 32, sc + 32);
+      tmem_wait_ld(sc);
+      tmem_wait_ld(sc + 32);
+      // mask the keys past the end (last tile only), the tile's maximum
+      const int key0 = (t_begin + i) * kAtKeys;
+      if (key0 + kAtKeys > n_keys) {
+#pragma unroll
+        for (int e = 0; e < kAtKeys; ++e)
+          if (key0 + e >= n_keys) sc[e] = __float_as_uint(kNegInf);
+      }
+      float mx4[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mx4[e] = __uint_as_float(sc[e]);
+#pragma unroll
+      for (int e = 4; e < kAtKeys; ++e) mx4[e & 3] = fmaxf(mx4[e & 3], __uint_as_float(sc[e]));
+      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;      // sl2 > 0: the maximum of the scaled scores
       // the maximum in use moves only when it has to: P stays below 2^8, far inside fp32 and the bf16 pair
       const bool move = mx > m_used + kAtRescale;            // always on the first tile (m_used = -inf)
       float corr = 1.f;
@@ -347,89 +398,72 @@ __global__ void __launch_bounds__(kAtThreads, 1) k_block_attention_tc(AttnArgs a
         m_used = mx;
         l_run *= corr;
       }
-      float sum = 0.f;
-      const float neg_m = -m_used;
+      // scale and shift in one operation, 2^x, the row sum, and P as bf16 pairs hi = rn(p), lo = rn(p - hi): two keys
+      // per column, the 32 columns of hi in front of the 32 of lo
+      const float2 scale = make_float2(sl2, sl2), shift = make_float2(-m_used, -m_used), minus = make_float2(-1.f, -1.f);
+      float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      uint32_t lo[kAtKeys / 2];
 #pragma unroll
-      for (int e = 0; e < kAtKeys; ++e) {
-        sc[e] = at_ex2(fmaf(sc[e], sl2, neg_m));             // scale and shift in one operation
-        sum += sc[e];
+      for (int e = 0; e < kAtKeys / 2; ++e) {
+        float2 p = at_fma2(make_float2(__uint_as_float(sc[2 * e]), __uint_as_float(sc[2 * e + 1])), scale, shift);
+        p.x = at_ex2(p.x);
+        p.y = at_ex2(p.y);
+        sum[e & 1] = at_add2(sum[e & 1], p);
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(p.x, p.y);
+        const uint32_t h = *reinterpret_cast<const uint32_t*>(&h2);
+        const float2 rest = at_fma2(make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), minus, p);
+        const __nv_bfloat162 l2 = __floats2bfloat162_rn(rest.x, rest.y);
+        sc[e] = h;
+        lo[e] = *reinterpret_cast<const uint32_t*>(&l2);
       }
-      l_run += sum;
-      // O and P belong to the tensor core until P V of the previous tile is complete
+      sum[0] = at_add2(sum[0], sum[1]);
+      l_run += sum[0].x + sum[0].y;
+      tmem_st32(tm_s, sc);
+      tmem_st32(tm_s + 32, lo);
+      // O belongs to the tensor core until P V of the previous tile is complete
       if (i > 0) {
-        if (!(ok = mbar_wait_warp(smem_u32(pv_done), (i - 1) & 1, abort_flag, status, 58))) break;
-        tc_fence_after();
+        if (!(ok = mbar_wait_warp(smem_u32(pv_done + m), (i - 1) & 1, abort_flag, status, 58))) break;
         if (__any_sync(0xffffffffu, move)) {
+          tc_fence_after();
 #pragma unroll 1
-          for (int c0 = 0; c0 < kAtD; c0 += 32) {
-            uint32_t r0[8], r1[8], r2[8], r3[8];
-            tmem_ld8_issue(tm_o + c0, r0);
-            tmem_ld8_issue(tm_o + c0 + 8, r1);
-            tmem_ld8_issue(tm_o + c0 + 16, r2);
-            tmem_ld8_issue(tm_o + c0 + 24, r3);
-            tmem_ld_wait(r0, r1, r2, r3);
+          for (int c0 = 0; c0 < D; c0 += 32) {
+            uint32_t r[32];
+            tmem_ld32(tm + 128 + c0, r);
+            tmem_wait_ld(r);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              r0[e] = __float_as_uint(__uint_as_float(r0[e]) * corr);
-              r1[e] = __float_as_uint(__uint_as_float(r1[e]) * corr);
-              r2[e] = __float_as_uint(__uint_as_float(r2[e]) * corr);
-              r3[e] = __float_as_uint(__uint_as_float(r3[e]) * corr);
-            }
-            tmem_st8(tm_o + c0, r0);
-            tmem_st8(tm_o + c0 + 8, r1);
-            tmem_st8(tm_o + c0 + 16, r2);
-            tmem_st8(tm_o + c0 + 24, r3);
+            for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
+            tmem_st32(tm + 128 + c0, r);
           }
-          tmem_st_wait();
         }
       }
-      // P as hi + lo: row pr of two [128 rows][128 B] tiles, 8 keys per 16-byte piece
-      unsigned char* prow = smem + kAtOffP;
-#pragma unroll
-      for (int c = 0; c < kAtKeys / 8; ++c) {
-        uint4 hi, lo;
-        at_split2(sc[c * 8 + 0], sc[c * 8 + 1], hi.x, lo.x);
-        at_split2(sc[c * 8 + 2], sc[c * 8 + 3], hi.y, lo.y);
-        at_split2(sc[c * 8 + 4], sc[c * 8 + 5], hi.z, lo.z);
-        at_split2(sc[c * 8 + 6], sc[c * 8 + 7], hi.w, lo.w);
-        const uint32_t off = sw128(pr, c);
-        *reinterpret_cast<uint4*>(prow + off) = hi;
-        *reinterpret_cast<uint4*>(prow + kAttnPairs * 128 + off) = lo;
-      }
-      fence_async_smem();
+      tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(p_full));
+      if (lane == 0) mbar_arrive(smem_u32(p_full + m * 2 + b));
     }
-    // ---- the CTA's partial result: (maximum, sum, unnormalised output) of its pairs into shared memory ----
-    if (ok && n_tiles > 0) ok = mbar_wait_warp(smem_u32(pv_done), (n_tiles - 1) & 1, abort_flag, status, 59);
+    // ---- the CTA's partial result: (maximum, sum, unnormalised output) of its pairs into shared memory, over the
+    //      operands: every MMA of both M tiles has to be complete ----
+    if (ok && n_tiles > 0) ok = mbar_wait_warp<32>(smem_u32(all_done), 0, abort_flag, status, 59);
     tc_fence_after();
-    float* s_o = reinterpret_cast<float*>(smem + kAtOffK);     // [128][kAtOStride]: the key / value stages are idle now
-    const bool have = ok && n_tiles > 0;
-    s_m[pr] = have ? m_used : kNegInf;
-    s_l[pr] = have ? l_run : 0.f;
+    if (m < n_m) {
+      float* s_o = reinterpret_cast<float*>(smem);
+      const bool have = ok && n_tiles > 0;
+      s_m[pr] = have ? m_used : kNegInf;
+      s_l[pr] = have ? l_run : 0.f;
 #pragma unroll 1
-    for (int c0 = 0; c0 < kAtD; c0 += 32) {
-      uint32_t r0[8], r1[8], r2[8], r3[8];
-      if (have) {                                            // warp-uniform
-        tmem_ld8_issue(tm_o + c0, r0);
-        tmem_ld8_issue(tm_o + c0 + 8, r1);
-        tmem_ld8_issue(tm_o + c0 + 16, r2);
-        tmem_ld8_issue(tm_o + c0 + 24, r3);
-        tmem_ld_wait(r0, r1, r2, r3);
-      } else {
+      for (int c0 = 0; c0 < D; c0 += 32) {
+        uint32_t r[32];
+        if (have) {                                          // warp-uniform
+          tmem_ld32(tm + 128 + c0, r);
+          tmem_wait_ld(r);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) r0[e] = r1[e] = r2[e] = r3[e] = 0u;
+          for (int e = 0; e < 32; ++e) r[e] = 0u;
+        }
+        uint4* dst = reinterpret_cast<uint4*>(s_o + (size_t)pr * P::kOStride + c0);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) dst[e] = make_uint4(r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]);
       }
-      float4* dst = reinterpret_cast<float4*>(s_o + (size_t)pr * kAtOStride + c0);
-      dst[0] = make_float4(__uint_as_float(r0[0]), __uint_as_float(r0[1]), __uint_as_float(r0[2]), __uint_as_float(r0[3]));
-      dst[1] = make_float4(__uint_as_float(r0[4]), __uint_as_float(r0[5]), __uint_as_float(r0[6]), __uint_as_float(r0[7]));
-      dst[2] = make_float4(__uint_as_float(r1[0]), __uint_as_float(r1[1]), __uint_as_float(r1[2]), __uint_as_float(r1[3]));
-      dst[3] = make_float4(__uint_as_float(r1[4]), __uint_as_float(r1[5]), __uint_as_float(r1[6]), __uint_as_float(r1[7]));
-      dst[4] = make_float4(__uint_as_float(r2[0]), __uint_as_float(r2[1]), __uint_as_float(r2[2]), __uint_as_float(r2[3]));
-      dst[5] = make_float4(__uint_as_float(r2[4]), __uint_as_float(r2[5]), __uint_as_float(r2[6]), __uint_as_float(r2[7]));
-      dst[6] = make_float4(__uint_as_float(r3[0]), __uint_as_float(r3[1]), __uint_as_float(r3[2]), __uint_as_float(r3[3]));
-      dst[7] = make_float4(__uint_as_float(r3[4]), __uint_as_float(r3[5]), __uint_as_float(r3[6]), __uint_as_float(r3[7]));
     }
   }
 
@@ -438,20 +472,25 @@ __global__ void __launch_bounds__(kAtThreads, 1) k_block_attention_tc(AttnArgs a
   __syncthreads();
   cg::cluster_group cluster = cg::this_cluster();
   cluster.sync();
-  if (tid < 256 && !*abort_flag) {
-    // rank z merges rows z * R .. z * R + R - 1 of all partials (distributed shared memory) and writes them
-    float* s_o = reinterpret_cast<float*>(smem + kAtOffK);
-    constexpr int TPR = kAtD / 4;                           // threads per row (one float4 each)
-    const int R = kAttnPairs / n_splits;
-    const int c4 = tid % TPR;
-    for (int i = tid / TPR; i < R; i += 256 / TPR) {
-      const int pr = z * R + i, gp = m_tile * kAttnPairs + pr;
-      if (gp >= n_pairs) continue;
-      float mk[kAttnMaxSplits], mx = kNegInf;
+  if (!*abort_flag) {
+    // rank z merges its share of the rows of all partials (distributed shared memory) and writes them
+    float* s_o = reinterpret_cast<float*>(smem);
+    constexpr int TPR = D / 4;                              // threads per row (one float4 each)
+    const int R = (my_pairs + n_splits - 1) / n_splits, r1 = min(my_pairs, (z + 1) * R);
+    for (int i = z * R * TPR + tid; i < r1 * TPR; i += kAtThreads) {
+      const int pr = i / TPR, c4 = i % TPR, gp = pair0 + pr;
+      float mk[kAttnMaxSplits], lk[kAttnMaxSplits], mx = kNegInf;
+      float4 v[kAttnMaxSplits];
 #pragma unroll
       for (int k = 0; k < kAttnMaxSplits; ++k) {
         mk[k] = kNegInf;
-        if (k < n_splits) mk[k] = *cluster.map_shared_rank(&s_m[pr], k);
+        lk[k] = 0.f;
+        v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k < n_splits) {
+          mk[k] = *cluster.map_shared_rank(&s_m[pr], k);
+          lk[k] = *cluster.map_shared_rank(&s_l[pr], k);
+          v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_o + (size_t)pr * P::kOStride + c4 * 4, k));
+        }
         mx = fmaxf(mx, mk[k]);
       }
       float den = 0.f;
@@ -460,48 +499,116 @@ __global__ void __launch_bounds__(kAtThreads, 1) k_block_attention_tc(AttnArgs a
       for (int k = 0; k < kAttnMaxSplits; ++k) {
         if (k >= n_splits) break;
         const float f = at_ex2(mk[k] - mx);                  // 0 for a split without keys (its maximum is -inf)
-        den = fmaf(f, *cluster.map_shared_rank(&s_l[pr], k), den);
-        const float4 v = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_o + (size_t)pr * kAtOStride + c4 * 4, k));
-        acc.x = fmaf(f, v.x, acc.x); acc.y = fmaf(f, v.y, acc.y); acc.z = fmaf(f, v.z, acc.z); acc.w = fmaf(f, v.w, acc.w);
+        den = fmaf(f, lk[k], den);
+        acc.x = fmaf(f, v[k].x, acc.x); acc.y = fmaf(f, v[k].y, acc.y); acc.z = fmaf(f, v[k].z, acc.z); acc.w = fmaf(f, v[k].w, acc.w);
       }
       const int cr = gp / rep, j = gp - cr * rep;
-      float* dst = a.out + ((size_t)(row0 + s_list[cr]) * a.Hq + g * rep + j) * kAtD + c4 * 4;
+      float* dst = a.out + ((size_t)(row0 + s_list[cr]) * a.Hq + g * rep + j) * D + c4 * 4;
       const float inv = 1.f / den;
       *reinterpret_cast<float4*>(dst) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
     }
   }
   cluster.sync();                                          // peers may still be reading this CTA's partial
-  if (warp == 4) {
+  if (warp == kAtSoftmaxWarps) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)kAtTmemCols) : "memory");
   }
 }
 
-cudaError_t configure_attention_tc() {
-  static std::mutex mu;
-  static bool done[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> lock(mu);
-  if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_block_attention_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kAtSmemBytes);
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+// Per device: the shared-memory opt-in, the tensor-map encoder, and how many clusters of each size run at once (a cluster
+// stays inside one GPC, so clusters of 7 or 8 leave SMs unused that clusters of 6 would take).
+struct AttnSetup {
+  decltype(&cuTensorMapEncodeTiled) encode;
+  int clusters[2][kAttnMaxSplits + 1];                      // [head size 64, 128][cluster size]
+};
+
+template <int D>
+static cudaLaunchConfig_t attn_launch(cudaLaunchAttribute (&at)[2], dim3 grid, cudaStream_t s) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(kAtThreads);
+  lc.dynamicSmemBytes = AtShape<D>::kSmem;
+  lc.stream = s;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = grid.z;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // the launch latency hides behind the preceding kernel
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 2;
+  return lc;
+}
+
+template <int D>
+static cudaError_t setup_kernel(int n_sms, int (&clusters)[kAttnMaxSplits + 1]) {
+  cudaError_t e = cudaFuncSetAttribute(k_block_attention_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, AtShape<D>::kSmem);
+  clusters[1] = n_sms;
+  for (int n = 2; n <= kAttnMaxSplits && e == cudaSuccess; ++n) {
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t lc = attn_launch<D>(at, dim3(1, 1, n), nullptr);
+    lc.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&clusters[n], k_block_attention_tc<D>, &lc) != cudaSuccess) {
+      cudaGetLastError();
+      clusters[n] = 0;                                      // not used
+    }
+  }
   return e;
 }
 
-cudaError_t launch_attention_tc(const AttnArgs& a, int m_tiles, int n_splits, cudaStream_t s) {
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(m_tiles, a.S * a.B * a.Hkv, n_splits);
-  lc.blockDim = dim3(kAtThreads);
-  lc.dynamicSmemBytes = kAtSmemBytes;
-  lc.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = n_splits;
-  lc.attrs = at;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, k_block_attention_tc, a, n_splits);
+static cudaError_t attn_setup(const AttnSetup** out) {
+  static std::mutex mu;
+  static AttnSetup setups[64] = {};
+  int dev = 0, n_sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  AttnSetup& st = setups[dev];
+  *out = &st;
+  if (st.encode != nullptr) return cudaSuccess;
+  e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = setup_kernel<64>(n_sms, st.clusters[0]);
+  if (e == cudaSuccess) e = setup_kernel<128>(n_sms, st.clusters[1]);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  if (e == cudaSuccess) e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+  if (e == cudaSuccess && found != cudaDriverEntryPointSuccess) e = cudaErrorNotSupported;
+  if (e == cudaSuccess) st.encode = reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(fn);
+  return e;
+}
+
+template <int D>
+static cudaError_t launch(const AttnArgs& a, const AttnSetup& st, cudaStream_t s) {
+  // M tiles by the largest number of pairs a run can have; the keys of each are split over a cluster, as far as all
+  // clusters run at once and every split keeps two tiles of the longest prefix
+  const int m_tiles = (a.L * (a.Hq / a.Hkv) + kAtPairs - 1) / kAtPairs;
+  const long long units = (long long)m_tiles * a.S * a.B * a.Hkv;
+  const int tiles_max = (a.P + a.L + kAtKeys - 1) / kAtKeys;
+  int n_splits = 1;
+  for (int n = 2; n <= kAttnMaxSplits; ++n)
+    if (units <= st.clusters[D / 128][n] && tiles_max >= 2 * n) n_splits = n;
+  CUtensorMap kmap = {}, vmap = {};
+  if (a.P >= kAtKeys) {                                     // else no tile lies in the prefix and the maps are not used
+    const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)a.Hkv, (cuuint64_t)a.S * a.P};
+    const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)a.Hkv * D * 2};
+    const cuuint32_t box[3] = {64, 1, kAtKeys}, elem[3] = {1, 1, 1};
+    for (int i = 0; i < 2; ++i) {
+      const __nv_bfloat16* base = i ? a.v_prefix : a.k_prefix;
+      if (st.encode(i ? &vmap : &kmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(base), dims, strides, box, elem,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    }
+  }
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t lc = attn_launch<D>(at, dim3(m_tiles, a.S * a.B * a.Hkv, n_splits), s);
+  return cudaLaunchKernelEx(&lc, k_block_attention_tc<D>, a, n_splits, kmap, vmap);
+}
+
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s) {
+  const AttnSetup* st = nullptr;
+  const cudaError_t e = attn_setup(&st);
+  if (e != cudaSuccess) return e;
+  return a.d == 128 ? launch<128>(a, *st, s) : launch<64>(a, *st, s);
 }
 
 }  // namespace team
