@@ -58,10 +58,11 @@ extern "C" int team_block_attention(const team_attn_config* cfg, const team_step
   a.out = out;
   a.status = status;
   a.S = cfg->n_seqs; a.B = cfg->n_branches; a.L = cfg->block; a.Hq = cfg->n_heads; a.Hkv = cfg->n_kv_heads;
-  a.d = cfg->head_dim; a.P = cfg->max_prefix; a.flags = cfg->flags;
+  a.d = cfg->head_dim; a.P = cfg->max_prefix; a.flags = cfg->flags; a.insert = 0;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = team::launch_attention_tc(a, s);
-  if (e == cudaSuccess) {
+  bool inserted = false;
+  cudaError_t e = team::launch_attention_tc(a, s, &inserted);
+  if (e == cudaSuccess && !inserted) {
     const int T = a.S * a.B * a.L, pieces = a.Hkv * a.d / 8, blocks = (T * pieces + 255) / 256;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(blocks < 1184 ? blocks : 1184);

@@ -24,11 +24,13 @@ struct AttnArgs {
   float* out;                    // [T, Hq, d]
   int32_t* status;               // [2] optional
   int S, B, L, Hq, Hkv, d, P, flags;
+  int insert;                    // the attention kernel performs the insertion
 };
 
 __device__ __forceinline__ bool attn_computed(int state, int flags) { return !((flags & TEAM_F_DCD) && state == TEAM_TOK_CACHED); }
 
-// the attention itself (team_attn_tc.cu); one-time set-up on a device's first call
-cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s);
+// the attention itself (team_attn_tc.cu), with the insertion where *inserted comes back true; one-time set-up on a
+// device's first call
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s, bool* inserted);
 
 }  // namespace team

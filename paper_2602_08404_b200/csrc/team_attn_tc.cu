@@ -1,10 +1,12 @@
 // The attention half of delayed caching (Sec. 4.1; block diffusion, Sec. 2) on the fifth-generation tensor cores:
 // S = Q K^T and O += P V are tcgen05.mma instructions with their accumulators, and P, in tensor memory.
 //
-// One CTA owns up to 256 (computed row, query head) pairs, as two M tiles of 128, that share one (sequence, branch) and
-// one key / value head, and a share of the keys (the CTAs of a thread-block cluster split the keys and merge their
-// partial results through distributed shared memory).  Both M tiles use the same key / value tile: the tensor core works
-// for one while the softmax of the other runs, and a tile is fetched once for 256 pairs.  Thirteen warps, three roles:
+// The (computed row, query head) pairs of a sequence that share one key / value head are packed over its branches (they
+// attend to the same prefix) and cut into M tiles of 128.  One CTA owns one or two M tiles and a share of the keys (the
+// CTAs of a thread-block cluster split the keys and merge their partial results through distributed shared memory).  The
+// keys of a CTA are the prefix and then the block once per branch that its pairs belong to; a pair sees its own branch's.
+// Two M tiles use the same key / value tile: the tensor core works for one while the softmax of the other runs, and a
+// tile is fetched once for 256 pairs.  Thirteen warps, three roles:
 //   warps 0-7  softmax, four per M tile: thread i owns pair i = lane i of tensor memory.  Per tile of 64 keys it reads its
 //              row of S, keeps a running maximum that only moves when the new maximum exceeds it by 2^8 (then the output
 //              accumulator in tensor memory is rescaled, which is rare after the first tiles), and writes
@@ -13,8 +15,11 @@
 //   warps 9-12 loaders.  A tile that lies in the prefix is fetched by one thread with TMA boxes of [64 keys][64
 //              elements], swizzled on the way; tiles that reach into the block (prefix, fresh rows and in-block cache mixed)
 //              are stored by all four warps.  Keys are the K-major and values, stored the same way, the MN-major operand.
-// What bounds it: the softmax (a 32-bit exponential, a bf16 split and a row sum per score; 16 exponentials per clock and
-// SM).  MEASURED_ATTN
+// What bounds it, per tile of 64 keys and two M tiles: the tensor core, 2000 clock cycles (S at N = 64 reads its A operand
+// as long as it computes, and P counts twice), with the softmax behind it (1300: 16 exponentials per clock and SM); and
+// around the tiles 6000 cycles until the first scores and 5000 to 10000 for the merge, whose reads of distributed shared
+// memory run at about 12 bytes per clock and SM.  Kernel at 4096 cached tokens, 32 query and 4 key / value heads of 128,
+// block of 32 x 4 branches: 43 us with one M tile per CTA, loads through registers and P in shared memory, 25 now.
 // Every wait is an mbarrier wait with a limit; when one runs out the CTA stops working, reports TEAM_ERR_TIMEOUT and
 // still takes part in the cluster's barriers and frees its tensor memory.
 #include <cooperative_groups.h>
@@ -31,7 +36,7 @@ namespace cg = cooperative_groups;
 namespace team {
 
 constexpr int kAtKeys = 64;                 // keys per tile
-constexpr int kAtPairs = 256;               // pairs per CTA: two M tiles
+constexpr int kAtPairs = 256;               // pairs per CTA at most: two M tiles
 constexpr int kAtSoftmaxWarps = 8, kAtLoadWarps = 4;
 constexpr int kAtLoadThreads = kAtLoadWarps * 32;
 constexpr int kAtThreads = (kAtSoftmaxWarps + 1 + kAtLoadWarps) * 32;
@@ -46,6 +51,9 @@ struct AtShape {
   static constexpr int kHalf = kAtKeys * 128;              // one half of a key or value tile: [64 keys][128 B]
   static constexpr int kOffK = 2 * NH * kQTile, kOffV = kOffK + kStages * NH * kHalf, kOffBars = kOffV + kStages * NH * kHalf;
   static constexpr int kSmem = kOffBars + 512 + 1024;      // + barriers + slack for the 1024-byte alignment
+  // head size 64 has room for a second output accumulator, which takes the products of P lo: half as many truncated
+  // additions to the large sum
+  static constexpr int kOLo = D == 64 ? 64 : 0;
   static constexpr int kOStride = D + 4;                   // floats per row of the partial output (aliases the operands)
   static_assert(kAtPairs * kOStride * 4 <= kOffBars, "partial output must fit");
 };
@@ -104,14 +112,28 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
                : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// D[tmem] (+)= A[tmem] * B[smem desc], bf16 inputs, fp32 accumulate, M = 128; issued by a converged warp
-__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// D[tmem] (+)= (A hi + A lo)[tmem] * B[smem desc] over 64 keys: eight instructions of 16 keys (8 columns of A, 2048 B of
+// B), first the 32 columns of hi, then the 32 of lo; bf16 inputs, fp32 accumulate, M = 128; issued by a converged warp.
+// The products of lo go to d_lo, which may be d_tmem.
+__device__ __forceinline__ void tc_mma_ts_hilo(uint32_t d_tmem, uint32_t d_lo, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
+      "{\n\t.reg .pred p, q, t, u;\n\t.reg .b64 b1, b2, b3;\n\t.reg .b32 a1, a2, a3, a4, a5, a6, a7;\n\t"
       "elect.sync _|q, 0xffffffff;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "setp.eq.b32 t, 0, 0;\n\t"
+      "setp.ne.b32 u, %6, 0;\n\t"
+      "add.s64 b1, %2, 128;\n\tadd.s64 b2, %2, 256;\n\tadd.s64 b3, %2, 384;\n\t"
+      "add.u32 a1, %1, 8;\n\tadd.u32 a2, %1, 16;\n\tadd.u32 a3, %1, 24;\n\tadd.u32 a4, %1, 32;\n\tadd.u32 a5, %1, 40;\n\t"
+      "add.u32 a6, %1, 48;\n\tadd.u32 a7, %1, 56;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%5], [a4], %2, %3, u;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%5], [a5], b1, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%5], [a6], b2, %3, t;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%5], [a7], b3, %3, t;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(d_lo), "r"(accumulate | (uint32_t)(d_lo == d_tmem))
       : "memory");
 }
 // MN-major operand, 128-byte swizzle: atoms of [8 k][64 mn], 1024 B apart along k, half_bytes apart along mn
@@ -124,11 +146,29 @@ __device__ __forceinline__ void tma_box(uint32_t dst, const void* map, int x, in
                ::"r"(dst), "l"(map), "r"(x), "r"(head), "r"(row), "r"(bar)
                : "memory");
 }
+// sets the bf16 values of v that are infinite or not a number to 0; whether there was one
+__device__ __forceinline__ bool at_drop_nonfinite(uint4& v) {
+  uint32_t* w = &v.x;
+  bool any = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if ((w[i] & 0x7f80u) == 0x7f80u) { w[i] &= 0xffff0000u; any = true; }
+    if ((w[i] & 0x7f800000u) == 0x7f800000u) { w[i] &= 0xffffu; any = true; }
+  }
+  return any;
+}
+// Where S (and P over it) of tile i, M tile m lives: two buffers per M tile, or four if there is one M tile only.
+__device__ __forceinline__ int s_buf(int i, int m, int n_m) { return n_m == 1 ? i & 3 : 2 * m + (i & 1); }
+__device__ __forceinline__ uint32_t s_phase(int i, int n_m) { return (i >> (n_m == 1 ? 2 : 1)) & 1; }
+__device__ __forceinline__ uint32_t s_cols(int i, int m, int n_m) {
+  const int b = s_buf(i, m, n_m);
+  return (b >> 1) * 256 + (b & 1) * kAtKeys;
+}
 __device__ __forceinline__ void bar_loaders() { asm volatile("bar.sync 1, %0;" ::"n"(kAtLoadThreads) : "memory"); }
 
 template <int D>
 __global__ void __launch_bounds__(kAtThreads, 1)
-k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
+k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
   using P = AtShape<D>;
   constexpr int NH = P::NH, ST = P::kStages;
   extern __shared__ unsigned char at_smem_raw[];
@@ -139,8 +179,8 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
   uint64_t* k_empty = k_full + ST;                // [ST] MMA commit: S of that tile is done
   uint64_t* v_full = k_empty + ST;                // [ST] the value tile has landed
   uint64_t* v_empty = v_full + ST;                // [ST] MMA commit: P V of that tile is done
-  uint64_t* s_full = v_empty + ST;                // [M tile][2] MMA commit: the scores are in tensor memory
-  uint64_t* p_full = s_full + 4;                  // [M tile][2] softmax warps (4): P is in tensor memory, O is rescaled
+  uint64_t* s_full = v_empty + ST;                // [4] MMA commit: the scores are in tensor memory
+  uint64_t* p_full = s_full + 4;                  // [4] softmax warps (4): P is in tensor memory, O is rescaled
   uint64_t* pv_done = p_full + 4;                 // [M tile] MMA commit: O holds the tiles so far
   uint64_t* q_full = pv_done + 2;                 // [1] softmax warps (8): the queries are in shared memory
   uint64_t* all_done = q_full + 1;                // [1] MMA commit: every MMA of the CTA is complete
@@ -148,12 +188,12 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int32_t* status_sink = reinterpret_cast<int32_t*>(tmem_slot + 2);      // [2] stands in for a null status pointer
   static_assert((4 * ST + 12) * 8 + 16 <= 512, "barriers must fit");
-  __shared__ int s_comp[TEAM_MAX_BLOCK], s_list[TEAM_MAX_BLOCK], s_cnt[2];
-  __shared__ float s_m[kAtPairs], s_l[kAtPairs];
+  __shared__ int s_row[kAtPairs + 1], s_off[kAtPairs], s_cnt[kAtThreads / 32], s_nonfinite;
+  __shared__ float s_m[kAtPairs], s_l[kAtPairs], s_f[kAttnMaxSplits][kAtPairs];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m_tile = blockIdx.x, run = blockIdx.y / a.Hkv, g = blockIdx.y - run * a.Hkv, z = blockIdx.z;
-  const int L = a.L, rep = a.Hq / a.Hkv;
-  const int row0 = run * L, s = run / a.B;
+  const int s = blockIdx.x / a.Hkv, g = blockIdx.x - s * a.Hkv, z = blockIdx.z;
+  const int L = a.L, rep = a.Hq / a.Hkv, n_rows = a.B * L, row0 = s * n_rows;
+  const int pair0 = blockIdx.y * cta_pairs, first_row = pair0 / rep;      // first of the sequence's computed rows
   int32_t* status = a.status != nullptr ? a.status : status_sink;
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) {
@@ -171,48 +211,72 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
     mbar_init(smem_u32(q_full), kAtSoftmaxWarps);
     mbar_init(smem_u32(all_done), 1);
     *abort_flag = 0;
+    s_nonfinite = 0;
     status_sink[0] = status_sink[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // everything from here on reads what preceding kernels may have written; the kernel behind this one may be scheduled
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // ---- the run's rows: layout contract, which of them are computed ----
-  const int plen = min(max(a.prefix_len[s], 0), a.P);
-  bool comp = false;
-  unsigned bal = 0u;
-  if (tid < TEAM_MAX_BLOCK) {                               // two warps cover the block's positions
-    if (tid < L) {
-      const int t = row0 + tid;
-      const bool ok = a.pos[t] == tid && a.group[t] == s && a.branch[t] == run % a.B;
-      if (!ok && a.status != nullptr) set_status(a.status, TEAM_ERR_STATE, 40);
-      comp = attn_computed(a.tok_state[t], a.flags);
-      s_comp[tid] = comp ? 1 : 0;
-    }
-    bal = __ballot_sync(0xffffffffu, comp);
-    if (lane == 0) s_cnt[warp] = __popc(bal);
-  }
-  __syncthreads();
-  if (comp) s_list[(warp ? s_cnt[0] : 0) + __popc(bal & ((1u << lane) - 1u))] = tid;
-  const int n_pairs = (s_cnt[0] + s_cnt[1]) * rep;
-  const int pair0 = m_tile * kAtPairs, my_pairs = min(kAtPairs, n_pairs - pair0);
-  if (my_pairs <= 0) return;                                // the whole cluster shares (m_tile, run): it leaves together
-  const int n_m = my_pairs > 128 ? 2 : 1;                   // M tiles in use
-  const int n_keys = plen + L;
-  const int tiles_total = (n_keys + kAtKeys - 1) / kAtKeys;
-  const int tps = (tiles_total + n_splits - 1) / n_splits;
-  const int t_begin = min(z * tps, tiles_total), t_end = min(t_begin + tps, tiles_total);
-  const int n_tiles = t_end - t_begin;
   if (warp == kAtSoftmaxWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"((uint32_t)kAtTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // everything from here on reads what preceding kernels may have written; the kernel behind this one may be scheduled
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // ---- the sequence's rows: layout contract, which of them are computed, this CTA's ----
+  const int plen = min(max(a.prefix_len[s], 0), a.P);
+  int n_comp = 0;
+  for (int base = 0; base < n_rows; base += kAtThreads) {
+    const int r = base + tid, t = row0 + r;
+    bool comp = false;
+    if (r < n_rows) {
+      const int b = r / L;
+      const bool ok = a.pos[t] == r - b * L && a.group[t] == s && a.branch[t] == b;
+      if (!ok && a.status != nullptr) set_status(a.status, TEAM_ERR_STATE, 40);
+      comp = attn_computed(a.tok_state[t], a.flags);
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, comp);
+    if (base > 0) __syncthreads();                          // the counts of the pass before have been read
+    if (lane == 0) s_cnt[warp] = __popc(bal);
+    __syncthreads();
+    int at = n_comp + __popc(bal & ((1u << lane) - 1u)) - first_row;
+#pragma unroll
+    for (int w = 0; w < kAtThreads / 32; ++w) {
+      const int c = s_cnt[w];
+      if (w < warp) at += c;
+      n_comp += c;
+    }
+    if (comp && at >= 0 && at <= kAtPairs) s_row[at] = r;
+  }
+  const int my_pairs = min(cta_pairs, n_comp * rep - pair0);
+  if (my_pairs <= 0) {                                      // the whole cluster has the same pairs: it leaves together
+    if (warp == kAtSoftmaxWarps)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"((uint32_t)kAtTmemCols) : "memory");
+    return;
+  }
+  const int n_m = my_pairs > 128 ? 2 : 1;                   // M tiles in use
+  __syncthreads();                                          // s_row is complete
+  const int b0 = s_row[0] / L, b1 = s_row[(pair0 + my_pairs - 1) / rep - first_row] / L;      // branches of the pairs
+  int my_branch = b0;
+  if (tid < kAtPairs) {
+    int off = -1;
+    if (tid < my_pairs) {
+      const int cr = (pair0 + tid) / rep, r = s_row[cr - first_row];
+      off = (row0 + r) * a.Hq + g * rep + (pair0 + tid - cr * rep);
+      my_branch = r / L;
+    }
+    s_off[tid] = off;
+  }
+  const int n_keys = plen + (b1 - b0 + 1) * L;
+  const int tiles_total = (n_keys + kAtKeys - 1) / kAtKeys;
+  const int tps = (tiles_total + n_splits - 1) / n_splits;
+  const int t_begin = min(z * tps, tiles_total), t_end = min(t_begin + tps, tiles_total);
+  const int n_tiles = t_end - t_begin;
   tc_fence_before();
-  __syncthreads();                                          // s_list and the tensor memory's address
+  __syncthreads();                                          // s_off and the tensor memory's address
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
   if (warp > kAtSoftmaxWarps) {
     // ------------------------------ loaders ------------------------------
@@ -258,17 +322,20 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
             if (key < plen) {
               o = (((size_t)s * a.P + key) * a.Hkv + g) * D;
             } else {
-              const int p = key - plen;
-              if (s_comp[p]) {
-                o = ((size_t)(row0 + p) * a.Hkv + g) * D;
+              const int r = b0 * L + key - plen;             // row of the sequence
+              if (attn_computed(a.tok_state[row0 + r], a.flags)) {
+                o = ((size_t)(row0 + r) * a.Hkv + g) * D;
                 ks = a.k_new; vs = a.v_new;
               } else {
-                o = (((size_t)s * L + p) * a.Hkv + g) * D;
+                o = (((size_t)s * L + r % L) * a.Hkv + g) * D;
                 ks = a.k_block; vs = a.v_block;
               }
             }
             kk[q] = *reinterpret_cast<const uint4*>(ks + o + c * 8);
             vv[q] = *reinterpret_cast<const uint4*>(vs + o + c * 8);
+            // the tile is multiplied with P = 0 for the pairs of other branches: a value of the block that is not finite
+            // must not reach them.  It counts as 0 here and is added to its own branch's outputs at the end.
+            if (b1 > b0 && key >= plen && at_drop_nonfinite(vv[q])) s_nonfinite = 1;
           }
         }
 #pragma unroll
@@ -293,68 +360,60 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
   } else if (warp == kAtSoftmaxWarps) {
     // ------------------------------ MMA issuer ------------------------------
     const uint32_t idesc_s = make_idesc_bf16(kAtKeys), idesc_o = make_idesc_bf16(D) | (1u << 16);      // V: MN-major
+    const int tiles = (int)warp_uniform(n_tiles), n_mt = (int)warp_uniform(n_m);
     bool ok = mbar_wait_warp(smem_u32(q_full), 0, abort_flag, status, 50);
-    auto issue_s = [&](int i) {
-      const int st = i % ST, b = i & 1;
-      if (!(ok = mbar_wait_warp(smem_u32(k_full + st), (i / ST) & 1, abort_flag, status, 53))) return;
-      tc_fence_after();
-      const uint32_t kst = sm0 + P::kOffK + st * NH * P::kHalf;
-      for (int m = 0; m < n_m; ++m) {
-        // the columns were P of tile i - 2: its product was issued before
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-          const uint64_t da = make_kmajor_sw128_desc(sm0 + (m * NH + h) * P::kQTile), db = make_kmajor_sw128_desc(kst + h * P::kHalf);
-#pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4) tc_mma(tmem_base + m * 256 + b * kAtKeys, da + 2 * k4, db + 2 * k4, idesc_s, (h | k4) != 0);
-        }
-        tc_commit(smem_u32(s_full + m * 2 + b));
-      }
-      tc_commit(smem_u32(k_empty + st));
-    };
-    if (ok && n_tiles > 0) issue_s(0);
-    for (int i = 0; i < n_tiles && ok; ++i) {
-      const int st = i % ST, b = i & 1;
-      if (i + 1 < n_tiles) {
-        issue_s(i + 1);
-        if (!ok) break;
-      }
-      if (!(ok = mbar_wait_warp(smem_u32(v_full + st), (i / ST) & 1, abort_flag, status, 56))) break;
-      const uint64_t db = make_mnmajor_sw128_desc(sm0 + P::kOffV + st * NH * P::kHalf, P::kHalf);
-      for (int m = 0; m < n_m && ok; ++m) {
-        if (!(ok = mbar_wait_warp(smem_u32(p_full + m * 2 + b), (i >> 1) & 1, abort_flag, status, 55))) break;
+    // S of tile i, M tile m: the columns were P of an earlier tile whose product has been issued before
+    auto issue_s = [&](int i, int m) {
+      const int st = i % ST;
+      if (m == 0) {
+        if (!(ok = mbar_wait_warp(smem_u32(k_full + st), (i / ST) & 1, abort_flag, status, 53))) return;
         tc_fence_after();
-        const uint32_t tm = tmem_base + m * 256;
+      }
+      const uint32_t kst = sm0 + P::kOffK + st * NH * P::kHalf;
 #pragma unroll
-        for (int h = 0; h < 2; ++h)                          // P hi, then P lo: 32 columns of 2 keys each
-#pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4)                     // 16 keys: 8 columns of P, 2048 B of V
-            tc_mma_ts(tm + 128, tm + b * kAtKeys + h * 32 + k4 * 8, db + 128 * k4, idesc_o, (i | h | k4) != 0);
+      for (int h = 0; h < NH; ++h)
+        tc_mma_k64(tmem_base + s_cols(i, m, n_mt), make_kmajor_sw128_desc(sm0 + (m * NH + h) * P::kQTile),
+                   make_kmajor_sw128_desc(kst + h * P::kHalf), idesc_s, h != 0);
+      tc_commit(smem_u32(s_full + s_buf(i, m, n_mt)));
+      if (m == n_mt - 1) tc_commit(smem_u32(k_empty + st));
+    };
+    // one M tile: scores three tiles ahead; two: one tile ahead, and the M tiles interleaved, so that the tensor core has
+    // work queued while this warp waits for P
+    const int ahead = n_mt == 1 ? 3 : 1;
+    for (int i = 0; i < ahead && i < tiles && ok; ++i)
+      for (int m = 0; m < n_mt && ok; ++m) issue_s(i, m);
+    for (int i = 0; i < tiles && ok; ++i) {
+      const int st = i % ST;
+      const uint64_t db = make_mnmajor_sw128_desc(sm0 + P::kOffV + st * NH * P::kHalf, P::kHalf);
+      for (int m = 0; m < n_mt && ok; ++m) {
+        if (i + ahead < tiles) {
+          issue_s(i + ahead, m);
+          if (!ok) break;
+        }
+        if (m == 0 && !(ok = mbar_wait_warp(smem_u32(v_full + st), (i / ST) & 1, abort_flag, status, 56))) break;
+        if (!(ok = mbar_wait_warp(smem_u32(p_full + s_buf(i, m, n_mt)), s_phase(i, n_mt), abort_flag, status, 55))) break;
+        tc_fence_after();
+        tc_mma_ts_hilo(tmem_base + m * 256 + 128, tmem_base + m * 256 + 128 + P::kOLo, tmem_base + s_cols(i, m, n_mt), db, idesc_o, i != 0);
         tc_commit(smem_u32(pv_done + m));
       }
       if (ok) tc_commit(smem_u32(v_empty + st));
     }
-    if (ok && n_tiles > 0) tc_commit(smem_u32(all_done));
+    if (ok && tiles > 0) tc_commit(smem_u32(all_done));
   } else {
     // ---- the queries of this CTA's pairs: A operand of S = Q K^T, per M tile NH halves of [128 rows][128 B], swizzled ----
     {
-      constexpr int PIECES = D / 8, PER = 8;                // 16-byte pieces per row; loads in flight per thread
-      for (int i0 = tid; i0 < n_m * 128 * PIECES; i0 += kAtSoftmaxWarps * 32 * PER) {
-        uint4 v[PER];
+      constexpr int PIECES = D / 8, PER = 128 * PIECES / (kAtSoftmaxWarps * 32);      // 16-byte pieces per row, per thread and M tile
+      const int c = tid % PIECES;
+      uint4 v[2 * PER];
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          const int i = i0 + q * kAtSoftmaxWarps * 32, pr = i / PIECES, c = i % PIECES;
-          v[q] = make_uint4(0u, 0u, 0u, 0u);
-          if (pr < my_pairs) {
-            const int gp = pair0 + pr, cr = gp / rep, j = gp - cr * rep;
-            v[q] = *reinterpret_cast<const uint4*>(a.q + ((size_t)(row0 + s_list[cr]) * a.Hq + g * rep + j) * D + c * 8);
-          }
-        }
+      for (int q = 0; q < 2 * PER; ++q) {
+        const int off = s_off[tid / PIECES + q * (kAtSoftmaxWarps * 32 / PIECES)];      // -1 past the CTA's pairs
+        v[q] = off >= 0 ? *reinterpret_cast<const uint4*>(a.q + (size_t)off * D + c * 8) : make_uint4(0u, 0u, 0u, 0u);
+      }
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          const int i = i0 + q * kAtSoftmaxWarps * 32, pr = i / PIECES, c = i % PIECES;
-          if (pr < n_m * 128)
-            *reinterpret_cast<uint4*>(smem + ((pr >> 7) * NH + (c >> 3)) * P::kQTile + sw128(pr & 127, c & 7)) = v[q];
-        }
+      for (int q = 0; q < 2 * PER; ++q) {
+        const int r = tid / PIECES + q * (kAtSoftmaxWarps * 32 / PIECES);
+        *reinterpret_cast<uint4*>(smem + ((r >> 7) * NH + (c >> 3)) * P::kQTile + sw128(r & 127, c & 7)) = v[q];
       }
       fence_async_smem();                                   // generic-proxy writes, read by the tensor core
       __syncwarp();
@@ -362,27 +421,28 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
     }
     // ------------------------------ softmax ------------------------------
     const int m = warp >> 2;                                 // M tile
-    const uint32_t tm = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + m * 256;      // this warp's quarter of the lanes
+    const uint32_t tm_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16), tm = tm_lane + m * 256;      // this warp's quarter of the lanes
+    const int own_lo = plen + (my_branch - b0) * L;          // first key of the pair's own block
     const int pr = tid;                                      // pair of the CTA = lane of tensor memory + 128 * M tile
     const float sl2 = rsqrtf((float)D) * 1.4426950408889634f;      // scores in base 2
     float m_used = kNegInf, l_run = 0.f;                     // running maximum in use (base 2) and row sum
     bool ok = true;
     for (int i = 0; i < n_tiles && ok && m < n_m; ++i) {
-      const int b = i & 1;
-      if (!(ok = mbar_wait_warp(smem_u32(s_full + m * 2 + b), (i >> 1) & 1, abort_flag, status, 57))) break;
+      const int b = s_buf(i, m, n_m);
+      if (!(ok = mbar_wait_warp(smem_u32(s_full + b), s_phase(i, n_m), abort_flag, status, 57))) break;
       tc_fence_after();
-      const uint32_t tm_s = tm + b * kAtKeys;
+      const uint32_t tm_s = tm_lane + s_cols(i, m, n_m);
       uint32_t sc[kAtKeys];
       tmem_ld32(tm_s, sc);
       tmem_ld32(tm_s + 32, sc + 32);
       tmem_wait_ld(sc);
       tmem_wait_ld(sc + 32);
-      // mask the keys past the end (last tile only), the tile's maximum
+      // mask the other branches' keys (tiles that reach into the block only), the tile's maximum
       const int key0 = (t_begin + i) * kAtKeys;
-      if (key0 + kAtKeys > n_keys) {
+      if (key0 + kAtKeys > plen) {
 #pragma unroll
         for (int e = 0; e < kAtKeys; ++e)
-          if (key0 + e >= n_keys) sc[e] = __float_as_uint(kNegInf);
+          if (key0 + e >= plen && (unsigned)(key0 + e - own_lo) >= (unsigned)L) sc[e] = __float_as_uint(kNegInf);
       }
       float mx4[4];
 #pragma unroll
@@ -391,7 +451,7 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
       for (int e = 4; e < kAtKeys; ++e) mx4[e & 3] = fmaxf(mx4[e & 3], __uint_as_float(sc[e]));
       const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;      // sl2 > 0: the maximum of the scaled scores
       // the maximum in use moves only when it has to: P stays below 2^8, far inside fp32 and the bf16 pair
-      const bool move = mx > m_used + kAtRescale;            // always on the first tile (m_used = -inf)
+      const bool move = mx > m_used + kAtRescale;            // always on the first tile with a key of the pair (m_used = -inf)
       float corr = 1.f;
       if (move) {
         corr = at_ex2(m_used - mx);                          // 0 on the first tile
@@ -400,15 +460,16 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
       }
       // scale and shift in one operation, 2^x, the row sum, and P as bf16 pairs hi = rn(p), lo = rn(p - hi): two keys
       // per column, the 32 columns of hi in front of the 32 of lo
-      const float2 scale = make_float2(sl2, sl2), shift = make_float2(-m_used, -m_used), minus = make_float2(-1.f, -1.f);
-      float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      const float sh = m_used == kNegInf ? 0.f : -m_used;    // no key of the pair so far: every score is -inf
+      const float2 scale = make_float2(sl2, sl2), shift = make_float2(sh, sh), minus = make_float2(-1.f, -1.f);
+      float2 sum[4] = {};
       uint32_t lo[kAtKeys / 2];
 #pragma unroll
       for (int e = 0; e < kAtKeys / 2; ++e) {
         float2 p = at_fma2(make_float2(__uint_as_float(sc[2 * e]), __uint_as_float(sc[2 * e + 1])), scale, shift);
         p.x = at_ex2(p.x);
         p.y = at_ex2(p.y);
-        sum[e & 1] = at_add2(sum[e & 1], p);
+        sum[e & 3] = at_add2(sum[e & 3], p);
         const __nv_bfloat162 h2 = __floats2bfloat162_rn(p.x, p.y);
         const uint32_t h = *reinterpret_cast<const uint32_t*>(&h2);
         const float2 rest = at_fma2(make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), minus, p);
@@ -416,7 +477,7 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
         sc[e] = h;
         lo[e] = *reinterpret_cast<const uint32_t*>(&l2);
       }
-      sum[0] = at_add2(sum[0], sum[1]);
+      sum[0] = at_add2(at_add2(sum[0], sum[1]), at_add2(sum[2], sum[3]));
       l_run += sum[0].x + sum[0].y;
       tmem_st32(tm_s, sc);
       tmem_st32(tm_s + 32, lo);
@@ -426,7 +487,7 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
         if (__any_sync(0xffffffffu, move)) {
           tc_fence_after();
 #pragma unroll 1
-          for (int c0 = 0; c0 < D; c0 += 32) {
+          for (int c0 = 0; c0 < 128; c0 += 32) {            // both accumulators with head size 64
             uint32_t r[32];
             tmem_ld32(tm + 128 + c0, r);
             tmem_wait_ld(r);
@@ -439,7 +500,7 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(p_full + m * 2 + b));
+      if (lane == 0) mbar_arrive(smem_u32(p_full + b));
     }
     // ---- the CTA's partial result: (maximum, sum, unnormalised output) of its pairs into shared memory, over the
     //      operands: every MMA of both M tiles has to be complete ----
@@ -456,6 +517,13 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
         if (have) {                                          // warp-uniform
           tmem_ld32(tm + 128 + c0, r);
           tmem_wait_ld(r);
+          if (P::kOLo > 0) {
+            uint32_t lo[32];
+            tmem_ld32(tm + 128 + P::kOLo + c0, lo);
+            tmem_wait_ld(lo);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(lo[e]));
+          }
         } else {
 #pragma unroll
           for (int e = 0; e < 32; ++e) r[e] = 0u;
@@ -473,42 +541,72 @@ k_block_attention_tc(AttnArgs a, int n_splits, const __grid_constant__ CUtensorM
   cg::cluster_group cluster = cg::this_cluster();
   cluster.sync();
   if (!*abort_flag) {
-    // rank z merges its share of the rows of all partials (distributed shared memory) and writes them
+    // rank z merges its share of the pairs of all partials (distributed shared memory) and writes them: first each
+    // split's weight per pair, then the outputs
     float* s_o = reinterpret_cast<float*>(smem);
-    constexpr int TPR = D / 4;                              // threads per row (one float4 each)
-    const int R = (my_pairs + n_splits - 1) / n_splits, r1 = min(my_pairs, (z + 1) * R);
-    for (int i = z * R * TPR + tid; i < r1 * TPR; i += kAtThreads) {
-      const int pr = i / TPR, c4 = i % TPR, gp = pair0 + pr;
-      float mk[kAttnMaxSplits], lk[kAttnMaxSplits], mx = kNegInf;
+    constexpr int TPR = D / 4;                              // threads per pair (one float4 each)
+    const int R = (my_pairs + n_splits - 1) / n_splits, r0 = z * R, r1 = min(my_pairs, r0 + R);
+    for (int pr = r0 + tid; pr < r1; pr += kAtThreads) {
+      float mk[kAttnMaxSplits], lk[kAttnMaxSplits], mx = kNegInf, den = 0.f;
+#pragma unroll
+      for (int k = 0; k < kAttnMaxSplits; ++k) {
+        mk[k] = k < n_splits ? *cluster.map_shared_rank(&s_m[pr], k) : kNegInf;
+        lk[k] = k < n_splits ? *cluster.map_shared_rank(&s_l[pr], k) : 0.f;
+        mx = fmaxf(mx, mk[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < kAttnMaxSplits; ++k) {
+        mk[k] = at_ex2(mk[k] - mx);                          // 0 for a split without a key of the pair (its maximum is -inf)
+        den = fmaf(mk[k], lk[k], den);
+      }
+      const float inv = 1.f / den;
+#pragma unroll
+      for (int k = 0; k < kAttnMaxSplits; ++k) s_f[k][pr] = mk[k] * inv;
+    }
+    const bool nonfinite = __any_sync(0xffffffffu, lane < n_splits && *cluster.map_shared_rank(&s_nonfinite, min(lane, n_splits - 1)) != 0);
+    __syncthreads();
+    for (int i = r0 * TPR + tid; i < r1 * TPR; i += kAtThreads) {
+      const int pr = i / TPR, c4 = i % TPR;
       float4 v[kAttnMaxSplits];
 #pragma unroll
       for (int k = 0; k < kAttnMaxSplits; ++k) {
-        mk[k] = kNegInf;
-        lk[k] = 0.f;
         v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k < n_splits) {
-          mk[k] = *cluster.map_shared_rank(&s_m[pr], k);
-          lk[k] = *cluster.map_shared_rank(&s_l[pr], k);
-          v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_o + (size_t)pr * P::kOStride + c4 * 4, k));
-        }
-        mx = fmaxf(mx, mk[k]);
+        if (k < n_splits) v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_o + (size_t)pr * P::kOStride + c4 * 4, k));
       }
-      float den = 0.f;
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int k = 0; k < kAttnMaxSplits; ++k) {
-        if (k >= n_splits) break;
-        const float f = at_ex2(mk[k] - mx);                  // 0 for a split without keys (its maximum is -inf)
-        den = fmaf(f, lk[k], den);
+        const float f = s_f[k][pr];
         acc.x = fmaf(f, v[k].x, acc.x); acc.y = fmaf(f, v[k].y, acc.y); acc.z = fmaf(f, v[k].z, acc.z); acc.w = fmaf(f, v[k].w, acc.w);
       }
-      const int cr = gp / rep, j = gp - cr * rep;
-      float* dst = a.out + ((size_t)(row0 + s_list[cr]) * a.Hq + g * rep + j) * D + c4 * 4;
-      const float inv = 1.f / den;
-      *reinterpret_cast<float4*>(dst) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+      if (nonfinite) {
+        const int t = s_off[pr] / a.Hq;                     // the pair's row; its block begins at t - pos
+        const int t_block = t - (t - row0) % L;
+        for (int p = 0; p < L; ++p) {
+          const bool fresh = attn_computed(a.tok_state[t_block + p], a.flags);
+          const __nv_bfloat16* v4 = (fresh ? a.v_new + ((size_t)(t_block + p) * a.Hkv + g) * D : a.v_block + (((size_t)s * L + p) * a.Hkv + g) * D) + c4 * 4;
+          const float x0 = __bfloat162float(v4[0]), x1 = __bfloat162float(v4[1]), x2 = __bfloat162float(v4[2]), x3 = __bfloat162float(v4[3]);
+          if (!isfinite(x0)) acc.x += x0;
+          if (!isfinite(x1)) acc.y += x1;
+          if (!isfinite(x2)) acc.z += x2;
+          if (!isfinite(x3)) acc.w += x3;
+        }
+      }
+      *reinterpret_cast<float4*>(a.out + (size_t)s_off[pr] * D + c4 * 4) = acc;
     }
   }
   cluster.sync();                                          // peers may still be reading this CTA's partial
+  if (a.insert) {
+    // this cluster holds all pairs of (sequence, key / value head), so nobody reads the in-block cache any more: the
+    // delayed insertion (see k_attn_insert), positions spread over the cluster
+    for (int i = tid; i < L * (D / 8); i += kAtThreads) {
+      const int p = i / (D / 8), c = i % (D / 8), st = a.tok_state[row0 + p];
+      if (p % n_splits != z || !attn_computed(st, a.flags) || st == TEAM_TOK_MASKED) continue;
+      const size_t src = ((size_t)(row0 + p) * a.Hkv + g) * D + c * 8, dst = (((size_t)s * L + p) * a.Hkv + g) * D + c * 8;
+      *reinterpret_cast<uint4*>(a.k_block + dst) = *reinterpret_cast<const uint4*>(a.k_new + src);
+      *reinterpret_cast<uint4*>(a.v_block + dst) = *reinterpret_cast<const uint4*>(a.v_new + src);
+    }
+  }
   if (warp == kAtSoftmaxWarps) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)kAtTmemCols) : "memory");
@@ -577,15 +675,29 @@ static cudaError_t attn_setup(const AttnSetup** out) {
 }
 
 template <int D>
-static cudaError_t launch(const AttnArgs& a, const AttnSetup& st, cudaStream_t s) {
-  // M tiles by the largest number of pairs a run can have; the keys of each are split over a cluster, as far as all
-  // clusters run at once and every split keeps two tiles of the longest prefix
-  const int m_tiles = (a.L * (a.Hq / a.Hkv) + kAtPairs - 1) / kAtPairs;
-  const long long units = (long long)m_tiles * a.S * a.B * a.Hkv;
+static cudaError_t launch(AttnArgs a, const AttnSetup& st, cudaStream_t s, bool* inserted) {
+  // One or two M tiles per CTA and how many CTAs split the keys: whatever should end first, by what was measured
+  // (clock cycles): a key tile takes 1500 for one M tile and 2100 for two, everything around the tiles 10000 per wave of
+  // clusters.  A decoded block has a quarter of its rows cached on average when delayed caching is on.
+  const long long pairs = (long long)a.B * a.L * (a.Hq / a.Hkv), expected = (a.flags & TEAM_F_DCD) ? (3 * pairs + 3) / 4 : pairs;
   const int tiles_max = (a.P + a.L + kAtKeys - 1) / kAtKeys;
-  int n_splits = 1;
-  for (int n = 2; n <= kAttnMaxSplits; ++n)
-    if (units <= st.clusters[D / 128][n] && tiles_max >= 2 * n) n_splits = n;
+  int cta_pairs = 128, n_splits = 1;
+  long long best = -1;
+  for (int m = 1; m <= 2; ++m) {
+    const long long units = (expected + 128 * m - 1) / (128 * m) * a.S * a.Hkv;
+    for (int n = 1; n <= kAttnMaxSplits && (n == 1 || tiles_max >= 2 * n); ++n) {
+      const int at_once = st.clusters[D / 128][n];
+      if (at_once < 1) continue;
+      const long long cost = ((units + at_once - 1) / at_once) * ((tiles_max + n - 1) / n * (m == 1 ? 1500 : 2100) + 10000);
+      if (best < 0 || cost < best) {
+        best = cost;
+        cta_pairs = 128 * m;
+        n_splits = n;
+      }
+    }
+  }
+  const int m_tiles = (int)((pairs + cta_pairs - 1) / cta_pairs);
+  a.insert = *inserted = m_tiles == 1;      // the only cluster of its sequence and head also inserts: one launch fewer
   CUtensorMap kmap = {}, vmap = {};
   if (a.P >= kAtKeys) {                                     // else no tile lies in the prefix and the maps are not used
     const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)a.Hkv, (cuuint64_t)a.S * a.P};
@@ -600,15 +712,15 @@ static cudaError_t launch(const AttnArgs& a, const AttnSetup& st, cudaStream_t s
     }
   }
   cudaLaunchAttribute at[2];
-  const cudaLaunchConfig_t lc = attn_launch<D>(at, dim3(m_tiles, a.S * a.B * a.Hkv, n_splits), s);
-  return cudaLaunchKernelEx(&lc, k_block_attention_tc<D>, a, n_splits, kmap, vmap);
+  const cudaLaunchConfig_t lc = attn_launch<D>(at, dim3(a.S * a.Hkv, m_tiles, n_splits), s);      // clusters without a computed row come last
+  return cudaLaunchKernelEx(&lc, k_block_attention_tc<D>, a, cta_pairs, n_splits, kmap, vmap);
 }
 
-cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s) {
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s, bool* inserted) {
   const AttnSetup* st = nullptr;
   const cudaError_t e = attn_setup(&st);
   if (e != cudaSuccess) return e;
-  return a.d == 128 ? launch<128>(a, *st, s) : launch<64>(a, *st, s);
+  return a.d == 128 ? launch<128>(a, *st, s, inserted) : launch<64>(a, *st, s, inserted);
 }
 
 }  // namespace team

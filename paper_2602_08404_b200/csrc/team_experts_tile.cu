@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = warp_uniform(*tmem_slot);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // Everything above overlaps the preceding kernel; its outputs (plan, token tiles) are complete from here.
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -455,12 +455,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_grouped_gemm(TileArgs a) {
         const uint32_t base = smem_u32(stages + (size_t)s * kStageBytes);
         const uint64_t d0 = make_kmajor_sw128_desc(base), d1 = make_kmajor_sw128_desc(base + kTileBytes),
                        d2 = make_kmajor_sw128_desc(base + 2 * kTileBytes);
-#pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) tc_mma(acc, d0 + 2 * k4, d2 + 2 * k4, idesc0, (kb | k4) != 0);
+        tc_mma_k64(acc, d0, d2, idesc0, kb != 0);
         if (accs == 2) {
           const uint64_t da = wk.nt == 2 ? d1 : d0, db = wk.nt == 2 ? d2 : d1;
-#pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4) tc_mma(acc + kTileChunk, da + 2 * k4, db + 2 * k4, idesc1, (kb | k4) != 0);
+          tc_mma_k64(acc + kTileChunk, da, db, idesc1, kb != 0);
         }
         tc_commit(smem_u32(bar_empty + s));
       }

@@ -130,3 +130,45 @@ def test_block_attention_reports_a_broken_row_layout():
                                   kb, kb.clone(), out, status) == B.TEAM_OK
     torch.cuda.synchronize()
     assert status.cpu().tolist() == [B.TEAM_ERR_STATE, 40]
+
+
+@pytest.mark.parametrize("d,Hq,Hkv,S,Bn,L,P", [(128, 6, 2, 1, 4, 11, 200), (64, 5, 1, 2, 3, 64, 64), (128, 1, 1, 1, 9, 33, 63), (64, 48, 2, 1, 2, 16, 0),
+                                               (128, 16, 1, 1, 1, 64, 511), (64, 7, 7, 3, 5, 3, 129), (128, 32, 4, 1, 4, 32, 700)],
+                         ids=lambda v: str(v))
+def test_pairs_of_several_branches_share_tiles(d, Hq, Hkv, S, Bn, L, P):
+    """Branches packed into M tiles that straddle them, block sizes that no key tile divides, pair counts around 128 and
+    256, prefixes around a key tile, arbitrary token states (cached in one branch and not in another)."""
+    rng = np.random.default_rng(d + Hq + L)
+    T = S * Bn * L
+    step = dict(tok_state=rng.integers(0, 3, T).astype(np.uint8), conf=np.zeros(T, np.float32), pos=np.tile(np.arange(L, dtype=np.int32), S * Bn),
+                group=np.repeat(np.arange(S, dtype=np.int32), Bn * L), branch=np.tile(np.repeat(np.arange(Bn, dtype=np.int32), L), S))
+    cfg = B.team_attn_config(Hq, Hkv, d, L, S, Bn, P, B.TEAM_F_DCD)
+    q, k, v = _bf16(rng, T, Hq, d), _bf16(rng, T, Hkv, d), _bf16(rng, T, Hkv, d)
+    kp, vp = _bf16(rng, S, max(P, 1), Hkv, d), _bf16(rng, S, max(P, 1), Hkv, d)
+    kb, vb = _bf16(rng, S, L, Hkv, d), _bf16(rng, S, L, Hkv, d)
+    plen = rng.integers(P // 2, P + 1, S).astype(np.int32)
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    ref, _, _ = A.block_attention(q, k, v, kp, vp, plen, kb, vb, step["tok_state"], step["pos"], step["group"], step["branch"], L, B.TEAM_F_DCD)
+    comp = A.computed_rows(step["tok_state"], B.TEAM_F_DCD)
+
+    def run(v_new):
+        out = torch.full((T, Hq, d), 3.0, device="cuda")
+        assert B.team_block_attention(cfg, B.state_to_device(step), _dev(q), _dev(k), _dev(v_new), _dev(kp), _dev(vp), torch.as_tensor(plen).cuda(),
+                                      _dev(kb), _dev(vb), out, status) == B.TEAM_OK
+        assert status.cpu().tolist() == [0, 0]
+        return out.cpu().numpy()
+
+    got = run(v)
+    assert np.abs(got[comp] - ref[comp]).max() <= TOL * np.abs(ref[comp]).max()
+    assert (got[~comp] == 3.0).all()
+    if Bn > 1:
+        # a value that is not finite stays inside its branch (and key / value head)
+        row = int(np.flatnonzero(comp & (step["branch"] == 1) & (step["group"] == 0))[0])
+        bad = v.copy()
+        bad[row, 0, 5] = np.inf
+        got_bad = run(bad)
+        hit = comp & (step["branch"] == 1) & (step["group"] == 0)
+        assert not np.isfinite(got_bad[hit][:, :Hq // Hkv, 5]).any()
+        finite = np.ones(got.shape, bool)
+        finite[np.ix_(hit, range(Hq // Hkv), [5])] = False
+        assert np.abs(got_bad[finite] - got[finite]).max() <= TOL * np.abs(ref[comp]).max()
