@@ -31,7 +31,7 @@ struct SelSmem {
   int32_t* hist;       // [kSelWarps][E+ns]
   int32_t* off;        // [E+ns+1]
   int32_t* key;        // [T] group*256 + branch
-  int32_t* pos;        // [T]
+  int2* walk;          // [T] (key * 2 + decoded, position): all that the walk over a run reads
   int32_t* warp_cnt;   // [kSelWarps + 1]
   int32_t* scan_tot;   // [3][kSelWarps] per-warp totals of the scan over experts: slots, work items, active experts
   int32_t* idx;        // [min(T*k, kIdxInSmemMax)]
@@ -55,7 +55,7 @@ __host__ __device__ inline size_t sel_smem_layout(Dims d, SelSmem* s, unsigned c
   size_t a_hist = take((size_t)kSelWarps * EN * 4);
   size_t a_off = take((size_t)(EN + 1) * 4);
   size_t a_key = take((size_t)d.T * 4);
-  size_t a_pos = take((size_t)d.T * 4);
+  size_t a_walk = take((size_t)d.T * 8);
   size_t a_wc = take((size_t)(kSelWarps + 1) * 4);
   size_t a_st = take((size_t)3 * kSelWarps * 4);
   size_t a_idx = take((size_t)n_idx * 4);
@@ -69,7 +69,7 @@ __host__ __device__ inline size_t sel_smem_layout(Dims d, SelSmem* s, unsigned c
     s->hist = reinterpret_cast<int32_t*>(base + a_hist);
     s->off = reinterpret_cast<int32_t*>(base + a_off);
     s->key = reinterpret_cast<int32_t*>(base + a_key);
-    s->pos = reinterpret_cast<int32_t*>(base + a_pos);
+    s->walk = reinterpret_cast<int2*>(base + a_walk);
     s->warp_cnt = reinterpret_cast<int32_t*>(base + a_wc);
     s->scan_tot = reinterpret_cast<int32_t*>(base + a_st);
     s->idx = n_idx ? reinterpret_cast<int32_t*>(base + a_idx) : nullptr;
@@ -135,8 +135,9 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
       b = min(max(b, 0), 255);
     }
     s.key[t] = g * 256 + b;
-    s.pos[t] = st.pos[t];
-    s.state[t] = st.tok_state[t];
+    const uint8_t state = st.tok_state[t];
+    s.walk[t] = make_int2((g * 256 + b) * 2 + (is_decoded(state) ? 1 : 0), st.pos[t]);
+    s.state[t] = state;
   }
   __syncthreads();
 
@@ -149,17 +150,34 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
     } else if (state == TEAM_TOK_NEW || !(p.flags & TEAM_F_LAC)) {
       c = TEAM_CLS_FIRST;
     } else {
-      const int key = s.key[t], mypos = s.pos[t];
+      const int key = s.walk[t].x >> 1, mypos = s.walk[t].y;
       const int lim = p.inclusive ? p.L_hot : p.L_hot - 1;   // |pos - j| <= lim
       bool hot = conf_r[t / kSelThreads] > p.tau_hot;
       if (p.prefix_decoded && mypos + 1 <= lim) hot = true;
-      for (int u = t - 1; !hot && u >= 0 && s.key[u] == key; --u) {
-        if (t - u > TEAM_MAX_BLOCK) { set_status(ws.status, TEAM_ERR_STATE, 2); break; }
-        if (is_decoded(s.state[u]) && abs(mypos - s.pos[u]) <= lim) hot = true;
-      }
-      for (int u = t + 1; !hot && u < T && s.key[u] == key; ++u) {
-        if (u - t > TEAM_MAX_BLOCK) { set_status(ws.status, TEAM_ERR_STATE, 2); break; }
-        if (is_decoded(s.state[u]) && abs(mypos - s.pos[u]) <= lim) hot = true;
+      // the row's own run, first downwards, then upwards, four rows per step (their loads overlap: one by one a block
+      // of 32 took 9600 clock cycles)
+#pragma unroll 1
+      for (int dir = -1; dir <= 1 && !hot; dir += 2) {
+        bool inside = true;
+#pragma unroll 1
+        for (int o = 1; inside && !hot; o += 4) {           // offsets 1-4, ..., 61-64, then the check
+          int2 w[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int u = t + dir * (o + q);
+            w[q] = s.walk[min(max(u, 0), T - 1)];
+            if (u < 0 || u >= T) w[q].x = -1;
+          }
+          if (o > TEAM_MAX_BLOCK) {                         // further away than a block is long
+            if ((w[0].x >> 1) == key) set_status(ws.status, TEAM_ERR_STATE, 2);
+            break;
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            inside = inside && (w[q].x >> 1) == key;
+            if (inside && (w[q].x & 1) && abs(mypos - w[q].y) <= lim) hot = true;
+          }
+        }
       }
       c = hot ? TEAM_CLS_FIRST : TEAM_CLS_COLD;
     }
@@ -247,7 +265,7 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
         for (int i = 0; i < kMaxPerLane; ++i)
           if (!((s.mask[g * n_words32 + i] >> lane) & 1u)) v[i] = kNegInf;
       }
-      TopkResult tr = warp_topk(v, k, lane, (E + 31) / 32);
+      TopkResult tr = warp_topk(v, k, lane, E);
       const float w = routing_weight(tr, k, lane, row_max, denom, p.norm_topk);
       if (lane < k) {
         if (s.idx) s.idx[t * k + lane] = tr.idx;

@@ -96,54 +96,58 @@ __device__ __forceinline__ int warp_topk_picks(uint32_t (&key)[kMaxPerLane], int
   return n;
 }
 
-// v[i] is the logit of expert i*32+lane, or -inf if that expert is not a candidate
-// (beyond E, or outside the allowed set); only the first ne = ceil(E / 32) entries are looked at.
-// Lane j < k receives the j-th choice.
-__device__ __forceinline__ TopkResult warp_topk(const float (&v)[kMaxPerLane], int k, int lane, int ne = kMaxPerLane) {
+// The same selection where many rows are routed at once: v[i] is the logit of expert i*32+lane, or -inf if that expert
+// is not a candidate (beyond E, or outside the allowed set); only the first NE entries are looked at.  Lane j < k
+// receives the j-th choice.
+//
+// One loop, not unrolled: with tens of warps per SM running it once, instruction issue and instruction fetches bound it,
+// not a pick's latency (sorted lists, with the picks moved to their lanes afterwards, took 17400 clock
+// cycles for 32 rows on one SM; calls of 128 rows 157 -> 142 us with this loop and the walk of the classification).  A pick is the lane's largest key, the warp's largest (one redux) and the
+// lowest expert id that holds it (another).
+template <int NE>
+__device__ __forceinline__ TopkResult warp_topk_loop(const float (&v)[kMaxPerLane], int k, int lane) {
   TopkResult r;
   r.idx = -1;
   r.val = kNegInf;
   r.top = kNegInf;
-  uint32_t key[kMaxPerLane];
-  int slot[kMaxPerLane];
+  r.margin = __builtin_huge_valf();
+  uint32_t key[NE];
 #pragma unroll
-  for (int i = 0; i < kMaxPerLane; ++i) {
-    key[i] = i < ne ? float_key(v[i]) : kKeyNegInf;
-    slot[i] = i;
-  }
-  sort_lane_keys(key, slot);
-  // the holder of a pick remembers it; afterwards pick j moves to lane j (one shuffle per pick, off the picks'
-  // dependent chain)
-  int order[kMaxPerLane];             // this lane's key i was picked as pick number order[i] (-1: not picked)
+  for (int i = 0; i < NE; ++i) key[i] = float_key(v[i]);
+  float last = kNegInf;
+#pragma unroll 1
+  for (int j = 0; j <= k; ++j) {
+    uint32_t best = key[0];
+    int slot = 0;
 #pragma unroll
-  for (int i = 0; i < kMaxPerLane; ++i) order[i] = -1;
-  const int n = warp_topk_picks(key, slot, k, lane,
-                                [&](int j, int e, uint32_t) {
-#pragma unroll
-                                  for (int i = 0; i < kMaxPerLane; ++i)
-                                    if (i == (e >> 5)) order[i] = j;
-                                },
-                                r.margin);
-  for (int j = 0; j < n; ++j) {
-    int slot = -1;
-    float mine_val = 0.f;
-#pragma unroll
-    for (int i = 0; i < kMaxPerLane; ++i)
-      if (order[i] == j) {
+    for (int i = 1; i < NE; ++i)
+      if (key[i] > best) {                                // equal keys: the lower expert id
+        best = key[i];
         slot = i;
-        mine_val = v[i];
       }
-    const uint32_t holder = __ballot_sync(0xffffffffu, slot >= 0);
-    const int src = __ffs(holder) - 1;
-    const int e = __shfl_sync(0xffffffffu, slot * 32 + lane, src);
-    const float val = __shfl_sync(0xffffffffu, mine_val, src);
+    const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+    if (top == kKeyNegInf) break;                         // no candidate left
+    const float val = key_float(top);
+    if (j == k) {
+      r.margin = last - val;
+      break;
+    }
+    const int e = (int)__reduce_min_sync(0xffffffffu, best == top ? (uint32_t)(slot * 32 + lane) : 0x7fffffffu);
+    const bool mine = (e & 31) == lane;
+#pragma unroll
+    for (int i = 0; i < NE; ++i)
+      if (mine && i == (e >> 5)) key[i] = kKeyNegInf;
     if (lane == j) {
       r.idx = e;
       r.val = val;
     }
     if (j == 0) r.top = val;
+    last = val;
   }
   return r;
+}
+__device__ __forceinline__ TopkResult warp_topk(const float (&v)[kMaxPerLane], int k, int lane, int n_experts) {
+  return n_experts <= 128 ? warp_topk_loop<4>(v, k, lane) : warp_topk_loop<kMaxPerLane>(v, k, lane);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
