@@ -287,7 +287,7 @@ int team_residual_add(team_ctx *ctx, void *x, const float *y, int32_t n_rows, vo
  * clears it).  detail_out (optional, host) receives a kernel-specific code. */
 int team_read_status(team_ctx *ctx, void *stream, int32_t *detail_out);
 
-/* Number of kernels the last compute call on this context launched. */
+/* Number of kernels the last compute call on this context launched (without the copies of team_moe_forward_host). */
 int team_last_launch_count(const team_ctx *ctx);
 
 /* Average device time (ms) of the expert kernel over the launches made since

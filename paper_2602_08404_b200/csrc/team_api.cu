@@ -495,9 +495,19 @@ int team_moe_forward_host(team_ctx* ctx, const void* x_host, const team_step_sta
   memcpy(hp + o_pos, st_host->pos, T * 4);
   memcpy(hp + o_grp, st_host->group, T * 4);
   memcpy(hp + o_br, st_host->branch, T * 4);
-  // one copy in: with few rows the block is small and a single transfer beats six
-  const size_t in_bytes = ctx->hs_in_bytes;
+  // few rows: the copies are kernels (team_hostio.cu), which move what the call has; else one transfer of the whole block
+  const size_t in_bytes = ctx->hs_in_bytes, y_bytes = T * H * 4;
   unsigned char* dp = ctx->hs_dev;
+  team::HostIn in;
+  in.src = reinterpret_cast<const uint4*>(hp);
+  in.dst = reinterpret_cast<uint4*>(dp);
+  const size_t part_at[team::HostIn::kParts] = {o_x, o_ts, o_conf, o_pos, o_grp, o_br};
+  const size_t part_bytes[team::HostIn::kParts] = {T * H * elt, T, T * 4, T * 4, T * 4, T * 4};
+  for (int i = 0, n = 0; i < team::HostIn::kParts; ++i) {
+    in.first[i] = (int)(part_at[i] / 16);                    // parts begin on 256-byte boundaries
+    in.pieces[i] = n += (int)((part_bytes[i] + 15) / 16);
+  }
+  const bool in_kernel = T * H * elt <= team::kHostIoMaxBytes, out_kernel = y_bytes <= team::kHostIoMaxBytes;
   team_step_state st = *st_host;
   st.tok_state = dp + o_ts;
   st.conf = reinterpret_cast<const float*>(dp + o_conf);
@@ -507,11 +517,12 @@ int team_moe_forward_host(team_ctx* ctx, const void* x_host, const team_step_sta
   float* y_dev = reinterpret_cast<float*>(dp + ctx->hs_y_off);
   // copy in, the layer, copy out: all addresses are the context's own, so the sequence is the same every step
   auto issue = [&]() -> int {
-    cudaError_t e = cudaMemcpyAsync(ctx->hs_dev, hp, in_bytes, cudaMemcpyHostToDevice, s);
+    cudaError_t e = in_kernel ? team::launch_host_in(in, s) : cudaMemcpyAsync(ctx->hs_dev, hp, in_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail_cuda(ctx, e, "copy in");
     const int r = team_moe_forward(ctx, dp + o_x, &st, out, y_dev, stream);
     if (r != TEAM_OK) return r;
-    e = cudaMemcpyAsync(hp + ctx->hs_y_off, y_dev, T * H * 4, cudaMemcpyDeviceToHost, s);
+    e = out_kernel ? team::launch_host_out(y_dev, hp + ctx->hs_y_off, y_bytes, s)
+                   : cudaMemcpyAsync(hp + ctx->hs_y_off, y_dev, y_bytes, cudaMemcpyDeviceToHost, s);
     return e == cudaSuccess ? TEAM_OK : fail_cuda(ctx, e, "copy out");
   };
   // Replayed as one graph launch when possible: a stream that can be captured (not the legacy default stream,
@@ -556,7 +567,7 @@ int team_moe_forward_host(team_ctx* ctx, const void* x_host, const team_step_sta
   }
   const cudaError_t es = cudaStreamSynchronize(s);
   if (es != cudaSuccess) return fail_cuda(ctx, es, "synchronise");
-  memcpy(y_host, hp + ctx->hs_y_off, T * H * 4);
+  memcpy(y_host, hp + ctx->hs_y_off, y_bytes);
   return TEAM_OK;
 }
 

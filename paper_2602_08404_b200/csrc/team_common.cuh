@@ -104,7 +104,19 @@ __device__ __forceinline__ void slot_row_weight(int slot, int T, int k, const fl
   }
 }
 
+// Inputs of the host-buffer step: parts of the staging block, in 16-byte pieces, at the same offsets on both sides.
+struct HostIn {
+  static constexpr int kParts = 6;      // x, tok_state, conf, pos, group, branch
+  const uint4* src;                     // pinned host block
+  uint4* dst;                           // device block
+  int first[kParts];                    // first piece of each part
+  int pieces[kParts];                   // pieces of this part and the ones in front of it
+};
+constexpr size_t kHostIoMaxBytes = 1 << 20;
+
 // Kernel launchers (host side), one per translation unit.
+cudaError_t launch_host_in(const HostIn& a, cudaStream_t s);
+cudaError_t launch_host_out(const void* src, void* dst, size_t bytes, cudaStream_t s);
 cudaError_t configure_router(int dtype, int hidden);
 int router_smem_bytes(int hidden);   // dynamic shared memory the logits kernels are opted in to for this hidden size
 cudaError_t configure_select(Dims max_dims);
