@@ -110,7 +110,7 @@ cudaError_t launch_pack_w_tiles(const void* w_gate, const void* w_up, const void
 // rows to the places their slots have.  Measured, end of the routing rounds to end of the gather: 35 -> 19 us at 1024 rows, 65 -> 36 us at 2048.
 // Padding rows stay what they are: they only reach accumulator columns that nobody reads.
 // ---------------------------------------------------------------------------------------------------------
-constexpr int kDispThreads = 512;
+constexpr int kDispThreads = 1024;
 
 struct DispatchArgs {
   const __nv_bfloat16* x;       // [T, H]
@@ -147,20 +147,28 @@ __global__ void __launch_bounds__(kDispThreads) k_dispatch_gather(DispatchArgs a
   asm volatile("griddepcontrol.wait;" ::: "memory");            // the rows' choices are complete
   // 32 rows per warp: lane = row collects its choices as a bit string over the experts, then 32 x 32 bit transposes turn
   // rows into experts (shared-memory atomics per slot took 10 us at 2048 rows)
-  for (int w = warp; w < W; w += kDispThreads / 32) {
+  auto choices = [&](int w, int j0, int (&ee)[8]) {             // eight of the row's choices, all loads in flight
     const int t = w * 32 + lane;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) ee[q] = w < W && t < T && j0 + q < k ? a.topk_idx[t * k + j0 + q] : -1;
+  };
+  int now[8];
+  choices(warp, 0, now);
+  for (int w = warp; w < W; w += kDispThreads / 32) {
     uint32_t m[8] = {};
-    for (int j0 = 0; j0 < k; j0 += 4) {
-      int ee[4];
+    int next[8];
+    choices(w + kDispThreads / 32, 0, next);
+    for (int j0 = 0; j0 < k; j0 += 8) {
+      if (j0 > 0) choices(w, j0, now);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) ee[q] = t < T && j0 + q < k ? a.topk_idx[t * k + j0 + q] : -1;
+      for (int q = 0; q < 8; ++q)
+        if (now[q] >= a.d.elo && now[q] < a.d.ehi) {            // this rank's own experts
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (ee[q] >= a.d.elo && ee[q] < a.d.ehi) {              // this rank's own experts
-#pragma unroll
-          for (int i = 0; i < 8; ++i) m[i] |= (ee[q] >> 5) == i ? 1u << (ee[q] & 31) : 0u;
+          for (int i = 0; i < 8; ++i) m[i] |= (now[q] >> 5) == i ? 1u << (now[q] & 31) : 0u;
         }
     }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) now[q] = next[q];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       if (i * 32 >= E) break;
