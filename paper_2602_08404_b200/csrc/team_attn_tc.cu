@@ -191,9 +191,9 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
   __shared__ int s_row[kAtPairs + 1], s_off[kAtPairs], s_cnt[kAtThreads / 32], s_nonfinite;
   __shared__ float s_m[kAtPairs], s_l[kAtPairs], s_f[kAttnMaxSplits][kAtPairs];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int s = blockIdx.x / a.Hkv, g = blockIdx.x - s * a.Hkv, z = blockIdx.z;
+  const int sg = blockIdx.x % (a.S * a.Hkv), s = sg / a.Hkv, g = sg - s * a.Hkv, z = blockIdx.z;
   const int L = a.L, rep = a.Hq / a.Hkv, n_rows = a.B * L, row0 = s * n_rows;
-  const int pair0 = blockIdx.y * cta_pairs, first_row = pair0 / rep;      // first of the sequence's computed rows
+  const int pair0 = (int)(blockIdx.x / (a.S * a.Hkv)) * cta_pairs, first_row = pair0 / rep;      // first of the sequence's computed rows
   int32_t* status = a.status != nullptr ? a.status : status_sink;
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) {
@@ -712,7 +712,7 @@ static cudaError_t launch(AttnArgs a, const AttnSetup& st, cudaStream_t s, bool*
     }
   }
   cudaLaunchAttribute at[2];
-  const cudaLaunchConfig_t lc = attn_launch<D>(at, dim3(a.S * a.Hkv, m_tiles, n_splits), s);      // clusters without a computed row come last
+  const cudaLaunchConfig_t lc = attn_launch<D>(at, dim3(a.S * a.Hkv * m_tiles, 1, n_splits), s);      // clusters without a computed row come last
   return cudaLaunchKernelEx(&lc, k_block_attention_tc<D>, a, cta_pairs, n_splits, kmap, vmap);
 }
 
