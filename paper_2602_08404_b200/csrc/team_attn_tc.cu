@@ -401,7 +401,9 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
     if (ok && tiles > 0) tc_commit(smem_u32(all_done));
   } else {
     // ---- the queries of this CTA's pairs: A operand of S = Q K^T, per M tile NH halves of [128 rows][128 B], swizzled ----
-    {
+    // A split without a key tile has no product to wait for (all_done) before its partial result goes over these bytes,
+    // so it must not store queries: a slower warp's would end up in the partial result.
+    if (n_tiles > 0) {
       constexpr int PIECES = D / 8, PER = 128 * PIECES / (kAtSoftmaxWarps * 32);      // 16-byte pieces per row, per thread and M tile
       const int c = tid % PIECES;
       uint4 v[2 * PER];
@@ -416,9 +418,9 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
         *reinterpret_cast<uint4*>(smem + ((r >> 7) * NH + (c >> 3)) * P::kQTile + sw128(r & 127, c & 7)) = v[q];
       }
       fence_async_smem();                                   // generic-proxy writes, read by the tensor core
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(q_full));
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(q_full));
     // ------------------------------ softmax ------------------------------
     const int m = warp >> 2;                                 // M tile
     const uint32_t tm_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16), tm = tm_lane + m * 256;      // this warp's quarter of the lanes

@@ -172,3 +172,34 @@ def test_pairs_of_several_branches_share_tiles(d, Hq, Hkv, S, Bn, L, P):
         finite = np.ones(got.shape, bool)
         finite[np.ix_(hit, range(Hq // Hkv), [5])] = False
         assert np.abs(got_bad[finite] - got[finite]).max() <= TOL * np.abs(ref[comp]).max()
+
+
+@pytest.mark.parametrize("L,rep", [(16, 8), (24, 8), (32, 8)], ids=["128_pairs", "192_pairs", "256_pairs"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_splits_without_keys_keep_a_non_finite_query_to_its_row(d, L, rep):
+    """The prefix is far below its maximum, so that most CTAs of a cluster have no key tile; their partial results must be
+    zeros, and not what is left of the queries: a query that is not finite would reach other rows through 0 * inf."""
+    rng = np.random.default_rng(d + L)
+    P, plen, Hkv = 4000, 70, 1
+    st = dict(tok_state=torch.zeros(L, dtype=torch.uint8, device="cuda"), pos=torch.arange(L, dtype=torch.int32, device="cuda"),
+              **{n: torch.zeros(L, dtype=torch.int32, device="cuda") for n in ("group", "branch")})
+    q, k, v = _bf16(rng, L, rep, d), _bf16(rng, L, Hkv, d), _bf16(rng, L, Hkv, d)
+    kp, vp = _bf16(rng, 1, P, Hkv, d), _bf16(rng, 1, P, Hkv, d)
+    kb = np.zeros((1, L, Hkv, d), np.float32)
+    at = np.arange(L, dtype=np.int32)
+    zero = np.zeros(L, np.int32)
+    ref, _, _ = A.block_attention(q, k, v, kp, vp, np.array([plen], np.int32), kb, kb, np.zeros(L, np.uint8), at, zero, zero, L, 0)
+    bad = [0, L // 2, L - 1]
+    q[bad[0]], q[bad[1]], q[bad[2]] = np.inf, np.nan, -np.inf
+    cfg = B.team_attn_config(rep, Hkv, d, L, 1, 1, P, 0)
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    rest = np.setdiff1d(at, bad)
+    args = [_dev(a) for a in (q, k, v, kp, vp)]
+    for _ in range(20):
+        out = torch.full((L, rep, d), 3.0, device="cuda")
+        assert B.team_block_attention(cfg, st, *args, torch.tensor([plen], dtype=torch.int32, device="cuda"), _dev(kb), _dev(kb), out,
+                                      status) == B.TEAM_OK
+        assert status.cpu().tolist() == [0, 0]
+        got = out.cpu().numpy()
+        assert not np.isfinite(got[bad]).any()
+        assert np.abs(got[rest] - ref[rest]).max() <= TOL * np.abs(ref[rest]).max()
