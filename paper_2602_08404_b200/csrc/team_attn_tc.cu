@@ -8,8 +8,8 @@
 // Two M tiles use the same key / value tile: the tensor core works for one while the softmax of the other runs, and a
 // tile is fetched once for 256 pairs.  Thirteen warps, three roles:
 //   warps 0-7  softmax, four per M tile: thread i owns pair i = lane i of tensor memory.  Per tile of 64 keys it reads its
-//              row of S, keeps a running maximum that only moves when the new maximum exceeds it by 2^8 (then the output
-//              accumulator in tensor memory is rescaled, which is rare after the first tiles), and writes
+//              row of S, keeps a running maximum (head size 128: one that only moves when the new maximum exceeds it by
+//              2^8; when it moves, the output accumulator in tensor memory is rescaled), and writes
 //              P = 2^(s - m) as a bf16 pair hi + lo over the columns of S (the A operand of the second product).
 //   warp 8     issues the MMAs: S(t+1) of both M tiles ahead of P V(t).
 //   warps 9-12 loaders.  A tile that lies in the prefix is fetched by one thread with TMA boxes of [64 keys][64
@@ -41,7 +41,6 @@ constexpr int kAtSoftmaxWarps = 8, kAtLoadWarps = 4;
 constexpr int kAtLoadThreads = kAtLoadWarps * 32;
 constexpr int kAtThreads = (kAtSoftmaxWarps + 1 + kAtLoadWarps) * 32;
 constexpr int kAtTmemCols = 512;            // per M tile: S / P twice 64 columns, O 128 (64 with head size 64)
-constexpr float kAtRescale = 8.f;           // the maximum moves only when it grows by more than 2^8
 
 template <int D>
 struct AtShape {
@@ -54,6 +53,13 @@ struct AtShape {
   // head size 64 has room for a second output accumulator, which takes the products of P lo: half as many truncated
   // additions to the large sum
   static constexpr int kOLo = D == 64 ? 64 : 0;
+  // How far the maximum may grow before the one in use moves.  Left behind, P no longer ends at 1: the largest weights lie
+  // anywhere in their binade, and the rounding of lo is up to twice as large relative to them.  With head size 64 that took
+  // the error from 2.0e-6 to 2.3e-6 (mma.sync fragments: 2.2e-6), so there the maximum always moves, at 0.8 us of 13.1 per
+  // call (six prefixes up to 1500).  With head size 128 the error with a maximum left behind is 2.8e-6 at 4096 keys, as it
+  // was or smaller at every shape measured; always moving it gives 2.5e-6 but takes 16 layers over 4096 keys from 448 to
+  // 467 us.
+  static constexpr float kMoveBy = D == 64 ? 0.f : 8.f;
   static constexpr int kOStride = D + 4;                   // floats per row of the partial output (aliases the operands)
   static_assert(kAtPairs * kOStride * 4 <= kOffBars, "partial output must fit");
 };
@@ -452,8 +458,8 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
 #pragma unroll
       for (int e = 4; e < kAtKeys; ++e) mx4[e & 3] = fmaxf(mx4[e & 3], __uint_as_float(sc[e]));
       const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;      // sl2 > 0: the maximum of the scaled scores
-      // the maximum in use moves only when it has to: P stays below 2^8, far inside fp32 and the bf16 pair
-      const bool move = mx > m_used + kAtRescale;            // always on the first tile with a key of the pair (m_used = -inf)
+      // the maximum in use moves only when it has to: P stays below 2^kMoveBy, far inside fp32 and the bf16 pair
+      const bool move = mx > m_used + P::kMoveBy;            // always on the first tile with a key of the pair (m_used = -inf)
       float corr = 1.f;
       if (move) {
         corr = at_ex2(m_used - mx);                          // 0 on the first tile
@@ -488,14 +494,18 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
         if (!(ok = mbar_wait_warp(smem_u32(pv_done + m), (i - 1) & 1, abort_flag, status, 58))) break;
         if (__any_sync(0xffffffffu, move)) {
           tc_fence_after();
+          constexpr int W = P::kMoveBy > 0.f ? 32 : 64;     // where it is in every tile's way: two loads in flight
 #pragma unroll 1
-          for (int c0 = 0; c0 < 128; c0 += 32) {            // both accumulators with head size 64
-            uint32_t r[32];
-            tmem_ld32(tm + 128 + c0, r);
-            tmem_wait_ld(r);
+          for (int c0 = 0; c0 < 128; c0 += W) {             // both accumulators with head size 64
+            uint32_t r[W];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
-            tmem_st32(tm + 128 + c0, r);
+            for (int c = 0; c < W; c += 32) tmem_ld32(tm + 128 + c0 + c, r + c);
+#pragma unroll
+            for (int c = 0; c < W; c += 32) tmem_wait_ld(r + c);
+#pragma unroll
+            for (int e = 0; e < W; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * corr);
+#pragma unroll
+            for (int c = 0; c < W; c += 32) tmem_st32(tm + 128 + c0 + c, r + c);
           }
         }
       }
