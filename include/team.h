@@ -212,7 +212,8 @@ int team_set_policy(team_ctx *ctx, const team_config *cfg);
 /* Router (Algorithm 1 "Router", Sec. 4.1 row selection): logits = x W_r^T in
  * fp32 for every computed row, softmax over all experts, plain top-k with
  * renormalised weights and the decision margin.  x: [T, H] row-major, dtype per
- * config.  Logits stay in the context for team_select_experts. */
+ * config, 16-byte aligned as everywhere (here 8 bytes are enough for bf16).
+ * Logits stay in the context for team_select_experts. */
 int team_route(team_ctx *ctx, const void *x, const team_step_state *st, team_routing *out, void *stream);
 
 /* The router step without any allocation.  (The paper has no counterpart; this is a deployment

@@ -370,6 +370,7 @@ int team_route(team_ctx* ctx, const void* x, const team_step_state* st, team_rou
   int rc = check_state(ctx, st);
   if (rc != TEAM_OK) return rc;
   if (x == nullptr || out == nullptr || !ctx->has_weights) return TEAM_ERR_ARG;
+  if ((uintptr_t)x & (ctx->cfg.dtype == TEAM_DTYPE_BF16 ? 7 : 15)) return TEAM_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const team::Dims d = dims_of(ctx->cfg, st->n_rows);
   ctx->last_launches = 0;

@@ -122,7 +122,8 @@ __device__ __forceinline__ void router_mma(float (&d)[4], uint32_t a0, uint32_t 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <int MT, int NT>
+// kX8: x is only 8-byte aligned (team_route takes such rows), loaded in two pieces
+template <int MT, int NT, bool kX8 = false>
 __global__ void __launch_bounds__(kMmaWarps * 32, 1)
 k_router_logits_mma(const __nv_bfloat16* __restrict__ x, const float* __restrict__ w_router,
                     const uint8_t* __restrict__ tok_state, float* __restrict__ logits, float* __restrict__ y_zero,
@@ -158,7 +159,15 @@ k_router_logits_mma(const __nv_bfloat16* __restrict__ x, const float* __restrict
 #pragma unroll
       for (int m = 0; m < MT; ++m)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) xv[u][m][h] = b < nb ? __ldg(xr[m][h] + b * 4) : make_uint4(0u, 0u, 0u, 0u);
+        for (int h = 0; h < 2; ++h) {
+          if constexpr (kX8) {
+            const uint2* p = reinterpret_cast<const uint2*>(xr[m][h]) + b * 8;
+            const uint2 lo = b < nb ? __ldg(p) : make_uint2(0u, 0u), hi = b < nb ? __ldg(p + 1) : make_uint2(0u, 0u);
+            xv[u][m][h] = make_uint4(lo.x, lo.y, hi.x, hi.y);
+          } else {
+            xv[u][m][h] = b < nb ? __ldg(xr[m][h] + b * 4) : make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
     }
   };
   load(warp, xc, wc);
@@ -380,11 +389,15 @@ struct MmaTile {
 };
 static const MmaTile kMmaTiles[] = {{64, 32, k_router_logits_mma<4, 4>}, {32, 32, k_router_logits_mma<2, 4>},
                                     {32, 16, k_router_logits_mma<2, 2>}, {16, 16, k_router_logits_mma<1, 2>},
-                                    {16, 8, k_router_logits_mma<1, 1>}};
-static MmaTile mma_tile(const Dims& d) {
-  for (const MmaTile& t : kMmaTiles)
+                                    {16, 8, k_router_logits_mma<1, 1>}, {32, 16, k_router_logits_mma<2, 2, true>}};
+constexpr int kMmaTileX8 = 5;          // the one for rows that are only 8-byte aligned
+static MmaTile mma_tile(const Dims& d, bool x8) {
+  if (x8) return kMmaTiles[kMmaTileX8];
+  for (int i = 0; i < kMmaTileX8; ++i) {
+    const MmaTile& t = kMmaTiles[i];
     if (((d.T + t.rows - 1) / t.rows) * ((d.E + t.experts - 1) / t.experts) >= 96) return t;
-  return kMmaTiles[4];
+  }
+  return kMmaTiles[kMmaTileX8 - 1];
 }
 
 // Opt in to the dynamic shared memory the kernels need (done once per context, outside any stream capture).
@@ -433,7 +446,8 @@ cudaError_t configure_router(int dtype, int hidden) {
 
 cudaError_t launch_router_logits(const void* x, int dtype, const float* w_router, const uint8_t* tok_state,
                                  float* logits, float* y_zero, Dims d, int flags, cudaStream_t s) {
-  if (small_router_ok(d)) {
+  const bool x8 = ((uintptr_t)x & 15) != 0;                          // bf16 only: the tensor-core kernel reads 8 bytes at a time
+  if (small_router_ok(d) && !x8) {
     dim3 grid((d.E + kSmallExperts - 1) / kSmallExperts), block(kSmallExperts * kSmallSplit * 32);
     const size_t smem = (size_t)d.T * d.H * sizeof(float) + kSmallExperts * kSmallSplit * kRowTile * sizeof(float);
     if (dtype == TEAM_DTYPE_F32)
@@ -445,7 +459,7 @@ cudaError_t launch_router_logits(const void* x, int dtype, const float* w_router
     return cudaGetLastError();
   }
   if (dtype == TEAM_DTYPE_BF16) {
-    const MmaTile t = mma_tile(d);
+    const MmaTile t = mma_tile(d, x8);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((d.T + t.rows - 1) / t.rows, (d.E + t.experts - 1) / t.experts);
     cfg.blockDim = dim3(kMmaWarps * 32);

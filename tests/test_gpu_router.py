@@ -63,3 +63,36 @@ def test_infinite_and_large_weights_keep_their_sums():
     assert not (got["topk_idx"] == 12).any()
     assert (got["topk_idx"][:, 1] == 13).all()
     assert got["margin"][0] > 1e37        # row 0: 0.5 * 3.4e38 is finite and above the third choice by that much
+
+
+def test_rows_that_are_only_8_byte_aligned():
+    """team_route takes bf16 rows at 8-byte alignment, with every tile size of its dispatch: the same sums as for aligned
+    rows.  What no load width fits is an argument error."""
+    for T, H, E in [(4, 256, 16), (9, 2048, 24), (65, 384, 33), (300, 640, 100), (1000, 256, 128), (2048, 128, 256)]:
+        g = torch.Generator().manual_seed(T)
+        x = torch.randn((T, H), generator=g).to(torch.bfloat16).cuda()
+        w = (torch.randn((E, H), generator=g) / H ** 0.5).cuda()
+        shifted = torch.zeros(T * H + 4, dtype=torch.bfloat16, device="cuda")[4:].view(T, H)
+        shifted.copy_(x)
+        assert x.data_ptr() % 16 == 0 and shifted.data_ptr() % 16 == 8
+        a, b = _route(x, w, 4), _route(shifted, w, 4)
+        if T > 8:
+            for n in a:
+                np.testing.assert_array_equal(a[n], b[n], err_msg=f"{n} {T}")
+        else:                             # aligned rows run the FMA kernel
+            np.testing.assert_allclose(a["probs"], b["probs"], rtol=0, atol=P.PROBS_ATOL)
+        odd = torch.zeros(T * H + 2, dtype=torch.bfloat16, device="cuda")[2:].view(T, H)
+        with pytest.raises(B.TeamError):
+            _route(odd, w, 4)
+
+
+def test_fp32_rows_need_16_bytes():
+    cfg = B.make_config(64, 8, 2, 16, max_rows=4, dtype=B.TEAM_DTYPE_F32)
+    ctx = B.team_create(cfg)
+    w = [torch.zeros(s, device="cuda") for s in ((8, 64), (8, 16, 64), (8, 16, 64), (8, 64, 16))]
+    B.team_set_weights(ctx, *w)
+    st = dict(tok_state=torch.zeros(4, dtype=torch.uint8, device="cuda"), conf=torch.zeros(4, device="cuda"),
+              **{n: torch.zeros(4, dtype=torch.int32, device="cuda") for n in ("pos", "group", "branch")})
+    with pytest.raises(B.TeamError):
+        B.team_route(ctx, torch.zeros(4 * 64 + 2, device="cuda")[2:].view(4, 64), st, dict(topk_idx=torch.zeros((4, 2), dtype=torch.int32, device="cuda")))
+    B.team_destroy(ctx)
