@@ -96,3 +96,56 @@ def test_fp32_rows_need_16_bytes():
     with pytest.raises(B.TeamError):
         B.team_route(ctx, torch.zeros(4 * 64 + 2, device="cuda")[2:].view(4, 64), st, dict(topk_idx=torch.zeros((4, 2), dtype=torch.int32, device="cuda")))
     B.team_destroy(ctx)
+
+
+def _time_route(ctx, x, st, out):
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    best = float("inf")
+    for _ in range(20):
+        ev[0].record()
+        for _ in range(10):
+            B.team_route(ctx, x, st, out)
+        ev[1].record()
+        ev[1].synchronize()
+        best = min(best, ev[0].elapsed_time(ev[1]) * 100)
+    return best
+
+
+def test_activations_that_are_not_finite_stay_in_their_rows():
+    """Rows of NaN and infinities: the other rows' results do not change by a bit; the x of cached rows is not used under
+    delayed caching, so whatever it holds costs nothing either."""
+    T, H, E, k = 300, 4096, 128, 4
+    g = torch.Generator().manual_seed(8)
+    x = torch.randn((T, H), generator=g).to(torch.bfloat16).cuda()
+    w = (torch.randn((E, H), generator=g) / H ** 0.5).cuda()
+    cfg = B.make_config(H, E, k, 64, max_rows=T, dtype=B.TEAM_DTYPE_BF16, flags=B.TEAM_F_DCD)
+    ctx = B.team_create(cfg)
+    gu, dn = (torch.zeros(m * E * 64 * H, dtype=torch.bfloat16, device="cuda") for m in (2, 1))
+    B.team_set_weights(ctx, w, w_gu_tiles=gu, w_down_tiles=dn)
+    state = torch.zeros(T, dtype=torch.uint8)
+    state[50:250] = B.TEAM_TOK_CACHED
+    st = dict(tok_state=state.cuda(), conf=torch.zeros(T, device="cuda"),
+              **{n: torch.zeros(T, dtype=torch.int32, device="cuda") for n in ("pos", "group", "branch")})
+    out = {n: v for n, v in B.alloc_routing(cfg, T).items() if n in ("probs", "topk_idx", "topk_w", "margin")}
+    B.team_route(ctx, x, st, out)
+    want = B.routing_to_host(out)
+    finite_us = _time_route(ctx, x, st, out)
+    bad = x.clone()
+    bad[50:150] = float("nan")
+    bad[150:250, 7] = float("inf")
+    B.team_route(ctx, bad, st, out)
+    got = B.routing_to_host(out)
+    for n in want:
+        np.testing.assert_array_equal(got[n], want[n], err_msg=n)
+    # a logit formed again is a chain of 4096 dependent steps, twice the rest of the call
+    assert _time_route(ctx, bad, st, out) < 1.25 * finite_us
+    bad[0], bad[17, 5], bad[299, 4000] = float("nan"), float("inf"), -float("inf")
+    B.team_route(ctx, bad, st, out)
+    got = B.routing_to_host(out)
+    rest = np.setdiff1d(np.arange(T), [0, 17, 299])
+    for n in want:
+        np.testing.assert_array_equal(got[n][rest], want[n][rest], err_msg=n)
+    assert np.isnan(got["probs"][[0, 17, 299]]).all()
+    # an infinite activation makes a logit infinite with the sign of its weight, as a plain fp32 sum does
+    assert set(got["topk_idx"][17].tolist()) <= set(torch.nonzero(w[:, 5].cpu() > 0)[:, 0].tolist())
+    B.team_destroy(ctx)
