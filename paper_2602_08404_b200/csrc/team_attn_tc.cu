@@ -339,10 +339,16 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
             }
             kk[q] = *reinterpret_cast<const uint4*>(ks + o + c * 8);
             vv[q] = *reinterpret_cast<const uint4*>(vs + o + c * 8);
-            // the tile is multiplied with P = 0 for the pairs of other branches: a value of the block that is not finite
-            // must not reach them.  It counts as 0 here and is added to its own branch's outputs at the end.
-            if (b1 > b0 && key >= plen && at_drop_nonfinite(vv[q])) s_nonfinite = 1;
           }
+        }
+        // the tile is multiplied with P = 0 for the pairs of other branches: a value of the block that is not finite must
+        // not reach them.  It counts as 0 here and is added to its own branch's outputs at the end.  (A loop of its own:
+        // looked at where it is loaded, every value would be waited for before the next one is requested: a call of 4
+        // branches x 16 rows, 2 query heads per key / value head of 128, no prefix, 15.8 us, 14.9 this way.)
+        if (b1 > b0) {
+#pragma unroll
+          for (int q = 0; q < PER; ++q)
+            if (key0 + (ltid + q * kAtLoadThreads) / PIECES >= plen && at_drop_nonfinite(vv[q])) s_nonfinite = 1;
         }
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
@@ -551,47 +557,68 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
   tc_fence_before();
   __syncthreads();
   cg::cluster_group cluster = cg::this_cluster();
-  cluster.sync();
+  if (n_splits > 1) cluster.sync();
   if (!*abort_flag) {
-    // rank z merges its share of the pairs of all partials (distributed shared memory) and writes them: first each
-    // split's weight per pair, then the outputs
+    // rank z writes its share of the pairs
     float* s_o = reinterpret_cast<float*>(smem);
     constexpr int TPR = D / 4;                              // threads per pair (one float4 each)
     const int R = (my_pairs + n_splits - 1) / n_splits, r0 = z * R, r1 = min(my_pairs, r0 + R);
-    for (int pr = r0 + tid; pr < r1; pr += kAtThreads) {
-      float mk[kAttnMaxSplits], lk[kAttnMaxSplits], mx = kNegInf, den = 0.f;
-#pragma unroll
-      for (int k = 0; k < kAttnMaxSplits; ++k) {
-        mk[k] = k < n_splits ? *cluster.map_shared_rank(&s_m[pr], k) : kNegInf;
-        lk[k] = k < n_splits ? *cluster.map_shared_rank(&s_l[pr], k) : 0.f;
-        mx = fmaxf(mx, mk[k]);
+    bool nonfinite;
+    if (n_splits == 1) {
+      // nothing to merge: read from this CTA's own shared memory, not at the 12 bytes per clock of the cluster's, and without
+      // the cluster's barriers (4 branches x 16 rows, 2 query heads per key / value head of 128, no prefix: 14.9 us for the
+      // call through the merge below, 10.7 here; 256 sequences of one row, 100 cached tokens: 77.1, 64.6)
+      nonfinite = s_nonfinite != 0;
+      for (int i = tid; i < my_pairs * TPR; i += kAtThreads) {
+        const int pr = i / TPR, c4 = i % TPR;
+        const float f = 1.f / s_l[pr];
+        const float4 v = *reinterpret_cast<const float4*>(s_o + (size_t)pr * P::kOStride + c4 * 4);
+        *reinterpret_cast<float4*>(a.out + (size_t)s_off[pr] * D + c4 * 4) = make_float4(f * v.x, f * v.y, f * v.z, f * v.w);
       }
+    } else {
+      // merge of all partials (distributed shared memory): first each split's weight per pair, then the outputs
+      for (int pr = r0 + tid; pr < r1; pr += kAtThreads) {
+        float mk[kAttnMaxSplits], lk[kAttnMaxSplits], mx = kNegInf, den = 0.f;
 #pragma unroll
-      for (int k = 0; k < kAttnMaxSplits; ++k) {
-        mk[k] = at_ex2(mk[k] - mx);                          // 0 for a split without a key of the pair (its maximum is -inf)
-        den = fmaf(mk[k], lk[k], den);
+        for (int k = 0; k < kAttnMaxSplits; ++k) {
+          mk[k] = k < n_splits ? *cluster.map_shared_rank(&s_m[pr], k) : kNegInf;
+          lk[k] = k < n_splits ? *cluster.map_shared_rank(&s_l[pr], k) : 0.f;
+          mx = fmaxf(mx, mk[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kAttnMaxSplits; ++k) {
+          mk[k] = at_ex2(mk[k] - mx);                        // 0 for a split without a key of the pair (its maximum is -inf)
+          den = fmaf(mk[k], lk[k], den);
+        }
+        const float inv = 1.f / den;
+#pragma unroll
+        for (int k = 0; k < kAttnMaxSplits; ++k) s_f[k][pr] = mk[k] * inv;
       }
-      const float inv = 1.f / den;
+      nonfinite = __any_sync(0xffffffffu, lane < n_splits && *cluster.map_shared_rank(&s_nonfinite, min(lane, n_splits - 1)) != 0);
+      __syncthreads();
+      for (int i = r0 * TPR + tid; i < r1 * TPR; i += kAtThreads) {
+        const int pr = i / TPR, c4 = i % TPR;
+        float4 v[kAttnMaxSplits];
 #pragma unroll
-      for (int k = 0; k < kAttnMaxSplits; ++k) s_f[k][pr] = mk[k] * inv;
+        for (int k = 0; k < kAttnMaxSplits; ++k) {
+          v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (k < n_splits) v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_o + (size_t)pr * P::kOStride + c4 * 4, k));
+        }
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < kAttnMaxSplits; ++k) {
+          const float f = s_f[k][pr];
+          acc.x = fmaf(f, v[k].x, acc.x); acc.y = fmaf(f, v[k].y, acc.y); acc.z = fmaf(f, v[k].z, acc.z); acc.w = fmaf(f, v[k].w, acc.w);
+        }
+        *reinterpret_cast<float4*>(a.out + (size_t)s_off[pr] * D + c4 * 4) = acc;
+      }
     }
-    const bool nonfinite = __any_sync(0xffffffffu, lane < n_splits && *cluster.map_shared_rank(&s_nonfinite, min(lane, n_splits - 1)) != 0);
-    __syncthreads();
-    for (int i = r0 * TPR + tid; i < r1 * TPR; i += kAtThreads) {
-      const int pr = i / TPR, c4 = i % TPR;
-      float4 v[kAttnMaxSplits];
-#pragma unroll
-      for (int k = 0; k < kAttnMaxSplits; ++k) {
-        v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k < n_splits) v[k] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_o + (size_t)pr * P::kOStride + c4 * 4, k));
-      }
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < kAttnMaxSplits; ++k) {
-        const float f = s_f[k][pr];
-        acc.x = fmaf(f, v[k].x, acc.x); acc.y = fmaf(f, v[k].y, acc.y); acc.z = fmaf(f, v[k].z, acc.z); acc.w = fmaf(f, v[k].w, acc.w);
-      }
-      if (nonfinite) {
+    if (nonfinite) {
+      // values of the block that were not finite counted as 0: they are added to their own branch's outputs
+      for (int i = r0 * TPR + tid; i < r1 * TPR; i += kAtThreads) {
+        const int pr = i / TPR, c4 = i % TPR;
+        float4* dst = reinterpret_cast<float4*>(a.out + (size_t)s_off[pr] * D + c4 * 4);
+        float4 acc = *dst;                                  // this thread's own store
         const int t = s_off[pr] / a.Hq;                     // the pair's row; its block begins at t - pos
         const int t_block = t - (t - row0) % L;
         for (int p = 0; p < L; ++p) {
@@ -603,11 +630,12 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
           if (!isfinite(x2)) acc.z += x2;
           if (!isfinite(x3)) acc.w += x3;
         }
+        *dst = acc;
       }
-      *reinterpret_cast<float4*>(a.out + (size_t)s_off[pr] * D + c4 * 4) = acc;
     }
   }
-  cluster.sync();                                          // peers may still be reading this CTA's partial
+  if (n_splits > 1) cluster.sync();                        // peers may still be reading this CTA's partial
+  else __syncthreads();
   if (a.insert) {
     // this cluster holds all pairs of (sequence, key / value head), so nobody reads the in-block cache any more: the
     // delayed insertion (see k_attn_insert), positions spread over the cluster
