@@ -8,8 +8,8 @@
 // Two M tiles use the same key / value tile: the tensor core works for one while the softmax of the other runs, and a
 // tile is fetched once for 256 pairs.  Thirteen warps, three roles:
 //   warps 0-7  softmax, four per M tile: thread i owns pair i = lane i of tensor memory.  Per tile of 64 keys it reads its
-//              row of S, keeps a running maximum (head size 128: one that only moves when the new maximum exceeds it by
-//              2^8; when it moves, the output accumulator in tensor memory is rescaled), and writes
+//              row of S, keeps a running maximum (one that only moves when the new maximum exceeds it by 2^8, except for
+//              few tiles of head size 64; then the output accumulator in tensor memory is rescaled), and writes
 //              P = 2^(s - m) as a bf16 pair hi + lo over the columns of S (the A operand of the second product).
 //   warp 8     issues the MMAs: S(t+1) of both M tiles ahead of P V(t).
 //   warps 9-12 loaders.  A tile that lies in the prefix is fetched by one thread with TMA boxes of [64 keys][64
@@ -53,13 +53,15 @@ struct AtShape {
   // head size 64 has room for a second output accumulator, which takes the products of P lo: half as many truncated
   // additions to the large sum
   static constexpr int kOLo = D == 64 ? 64 : 0;
-  // How far the maximum may grow before the one in use moves.  Left behind, P no longer ends at 1: the largest weights lie
-  // anywhere in their binade, and the rounding of lo is up to twice as large relative to them.  With head size 64 that took
-  // the error from 2.0e-6 to 2.3e-6 (mma.sync fragments: 2.2e-6), so there the maximum always moves, at 0.8 us of 13.1 per
-  // call (six prefixes up to 1500).  With head size 128 the error with a maximum left behind is 2.8e-6 at 4096 keys, as it
-  // was or smaller at every shape measured; always moving it gives 2.5e-6 but takes 16 layers over 4096 keys from 448 to
-  // 467 us.
-  static constexpr float kMoveBy = D == 64 ? 0.f : 8.f;
+  // The maximum in use may stay behind the running one by 2^kMoveBy, which saves most of the rescaling of the output
+  // accumulator.  But P then no longer ends at 1: the largest weights lie anywhere in their binade, and the rounding of lo is
+  // up to twice as large relative to them.  With head size 64 nothing else is as large while a CTA has few tiles, so up to
+  // kExactTiles of them the maximum always moves: at 1, 4, 8, 12, 16, 32 tiles the error against 64 bits is 1.9, 2.1, 2.2,
+  // 2.3, 2.2, 2.4e-6 that way, 1.9, 2.4, 2.4, 2.6, 2.5, 2.7e-6 with a maximum left behind, and 1.9, 2.1, 2.4, 2.8, 3.2,
+  // 5.2e-6 with mma.sync fragments.  It costs 15 % of a tile.  With head size 128 the maximum is left behind: 2.8e-6 at 4096 keys, as
+  // it was or smaller at every shape measured; always moving it gives 2.5e-6 but takes 16 layers from 448 to 467 us.
+  static constexpr float kMoveBy = 8.f;
+  static constexpr int kExactTiles = D == 64 ? 11 : 0;
   static constexpr int kOStride = D + 4;                   // floats per row of the partial output (aliases the operands)
   static_assert(kAtPairs * kOStride * 4 <= kOffBars, "partial output must fit");
 };
@@ -439,6 +441,7 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
     const int own_lo = plen + (my_branch - b0) * L;          // first key of the pair's own block
     const int pr = tid;                                      // pair of the CTA = lane of tensor memory + 128 * M tile
     const float sl2 = rsqrtf((float)D) * 1.4426950408889634f;      // scores in base 2
+    const float move_by = n_tiles > P::kExactTiles ? P::kMoveBy : 0.f;
     float m_used = kNegInf, l_run = 0.f;                     // running maximum in use (base 2) and row sum
     bool ok = true;
     for (int i = 0; i < n_tiles && ok && m < n_m; ++i) {
@@ -465,7 +468,7 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
       for (int e = 4; e < kAtKeys; ++e) mx4[e & 3] = fmaxf(mx4[e & 3], __uint_as_float(sc[e]));
       const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;      // sl2 > 0: the maximum of the scaled scores
       // the maximum in use moves only when it has to: P stays below 2^kMoveBy, far inside fp32 and the bf16 pair
-      const bool move = mx > m_used + P::kMoveBy;            // always on the first tile with a key of the pair (m_used = -inf)
+      const bool move = mx > m_used + move_by;               // always on the first tile with a key of the pair (m_used = -inf)
       float corr = 1.f;
       if (move) {
         corr = at_ex2(m_used - mx);                          // 0 on the first tile
@@ -500,7 +503,7 @@ k_block_attention_tc(AttnArgs a, int cta_pairs, int n_splits, const __grid_const
         if (!(ok = mbar_wait_warp(smem_u32(pv_done + m), (i - 1) & 1, abort_flag, status, 58))) break;
         if (__any_sync(0xffffffffu, move)) {
           tc_fence_after();
-          constexpr int W = P::kMoveBy > 0.f ? 32 : 64;     // where it is in every tile's way: two loads in flight
+          constexpr int W = P::kExactTiles > 0 ? 64 : 32;     // where it is in every tile's way: two loads in flight
 #pragma unroll 1
           for (int c0 = 0; c0 < 128; c0 += W) {             // both accumulators with head size 64
             uint32_t r[W];

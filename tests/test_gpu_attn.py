@@ -205,17 +205,20 @@ def test_splits_without_keys_keep_a_non_finite_query_to_its_row(d, L, rep):
         assert np.abs(got[rest] - ref[rest]).max() <= TOL * np.abs(ref[rest]).max()
 
 
-def test_head_size_64_keeps_its_accuracy():
-    """The 2-norm error against 64 bits at six ragged prefixes up to 1500.  What limits it is the rounding of P to a bf16
-    pair: at most 2^-18 of the power of two that P lies below, 1.7e-6 rms of it, which with the largest P at 1
-    and the softmax of N(0, 1) scores comes to 2.0e-6 of the output.  2.15e-6 was seen with the products in mma.sync fragments and
-    2.3e-6 with a maximum left behind: P then lies anywhere in its binade."""
-    S, L, Hq, Hkv, d, P = 6, 16, 16, 4, 64, 1500
+@pytest.mark.parametrize("plens,bound", [([1500, 750, 900, 1111, 1300, 1437], 2.15e-6), ([240] * 38, 2.15e-6), ([752] * 38, 2.78e-6), ([1520] * 38, 4.1e-6)],
+                         ids=["split", "4_tiles", "12_tiles", "24_tiles"])
+def test_head_size_64_keeps_its_accuracy(plens, bound):
+    """The 2-norm error against 64 bits.  What limits it where a CTA has few key tiles is the rounding of P to a bf16
+    pair: at most 2^-18 of the power of two that P lies below, 1.7e-6 rms of it, which with the largest P at 1 and the softmax of
+    N(0, 1) scores comes to 2.0e-6 of the output; a maximum left behind (P anywhere in its binade) makes it 2.3e-6.
+    With more tiles the truncated additions to the output accumulator weigh more.  Bounds: the errors of the same products
+    with mma.sync fragments, 2.15, 2.14, 2.79 and 4.15e-6."""
+    S, L, Hq, Hkv, d, P = len(plens), 16, 16, 4, 64, max(plens)
     T, rep = S * L, Hq // Hkv
     g = torch.Generator(device="cuda").manual_seed(64)
     q, k, v, kp, vp = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
                        for s in ((T, Hq, d), (T, Hkv, d), (T, Hkv, d), (S, P, Hkv, d), (S, P, Hkv, d)))
-    plen = torch.tensor([1500, 750, 900, 1111, 1300, 1437], dtype=torch.int32, device="cuda")
+    plen = torch.tensor(plens, dtype=torch.int32, device="cuda")
     st = dict(tok_state=torch.zeros(T, dtype=torch.uint8, device="cuda"), pos=torch.arange(L, dtype=torch.int32, device="cuda").repeat(S),
               group=torch.arange(S, dtype=torch.int32, device="cuda").repeat_interleave(L), branch=torch.zeros(T, dtype=torch.int32, device="cuda"))
     kb = torch.zeros((S, L, Hkv, d), dtype=torch.bfloat16, device="cuda")
@@ -227,4 +230,4 @@ def test_head_size_64_keeps_its_accuracy():
         keys, vals = (torch.cat([p[s, :plen[s]], n[rows]]).double() for p, n in ((kp, k), (vp, v)))
         w = torch.softmax(torch.einsum("tgrd,jgd->tgrj", q[rows].double().view(L, Hkv, rep, d), keys) / d ** 0.5, dim=-1)
         ref[rows] = torch.einsum("tgrj,jgd->tgrd", w, vals).reshape(L, Hq, d)
-    assert float((out.double() - ref).norm() / ref.norm()) < 2.15e-6
+    assert float((out.double() - ref).norm() / ref.norm()) < bound
