@@ -3,7 +3,8 @@
 // of cached tokens are not computed and their keys / values come from an in-block cache, followed by the delayed
 // insertion of the newly accepted tokens' keys / values into that cache.
 //
-// The attention kernel is in team_attn_tc.cu.
+// The attention kernels are in team_attn_tc.cu (tensor memory; the choice between the two) and team_attn_frag.cu (warp-level
+// fragments, head size 64 with few pairs over few keys).
 // k_attn_insert: after the pass, the fresh key / value of every decoded row computed in the base branch goes into
 // the in-block cache at its position.
 #include "team_attn.cuh"

@@ -1,4 +1,4 @@
-// Shared by the attention kernel and the insertion (Sec. 4.1, the attention half of delayed caching): argument block and
+// Shared by the attention kernels and the insertion (Sec. 4.1, the attention half of delayed caching): argument block and
 // the test for "this row is computed".
 #pragma once
 
@@ -29,8 +29,12 @@ struct AttnArgs {
 
 __device__ __forceinline__ bool attn_computed(int state, int flags) { return !((flags & TEAM_F_DCD) && state == TEAM_TOK_CACHED); }
 
-// the attention itself (team_attn_tc.cu), with the insertion where *inserted comes back true; one-time set-up on a
-// device's first call
+// the attention itself, on one of the kernels, with the insertion where *inserted comes back true; one-time set-up on a
+// device's first call (team_attn_tc.cu)
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s, bool* inserted);
+
+// head size 64 on warp-level fragments (team_attn_frag.cu)
+cudaError_t configure_attention_frag();
+cudaError_t launch_attention_frag(const AttnArgs& a, int m_tiles, int n_splits, cudaStream_t s);
 
 }  // namespace team

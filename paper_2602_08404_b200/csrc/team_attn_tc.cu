@@ -709,12 +709,45 @@ static cudaError_t attn_setup(const AttnSetup** out) {
   e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = setup_kernel<64>(n_sms, st.clusters[0]);
   if (e == cudaSuccess) e = setup_kernel<128>(n_sms, st.clusters[1]);
+  if (e == cudaSuccess) e = configure_attention_frag();
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult found;
   if (e == cudaSuccess) e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
   if (e == cudaSuccess && found != cudaDriverEntryPointSuccess) e = cudaErrorNotSupported;
   if (e == cudaSuccess) st.encode = reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(fn);
   return e;
+}
+
+// Waves of clusters of which `at_once` run at once.
+static long long at_waves(long long clusters, int at_once) { return clusters <= at_once ? 1 : (clusters + at_once - 1) / at_once; }
+
+// Head size 64: whether a call runs the fragment kernel (then how) instead of the tensor-memory kernel, planned as given.
+//
+// With few pairs over few key tiles it takes fewer steps: 4 sequences x 4 key / value heads, 4 pairs, no prefix 5.9 us against
+// 7.9; 64 pairs, 3000 cached tokens 13.0 against 13.2; 256 pairs 17.3 against 15.8.  Both are estimated in ns: every wave of
+// clusters takes its tiles of keys and what is around them, which grows with a CTA's pairs (fitted to 1400 and 2800 replayed calls
+// of 1 to 1024 sequences x heads, 4 to 1024 pairs, prefixes of 0 to 6000, within 5 and 6 % rms).  How many rows are
+// computed is not known here: with delayed caching the estimates are means over 4, 3, 2 and 1 quarters of them.
+static bool use_fragments(const AttnArgs& a, const AttnSetup& st, int tiles_max, int tc_m, int tc_splits, int* m_tiles, int* n_splits) {
+  const int run_pairs = a.L * (a.Hq / a.Hkv);              // of a sequence and branch
+  const long long heads = (long long)a.S * a.Hkv, runs = heads * a.B;
+  // M tiles by the largest number of pairs; splits until the grid fills the SMs, each keeping at least two tiles
+  *m_tiles = (run_pairs + 127) / 128;
+  int n = 1;
+  while (n < kAttnMaxSplits && *m_tiles * runs * n * 2 <= st.clusters[0][1] && tiles_max >= 4 * n) n *= 2;
+  *n_splits = n;
+  if (st.clusters[0][n] < 1) return false;
+  const int split = tc_splits > 1, tc_tiles = (tiles_max + tc_splits - 1) / tc_splits, tiles = (tiles_max + n - 1) / n;
+  const int tile = tc_tiles > AtShape<64>::kExactTiles ? (tc_m == 1 ? 870 : 1130) : (tc_m == 1 ? 970 : 1290);
+  long long tc = 0, frag = 0;
+  for (int q = (a.flags & TEAM_F_DCD) ? 1 : 4; q <= 4; ++q) {
+    const long long run = ((long long)q * run_pairs + 3) / 4, all = ((long long)q * run_pairs * a.B + 3) / 4;
+    const int warps = ((int)(run < 128 ? run : 128) + 15) / 16, of_cta = (int)(all < 128 * tc_m ? all : 128 * tc_m);
+    tc += at_waves((all + 128 * tc_m - 1) / (128 * tc_m) * heads, st.clusters[0][tc_splits]) *
+          (tc_tiles * tile + (split ? 6550 : 6050) + of_cta * (split ? 2330 : 1600) / 128);
+    frag += at_waves((run + 127) / 128 * runs, st.clusters[0][n]) * (tiles * (857 + 88 * warps) + 4000 + 376 * warps) + 900;
+  }
+  return frag * 103 < tc * 100;        // clearly less: the estimates scatter by more than that
 }
 
 template <int D>
@@ -737,6 +770,13 @@ static cudaError_t launch(AttnArgs a, const AttnSetup& st, cudaStream_t s, bool*
         cta_pairs = 128 * m;
         n_splits = n;
       }
+    }
+  }
+  if (D == 64) {
+    int frag_m_tiles, frag_splits;
+    if (use_fragments(a, st, tiles_max, cta_pairs / 128, n_splits, &frag_m_tiles, &frag_splits)) {
+      *inserted = false;
+      return launch_attention_frag(a, frag_m_tiles, frag_splits, s);
     }
   }
   const int m_tiles = (int)((pairs + cta_pairs - 1) / cta_pairs);

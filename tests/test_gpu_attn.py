@@ -205,6 +205,19 @@ def test_splits_without_keys_keep_a_non_finite_query_to_its_row(d, L, rep):
         assert np.abs(got[rest] - ref[rest]).max() <= TOL * np.abs(ref[rest]).max()
 
 
+def _reference(q, k, v, kp, vp, plen, S, L):
+    """One branch, every row computed, in 64 bits."""
+    T, Hq, d = q.shape
+    Hkv = k.shape[1]
+    ref = torch.zeros((T, Hq, d), dtype=torch.float64, device="cuda")
+    for s in range(S):
+        rows = slice(s * L, (s + 1) * L)
+        keys, vals = (torch.cat([p[s, :plen[s]], n[rows]]).double() for p, n in ((kp, k), (vp, v)))
+        w = torch.softmax(torch.einsum("tgrd,jgd->tgrj", q[rows].double().view(L, Hkv, Hq // Hkv, d), keys) / d ** 0.5, dim=-1)
+        ref[rows] = torch.einsum("tgrj,jgd->tgrd", w, vals).reshape(L, Hq, d)
+    return ref
+
+
 @pytest.mark.parametrize("plens,bound", [([1500, 750, 900, 1111, 1300, 1437], 2.15e-6), ([240] * 38, 2.15e-6), ([752] * 38, 2.78e-6), ([1520] * 38, 4.1e-6)],
                          ids=["split", "4_tiles", "12_tiles", "24_tiles"])
 def test_head_size_64_keeps_its_accuracy(plens, bound):
@@ -214,7 +227,7 @@ def test_head_size_64_keeps_its_accuracy(plens, bound):
     With more tiles the truncated additions to the output accumulator weigh more.  Bounds: the errors of the same products
     with mma.sync fragments, 2.15, 2.14, 2.79 and 4.15e-6."""
     S, L, Hq, Hkv, d, P = len(plens), 16, 16, 4, 64, max(plens)
-    T, rep = S * L, Hq // Hkv
+    T = S * L
     g = torch.Generator(device="cuda").manual_seed(64)
     q, k, v, kp, vp = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
                        for s in ((T, Hq, d), (T, Hkv, d), (T, Hkv, d), (S, P, Hkv, d), (S, P, Hkv, d)))
@@ -224,10 +237,32 @@ def test_head_size_64_keeps_its_accuracy(plens, bound):
     kb = torch.zeros((S, L, Hkv, d), dtype=torch.bfloat16, device="cuda")
     out = torch.zeros((T, Hq, d), device="cuda")
     assert B.team_block_attention(B.team_attn_config(Hq, Hkv, d, L, S, 1, P, 0), st, q, k, v, kp, vp, plen, kb, kb.clone(), out) == B.TEAM_OK
-    ref = torch.zeros((T, Hq, d), dtype=torch.float64, device="cuda")
-    for s in range(S):
-        rows = slice(s * L, (s + 1) * L)
-        keys, vals = (torch.cat([p[s, :plen[s]], n[rows]]).double() for p, n in ((kp, k), (vp, v)))
-        w = torch.softmax(torch.einsum("tgrd,jgd->tgrj", q[rows].double().view(L, Hkv, rep, d), keys) / d ** 0.5, dim=-1)
-        ref[rows] = torch.einsum("tgrj,jgd->tgrd", w, vals).reshape(L, Hq, d)
+    ref = _reference(q, k, v, kp, vp, plen, S, L)
     assert float((out.double() - ref).norm() / ref.norm()) < bound
+
+
+@pytest.mark.parametrize("S,Hkv,rep,L,Bn,P", [(1, 1, 1, 1, 1, 0), (1, 4, 4, 1, 1, 5), (3, 2, 16, 8, 1, 56), (2, 1, 43, 3, 2, 61), (40, 4, 2, 8, 1, 120), (1, 2, 4, 64, 1, 1000),
+                                              (150, 1, 1, 5, 1, 190)], ids=lambda v: str(v))
+def test_few_pairs_of_head_size_64(S, Hkv, rep, L, Bn, P):
+    """The fragment kernel: one pair, one M tile exactly and one pair more, keys split and not, several waves of CTAs, cached rows."""
+    rng = np.random.default_rng(S + L + P)
+    T, Hq, d = S * Bn * L, Hkv * rep, 64
+    step = dict(tok_state=rng.integers(0, 3, T).astype(np.uint8), conf=np.zeros(T, np.float32), pos=np.tile(np.arange(L, dtype=np.int32), S * Bn),
+                group=np.repeat(np.arange(S, dtype=np.int32), Bn * L), branch=np.tile(np.repeat(np.arange(Bn, dtype=np.int32), L), S))
+    step["tok_state"][0] = B.TEAM_TOK_NEW
+    q, k, v = _bf16(rng, T, Hq, d), _bf16(rng, T, Hkv, d), _bf16(rng, T, Hkv, d)
+    kp, vp = _bf16(rng, S, max(P, 1), Hkv, d), _bf16(rng, S, max(P, 1), Hkv, d)
+    kb, vb = _bf16(rng, S, L, Hkv, d), _bf16(rng, S, L, Hkv, d)
+    plen = rng.integers(P // 2, P + 1, S).astype(np.int32)
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    out = torch.full((T, Hq, d), 3.0, device="cuda")
+    kb_dev, vb_dev = _dev(kb), _dev(vb)
+    assert B.team_block_attention(B.team_attn_config(Hq, Hkv, d, L, S, Bn, P, B.TEAM_F_DCD), B.state_to_device(step), _dev(q), _dev(k), _dev(v), _dev(kp),
+                                  _dev(vp), torch.as_tensor(plen).cuda(), kb_dev, vb_dev, out, status) == B.TEAM_OK
+    assert status.cpu().tolist() == [0, 0]
+    ref, kb, vb = A.block_attention(q, k, v, kp, vp, plen, kb, vb, step["tok_state"], step["pos"], step["group"], step["branch"], L, B.TEAM_F_DCD)
+    comp, got = A.computed_rows(step["tok_state"], B.TEAM_F_DCD), out.cpu().numpy()
+    assert np.abs(got[comp] - ref[comp]).max() <= TOL * np.abs(ref[comp]).max()
+    assert (got[~comp] == 3.0).all()
+    np.testing.assert_array_equal(kb_dev.float().cpu().numpy(), kb.astype(np.float32))
+    np.testing.assert_array_equal(vb_dev.float().cpu().numpy(), vb.astype(np.float32))
