@@ -241,6 +241,29 @@ def test_head_size_64_keeps_its_accuracy(plens, bound):
     assert float((out.double() - ref).norm() / ref.norm()) < bound
 
 
+@pytest.mark.parametrize("rep,L", [(4, 16), (8, 24), (7, 40)], ids=["64_pairs", "192_pairs", "280_pairs"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_long_walks_reuse_the_rings(d, rep, L):
+    """Enough sequences that the keys are split little or not at all: CTAs of one and of two M tiles walk about 20 to 30 key
+    tiles, through every stage of the key and value rings and every score buffer several times."""
+    S, Hkv, P = 40, 4, 1900
+    T, Hq = S * L, Hkv * rep
+    g = torch.Generator(device="cuda").manual_seed(d + rep)
+    q, k, v, kp, vp = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+                       for s in ((T, Hq, d), (T, Hkv, d), (T, Hkv, d), (S, P, Hkv, d), (S, P, Hkv, d)))
+    plen = torch.randint(P // 2, P + 1, (S,), generator=g, device="cuda", dtype=torch.int32)
+    plen[0], plen[1], plen[2] = P, 1216, 1215              # 19 tiles exactly, and one key less
+    st = dict(tok_state=torch.zeros(T, dtype=torch.uint8, device="cuda"), pos=torch.arange(L, dtype=torch.int32, device="cuda").repeat(S),
+              group=torch.arange(S, dtype=torch.int32, device="cuda").repeat_interleave(L), branch=torch.zeros(T, dtype=torch.int32, device="cuda"))
+    kb = torch.zeros((S, L, Hkv, d), dtype=torch.bfloat16, device="cuda")
+    out = torch.zeros((T, Hq, d), device="cuda")
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    assert B.team_block_attention(B.team_attn_config(Hq, Hkv, d, L, S, 1, P, 0), st, q, k, v, kp, vp, plen, kb, kb.clone(), out, status) == B.TEAM_OK
+    assert status.cpu().tolist() == [0, 0]
+    ref = _reference(q, k, v, kp, vp, plen, S, L)
+    assert float((out.double() - ref).abs().max()) <= TOL * float(ref.abs().max())
+
+
 @pytest.mark.parametrize("S,Hkv,rep,L,Bn,P", [(1, 1, 1, 1, 1, 0), (1, 4, 4, 1, 1, 5), (3, 2, 16, 8, 1, 56), (2, 1, 43, 3, 2, 61), (40, 4, 2, 8, 1, 120), (1, 2, 4, 64, 1, 1000),
                                               (150, 1, 1, 5, 1, 190)], ids=lambda v: str(v))
 def test_few_pairs_of_head_size_64(S, Hkv, rep, L, Bn, P):
