@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(kDispThreads) k_dispatch_gather(DispatchArgs a
   int32_t* s_row0 = s_n + EN;
   int32_t* s_cost = s_row0 + EN;          // [EN + 1] cost of the experts in front of this one
   int32_t* s_widx = s_cost + EN + 1;
+  __shared__ int3 s_tot[(TEAM_MAX_EXPERTS + TEAM_MAX_SHARED + 31) / 32];      // per warp of experts: rows, cost, experts with work
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");            // the rows' choices are complete
@@ -191,51 +192,72 @@ __global__ void __launch_bounds__(kDispThreads) k_dispatch_gather(DispatchArgs a
     }
   }
   __syncthreads();
-  for (int e = warp; e < EN; e += kDispThreads / 32) {          // slots of the expert in front of each word (W <= 64)
-    int run = 0;
-    for (int w0 = 0; w0 < W; w0 += 32) {
-      const int w = w0 + lane, c = w < W ? __popc(bits[e * W1 + w]) : 0;
-      int incl = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
+  // slots of the expert in front of each word (W <= 64), by a thread per expert where there are few words, else by a warp
+  if (W <= 4) {
+    if (tid < EN) {
+      int run = 0;
+      for (int w = 0; w < W; ++w) {
+        pre[tid * W1 + w] = (uint16_t)run;
+        run += __popc(bits[tid * W1 + w]);
       }
-      if (w < W) pre[e * W1 + w] = (uint16_t)(run + incl - c);
-      run += __shfl_sync(0xffffffffu, incl, 31);
+      s_n[tid] = run;
     }
-    if (lane == 0) s_n[e] = run;
+  } else {
+    for (int e = warp; e < EN; e += kDispThreads / 32) {
+      int run = 0;
+      for (int w0 = 0; w0 < W; w0 += 32) {
+        const int w = w0 + lane, c = w < W ? __popc(bits[e * W1 + w]) : 0;
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int up = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += up;
+        }
+        if (w < W) pre[e * W1 + w] = (uint16_t)(run + incl - c);
+        run += __shfl_sync(0xffffffffu, incl, 31);
+      }
+      if (lane == 0) s_n[e] = run;
+    }
+    __syncthreads();
+  }
+  // places of the experts, costs in front of them: expert = thread, every warp scans its 32 and adds what the warps in
+  // front of it have (one warp that walks over all experts takes 1.5 us at 256 of them)
+  const int used_warps = (EN + 31) >> 5;
+  int n_slots = 0, rows_in = 0, cost_in = 0;
+  uint32_t act = 0;
+  if (warp < used_warps) {
+    n_slots = tid < EN ? s_n[tid] : 0;
+    rows_in = padded_rows(n_slots);
+    cost_in = tile_cost(n_slots);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int r1 = __shfl_up_sync(0xffffffffu, rows_in, o), c1 = __shfl_up_sync(0xffffffffu, cost_in, o);
+      if (lane >= o) { rows_in += r1; cost_in += c1; }
+    }
+    act = __ballot_sync(0xffffffffu, n_slots > 0);
+    if (lane == 31) s_tot[warp] = make_int3(rows_in, cost_in, __popc(act));
   }
   __syncthreads();
-  if (warp == 0) {                                              // places of the experts, costs in front of them
-    int rows = 0, cost = 0, used = 0;
-    for (int e0 = 0; e0 < EN; e0 += 32) {
-      const int e = e0 + lane, n = e < EN ? s_n[e] : 0;
-      const int pr = padded_rows(n), cs = tile_cost(n);
-      int ir = pr, ic = cs;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int r1 = __shfl_up_sync(0xffffffffu, ir, o), c1 = __shfl_up_sync(0xffffffffu, ic, o);
-        if (lane >= o) { ir += r1; ic += c1; }
-      }
-      const uint32_t act = __ballot_sync(0xffffffffu, n > 0);
-      if (e < EN) {
-        s_row0[e] = rows + ir - pr;
-        s_cost[e] = cost + ic - cs;
-        s_widx[e] = used + __popc(act & ((1u << lane) - 1u));
-      }
-      rows += __shfl_sync(0xffffffffu, ir, 31);
-      cost += __shfl_sync(0xffffffffu, ic, 31);
-      used += __popc(act);
+  if (tid < EN) {
+    int rows = rows_in - padded_rows(n_slots), cost = cost_in - tile_cost(n_slots), used = __popc(act & ((1u << lane) - 1u));
+    for (int w = 0; w < warp; ++w) {
+      rows += s_tot[w].x;
+      cost += s_tot[w].y;
+      used += s_tot[w].z;
     }
-    if (lane == 0) s_cost[EN] = cost;
+    s_row0[tid] = rows;
+    s_cost[tid] = cost;
+    s_widx[tid] = used;
+    if (tid == EN - 1) s_cost[EN] = cost + tile_cost(n_slots);
   }
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int e = tid; e < EN; e += kDispThreads)
       if (s_n[e] > 0) a.plan.work[s_widx[e]] = make_int4(e, s_row0[e], s_n[e], 0);
     // where CTA b of the GEMMs begins: the expert that holds cost total * b / gemm_ctas, and the unit inside it
-    const long long total = s_cost[EN];
+    // (32 bits: 260 experts of 2048 slots cost 260 * 4096)
+    const uint32_t total = s_cost[EN];
+    const uint32_t tiles_a = a.d.I / 64, tiles_b = a.d.H / 128;
     for (int b = tid; b <= a.gemm_ctas; b += kDispThreads) {
       const int at = (int)(total * b / a.gemm_ctas);
       int lo = 0, hi = EN;                                      // the last expert with s_cost[e] <= at (empty ones: cost 0)
@@ -246,8 +268,12 @@ __global__ void __launch_bounds__(kDispThreads) k_dispatch_gather(DispatchArgs a
       int units_a = 0, units_b = 0;
       const int cost = s_cost[lo + 1] - s_cost[lo], chunks = (s_n[lo] + kTileChunk - 1) / kTileChunk;
       if (cost > 0) {                                           // 0: behind the last expert
-        units_a = (int)((long long)(at - s_cost[lo]) * (a.d.I / 64) * chunks / cost);
-        units_b = (int)((long long)(at - s_cost[lo]) * (a.d.H / 128) * chunks / cost);
+        auto part = [&](uint32_t tiles) {                       // at most 4096 * 16 * tiles / cost
+          return tiles < 65536u ? (int)((uint32_t)(at - s_cost[lo]) * chunks * tiles / (uint32_t)cost)
+                                : (int)((unsigned long long)(at - s_cost[lo]) * chunks * tiles / (uint32_t)cost);
+        };
+        units_a = part(tiles_a);
+        units_b = part(tiles_b);
       }
       a.plan.begin[b] = make_int4(s_widx[lo], units_a, units_b, 0);
     }
