@@ -19,10 +19,15 @@ CHUNKS = W.Shape("tile_chunks_bf16", 384, 6, 3, 192, 1, "bf16", 25, 3, 5, 1, 2, 
 FULL = W.Shape("tile_full_bf16", 256, 2, 2, 64, 0, "bf16", 32, 2, 4, 1, 3, 0.7, seqs=4, seed=22)
 OVER = dataclasses.replace(FULL, name="tile_over_bf16", block=43, seqs=3, seed=23)
 ONE = W.Shape("tile_one_row_bf16", 128, 200, 4, 64, 0, "bf16", 1, 1, 1, 1, 1, 0.7, seed=24)
+# a second batch of choices per row, several shared experts, experts of several warps
+TOP12 = W.Shape("tile_top12_bf16", 128, 250, 12, 64, 4, "bf16", 10, 2, 3, 1, 2, 0.7, seqs=7, seed=27)
+# more rows than one pass of a CTA's warps takes, in one and in many groups
+ROWS = W.Shape("tile_1088_rows_bf16", 128, 40, 3, 64, 2, "bf16", 64, 2, 8, 1, 3, 0.7, seqs=17, seed=25)
+WIDE = W.Shape("tile_1100_rows_bf16", 128, 33, 9, 64, 1, "bf16", 11, 2, 3, 1, 3, 0.7, seqs=25, branches=4, seed=31)
 
 
 @pytest.mark.parametrize("flags", [0, B.TEAM_F_DCD | B.TEAM_F_LAC], ids=["vanilla", "team"])
-@pytest.mark.parametrize("shape", [CHUNKS, FULL, OVER, ONE, W.MINI_SHARED, W.MINI_WRAP], ids=lambda s: s.name)
+@pytest.mark.parametrize("shape", [CHUNKS, FULL, OVER, ONE, TOP12, ROWS, WIDE, W.MINI_SHARED, W.MINI_WRAP], ids=lambda s: s.name)
 def test_chunks_and_tiles(shape, flags):
     weights = W.make_weights(shape)
     steps = W.make_schedule(shape)
