@@ -3,8 +3,10 @@
 // A copy node of a graph waits for the whole grid in front of it, is handed to a copy engine and hands back: 15 us from
 // the end of the step's kernel to the end of the 32 KB copy of y, for 1 us of PCIe time.  A kernel that is chained with
 // programmatic dependent launch reads or writes the pinned block (mapped into the device's address space) as soon as
-// its predecessor is done: the call of 4 rows 70.5 -> 63.1 us.  Up to kHostIoMaxBytes per direction; larger blocks are bound by PCIe, not by latency, and
-// stay on the copy engines.
+// its predecessor is done: the call of 4 rows 70.5 -> 63.1 us.  Up to kHostIoMaxBytes per direction.  Both ways at hidden 2048
+// and few experts, copy engine and kernel, us per call: 8 rows 76 and 60, 32 rows 93 and 79, 128 rows 202 and 184, 256 rows
+// (1 MB of x, 2 MB of y) 345 and 322, 1024 rows 1189 and 1163, which is as much as two runs differ there: PCIe and the host's own
+// copies bind larger blocks, and an engine moves those without taking SMs.
 #include "team_common.cuh"
 
 namespace team {
