@@ -303,6 +303,17 @@ __global__ void __launch_bounds__(kAttnThreads, 1) k_block_attention(AttnArgs a,
     }
   }
   cluster.sync();                                          // peers may still be reading this CTA's partial
+  if (a.insert) {
+    // this cluster holds all pairs of (sequence, key / value head), so nobody reads the in-block cache any more: the
+    // delayed insertion (see k_attn_insert), positions spread over the cluster
+    for (int i = tid; i < L * (D / 8); i += kAttnThreads) {
+      const int p = i / (D / 8), c = i % (D / 8);
+      if (p % n_splits != z || !s_comp[p] || a.tok_state[row0 + p] == TEAM_TOK_MASKED) continue;
+      const size_t src = ((size_t)(row0 + p) * a.Hkv + g) * D + c * 8, dst = (((size_t)s * L + p) * a.Hkv + g) * D + c * 8;
+      *reinterpret_cast<uint4*>(a.k_block + dst) = *reinterpret_cast<const uint4*>(a.k_new + src);
+      *reinterpret_cast<uint4*>(a.v_block + dst) = *reinterpret_cast<const uint4*>(a.v_new + src);
+    }
+  }
 }
 
 static constexpr int attn_smem_bytes() {

@@ -737,6 +737,10 @@ static bool use_fragments(const AttnArgs& a, const AttnSetup& st, int tiles_max,
   while (n < kAttnMaxSplits && *m_tiles * runs * n * 2 <= st.clusters[0][1] && tiles_max >= 4 * n) n *= 2;
   *n_splits = n;
   if (st.clusters[0][n] < 1) return false;
+  // The insertion (0.9 us) is part of either kernel where one cluster holds all pairs of a (sequence, key / value head), else a
+  // launch of its own, which takes 2 us of the host's time: calls that are not replayed are bound by that (4 branches x 4
+  // rows, 16 pairs, 100 cached tokens: 12.7 us a call on the tensor-memory kernel, 15.4 with two launches; replayed 8.2 and 7.2).
+  const bool insert_launch = a.B > 1 || *m_tiles > 1, tc_launch = (long long)run_pairs * a.B > 128 * tc_m;
   const int split = tc_splits > 1, tc_tiles = (tiles_max + tc_splits - 1) / tc_splits, tiles = (tiles_max + n - 1) / n;
   const int tile = tc_tiles > AtShape<64>::kExactTiles ? (tc_m == 1 ? 870 : 1130) : (tc_m == 1 ? 970 : 1290);
   long long tc = 0, frag = 0;
@@ -745,9 +749,10 @@ static bool use_fragments(const AttnArgs& a, const AttnSetup& st, int tiles_max,
     const int warps = ((int)(run < 128 ? run : 128) + 15) / 16, of_cta = (int)(all < 128 * tc_m ? all : 128 * tc_m);
     tc += at_waves((all + 128 * tc_m - 1) / (128 * tc_m) * heads, st.clusters[0][tc_splits]) *
           (tc_tiles * tile + (split ? 6550 : 6050) + of_cta * (split ? 2330 : 1600) / 128);
-    frag += at_waves((run + 127) / 128 * runs, st.clusters[0][n]) * (tiles * (857 + 88 * warps) + 4000 + 376 * warps) + 900;
+    frag += at_waves((run + 127) / 128 * runs, st.clusters[0][n]) * (tiles * (857 + 88 * warps) + 4000 + 376 * warps) +
+            (insert_launch && !tc_launch ? 2900 : 900);
   }
-  return frag * 103 < tc * 100;        // clearly less: the estimates scatter by more than that
+  return frag * 105 < tc * 100;        // clearly less: the estimates scatter by more than that
 }
 
 template <int D>
@@ -775,7 +780,7 @@ static cudaError_t launch(AttnArgs a, const AttnSetup& st, cudaStream_t s, bool*
   if (D == 64) {
     int frag_m_tiles, frag_splits;
     if (use_fragments(a, st, tiles_max, cta_pairs / 128, n_splits, &frag_m_tiles, &frag_splits)) {
-      *inserted = false;
+      a.insert = *inserted = a.B == 1 && frag_m_tiles == 1;
       return launch_attention_frag(a, frag_m_tiles, frag_splits, s);
     }
   }
