@@ -809,7 +809,7 @@ def run_attn(args):
                        "l2": f"inputs larger than L2: KV caches rotate over {R} layers", "parallelism": "replicas"},
             "clocks": sampler.summary(), "delayed_caching": t, "recompute_all": res["recompute_all"],
             # a contraction: at this shape the flops take longer on the tensor roof than the bytes on the HBM roof
-            "roofline": {"bound": "tensor", "kernel": "k_block_attention", "achieved": t["tensor_tflops"],
+            "roofline": {"bound": "tensor", "kernel": "k_block_attention_tc", "achieved": t["tensor_tflops"],
                          "peak": measured_peaks()[2], "peak_kind": "of " + measured_peaks()[3] + " (bf16 sustained)",
                          "unit": "TFLOP/s", "frac": t["tensor_tflops"] / measured_peaks()[2], "hbm_frac": t["hbm_frac"],
                          "traffic": None},

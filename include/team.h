@@ -254,15 +254,17 @@ int team_select_experts(team_ctx *ctx, const team_step_state *st, team_routing *
  * combine.  y: fp32 [T, H]; rows with class TEAM_CLS_SKIP are left untouched
  * (they keep the previous step's output), all other rows are overwritten.
  * `out` may be NULL; tables nobody asked for may not be built at all (with at
- * most 8 rows the expert kernel works from the rows' choices alone). */
+ * most 8 rows, and on the tensor-memory kernels, the experts work from the rows'
+ * choices alone). */
 int team_moe_forward(team_ctx *ctx, const void *x, const team_step_state *st, team_routing *out,
                      float *y, void *stream);
 
 /* The same layer step for callers whose buffers live in HOST memory (pageable
  * or pinned): x_host [T, H] in the config's dtype, the five arrays of st_host
  * as host pointers, y_host fp32 [T, H].  The call packs the inputs into a pinned
- * staging block owned by the context, moves them to the device with one copy,
- * runs team_moe_forward on `stream`, copies y back and synchronises the stream
+ * staging block owned by the context, moves them to the device (by a kernel that
+ * copies the call's rows, above 1 MB with one copy of the whole block), runs
+ * team_moe_forward on `stream`, copies y back (likewise) and synchronises the stream
  * before it returns, so y_host is valid on return.  Rows with class
  * TEAM_CLS_SKIP receive what the previous call on this context left in the
  * context's device-side y (zero before the first call): use one context per

@@ -161,7 +161,11 @@ cudaError_t timing_events(team_ctx* ctx, cudaEvent_t* e0, cudaEvent_t* e1) {
 
 bool use_tensor_path(const team_ctx* ctx) { return ctx->cfg.dtype == TEAM_DTYPE_BF16 && !ctx->force_simt; }
 
-// Calls of fewer rows than this run the weight-streaming kernel when the shape allows both (measured crossover).
+// Contexts of fewer rows than this run the weight-streaming kernel when the shape allows both.  Replayed steps, streaming and
+// tensor-memory kernels, us: one block of 32 rows 98 and 96 (SDAR shape), 83 and 81 (256 experts, a shared one), 48 rows 96
+// and 104, 105 and 97, 64 rows in 4 branches 142 and 122, 120 and 105, 64 rows of 4 sequences 172 and 170, 153 and 163, 96
+// rows of 6 sequences 199 and 190, 223 and 202.  By time alone the line would lie at about 64 rows; it stays at 96, where no
+// shape measured is slower, because it also says which weight layout a context needs.
 constexpr int kTileMinRows = 96;
 
 void choose_expert_kernel(team_ctx* ctx) {

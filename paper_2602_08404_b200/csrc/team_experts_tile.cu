@@ -52,7 +52,7 @@ __host__ __device__ inline int padded_rows(int n) { return n / kTileChunk * kTil
 // What an expert with n token-slots costs per weight tile, in the time of 128 bytes of weights.  One chunk: a weight tile
 // and half a token tile (two weight tiles share it).  More: a step moves one weight tile for two chunks and is bound by
 // its stages, not by HBM, so it costs as much as a step of two weight tiles and its token tiles more.  Measured with 128,
-// 256 and 384 per pair of chunks: 185 rows with a shared expert 132.4, 126.7 and 125.5 us, 2048 rows 319.8, 318.4, 350.
+// 256 and 384 per pair of chunks, replayed: 185 rows with a shared expert 131.6, 124.9 and 122.8 us, 2048 rows 319, 307, 336.
 __device__ __forceinline__ int tile_cost(int n) {
   const int chunks = (n + kTileChunk - 1) / kTileChunk;
   return chunks <= 1 ? chunks * 128 + padded_rows(n) / 2 : (chunks + 1) / 2 * 256 + padded_rows(n);
@@ -105,10 +105,10 @@ cudaError_t launch_pack_w_tiles(const void* w_gate, const void* w_up, const void
 // the token rows themselves as B tiles: [chunk rows padded to 16][H] as [kb][np rows][64 k] swizzled.
 //
 // One CTA doing this alone (a counting sort of T * k slots) is a serial 22 us at 1024 rows and 28 us at 2048, followed
-// by a gather that has to wait for it (13 / 37 us).  Here every CTA forms the tables for itself from the rows' choices,
+// by a gather that has to wait for it (13 and 37 us).  Here every CTA forms the tables for itself from the rows' choices,
 // as a bit matrix [expert][row] in shared memory: the rank of row t inside expert e is a population count (slots
 // ascend inside an expert as rows do), so nothing is sorted and no CTA waits for another one, and then copies its own
-// rows to the places their slots have.  Measured, end of the routing rounds to end of the gather: 35 -> 19 us at 1024 rows, 65 -> 36 us at 2048.
+// rows to the places their slots have: 14 us at 1024 rows and 24 at 2048 (SDAR shape, serialised under ncu).
 // Padding rows stay what they are: they only reach accumulator columns that nobody reads.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kDispThreads = 1024;

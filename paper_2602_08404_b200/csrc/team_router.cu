@@ -98,9 +98,9 @@ k_router_logits(const float* __restrict__ x, const float* __restrict__ w_router,
 // of two bf16 numbers is exact in fp32.  The tensor core truncates while it accumulates (chains over the whole hidden
 // dimension were off by 1.05e-6 against 64 bits), so a chain is the three parts of one fragment of 16 elements, the
 // smallest first, and the fragments are added with rounded fp32 additions: 1.08e-7, against 1.57e-7 of the fp32 FMA
-// kernels that this one replaced (2-norm, 16 to 2048 rows, hidden 2048).  Measured at hidden 2048 x 128 experts, in the
-// call, end to end: 2048 rows 48 -> 29 us, 1024 rows 26 -> 17, 128 rows 11 -> 6; the mma.sync rate and the reads of x
-// and W from L2 are what is left.  mma.sync and not tcgen05: a tcgen05 chain cannot be cut every 16 elements.
+// kernels that this one replaced (2-norm, 16 to 2048 rows, hidden 2048).  team_route at hidden 2048 x 128 experts, replayed, with its top-k:
+// 2048 rows 46.0 -> 17.4 us, 1024 rows 25.9 -> 12.5, 128 rows 12.9 -> 7.1; the mma.sync rate and the reads of x and W from
+// L2 are what is left.  mma.sync and not tcgen05: a tcgen05 chain cannot be cut every 16 elements.
 //
 // A warp owns MT x 16 rows by NT x 8 experts and every eighth block of 32 hidden elements.  Lane (g, c) of a fragment
 // takes elements 8c .. 8c+7 of its row's block -- 16 contiguous bytes of x, 32 of W -- which is a permutation of the

@@ -315,8 +315,8 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
     }
   }
 
-  // The dispatch tables are skipped when nobody reads them: no export asked for, and an expert kernel that
-  // works from the rows' choices alone (at most 8 rows, all resident).
+  // The dispatch tables are skipped when nobody reads them: no export asked for, and an expert kernel that works from the
+  // rows' choices alone (at most 8 rows, all resident; the tensor-memory kernels at any number of rows).
   if (mode == kSelRounds || skip_dispatch) return;
   if (mode == kSelCluster) {
     // all CTAs' choices are in the routing tables and visible; CTA 0 alone builds the dispatch tables from them

@@ -101,9 +101,9 @@ __device__ __forceinline__ int warp_topk_picks(uint32_t (&key)[kMaxPerLane], int
 // receives the j-th choice.
 //
 // One loop, not unrolled: with tens of warps per SM running it once, instruction issue and instruction fetches bound it,
-// not a pick's latency (sorted lists, with the picks moved to their lanes afterwards, took 17400 clock
-// cycles for 32 rows on one SM; calls of 128 rows 157 -> 142 us with this loop and the walk of the classification).  A pick is the lane's largest key, the warp's largest (one redux) and the
-// lowest expert id that holds it (another).
+// not a pick's latency (sorted lists, with the picks moved to their lanes afterwards, took 17400 clock cycles for 32 rows on
+// one SM; calls of 128 rows 157 -> 142 us with this loop and the walk of the classification).  A pick is the lane's largest
+// key, the warp's largest (one redux) and the lowest expert id that holds it (another).
 template <int NE>
 __device__ __forceinline__ TopkResult warp_topk_loop(const float (&v)[kMaxPerLane], int k, int lane) {
   TopkResult r;

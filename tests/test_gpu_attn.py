@@ -65,7 +65,8 @@ def test_block_attention_over_a_schedule(shape, flags, d, Hq, Hkv, P):
 @pytest.mark.parametrize("d,Hq,Hkv", [(128, 16, 2), (64, 8, 1)], ids=["d128", "d64"])
 def test_block_attention_long_prefix(flags, d, Hq, Hkv):
     """A prefix of many key tiles with a ragged end, eight query heads per key/value head (more (row, head) pairs than
-    one CTA holds) and few enough CTAs that the keys are split over a cluster; queries scaled up so that the running
+    one CTA holds) and few enough CTAs that the keys are split over a cluster (two or three tiles per CTA);
+    queries scaled up so that the running
     maximum keeps moving (the rescaling of the output accumulator is exercised, not only its first tile)."""
     shape = W.paper_point()
     rng = np.random.default_rng(977 + d)
