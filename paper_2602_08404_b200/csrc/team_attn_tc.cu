@@ -741,7 +741,8 @@ static bool use_fragments(const AttnArgs& a, const AttnSetup& st, int tiles_max,
   // launch of its own, which takes 2 us of the host's time: calls that are not replayed are bound by that (4 branches x 4
   // rows, 16 pairs, 100 cached tokens: 12.7 us a call on the tensor-memory kernel, 15.4 with two launches; replayed 8.2 and 7.2).
   const bool insert_launch = a.B > 1 || *m_tiles > 1, tc_launch = (long long)run_pairs * a.B > 128 * tc_m;
-  const int split = tc_splits > 1, tc_tiles = (tiles_max + tc_splits - 1) / tc_splits, tiles = (tiles_max + n - 1) / n;
+  const int split = tc_splits > 1;
+  const long long tc_tiles = (tiles_max + tc_splits - 1) / tc_splits, tiles = (tiles_max + n - 1) / n;
   const int tile = tc_tiles > AtShape<64>::kExactTiles ? (tc_m == 1 ? 870 : 1130) : (tc_m == 1 ? 970 : 1290);
   long long tc = 0, frag = 0;
   for (int q = (a.flags & TEAM_F_DCD) ? 1 : 4; q <= 4; ++q) {
