@@ -11,7 +11,7 @@
 // its partial (max, sum, output) in its own shared memory and rank z of the cluster merges rows z*128/n .. of all partials
 // through distributed shared memory and writes them.
 // What bounds it with few tiles: the chain of latencies from the step state over the first loads to the merge, 4.5 us per
-// wave of CTAs; the tensor-memory kernel, with its hand-offs between warps and its tensor-memory round trips, needs 8.
+// wave of CTAs; the tensor-memory kernel, with its hand-offs between warps and its tensor-memory round trips, needs 6 to 7.
 #include <cooperative_groups.h>
 
 #include "team_attn.cuh"

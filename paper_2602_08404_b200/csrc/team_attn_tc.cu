@@ -18,8 +18,9 @@
 // What bounds it: a tile of 64 keys and two M tiles takes 2100 clock cycles, of which the counters show the tensor pipe busy
 // for 1300 (S at N = 64 reads its A operand as long as it computes, and P counts twice) and the softmax needs 1300 (16
 // exponentials per clock and SM); the rest is hand-offs between the two.  Around the tiles: 6000 cycles until the first scores
-// and 5000 to 10000 for the merge, whose reads of distributed shared memory run at about 12 bytes per clock and SM.  Kernel at 4096 cached tokens, 32 query and 4 key / value heads of 128,
-// block of 32 x 4 branches: 43 us with one M tile per CTA, loads through registers and P in shared memory, 25 now.
+// and 5000 to 10000 for the merge, whose reads of distributed shared memory run at about 12 bytes per clock and SM.  Kernel
+// at 4096 cached tokens, 32 query and 4 key / value heads of 128, block of 32 x 4 branches: 43 us with one M tile per CTA,
+// loads through registers and P in shared memory, 25 now.
 // Every wait is an mbarrier wait with a limit; when one runs out the CTA stops working, reports TEAM_ERR_TIMEOUT and
 // still takes part in the cluster's barriers and frees its tensor memory.
 #include <cooperative_groups.h>
