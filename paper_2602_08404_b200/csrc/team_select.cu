@@ -505,7 +505,12 @@ cudaError_t configure_select(Dims max_dims) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const int smem = (int)select_smem_bytes(max_dims);
+  // the most that any number of rows needs: the choices are kept up to kIdxInSmemMax of them, so a call of that many may need more
+  // than one of max_rows
+  Dims most_idx = max_dims;
+  most_idx.T = most_idx.T < kIdxInSmemMax / most_idx.k ? most_idx.T : kIdxInSmemMax / most_idx.k;
+  const size_t at_max = select_smem_bytes(max_dims), at_most_idx = select_smem_bytes(most_idx);
+  const int smem = (int)(at_max > at_most_idx ? at_max : at_most_idx);
   std::lock_guard<std::mutex> lock(mu);
   if (dev >= 0 && dev < 64 && prepared[dev] >= smem && prepared[dev] > 0) return cudaSuccess;
   for (const void* fn : {reinterpret_cast<const void*>(&k_select<kSelMaxThreads>), reinterpret_cast<const void*>(&k_select<kSelMaxThreads / 2>)}) {
