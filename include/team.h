@@ -247,7 +247,8 @@ int team_route_static(const team_config *cfg, const void *x, const void *w_route
                       team_routing *out, void *stream);
 
 /* TEAM selection (Eq. 4, Algorithm 1 steps 1-3) and dispatch tables, from the
- * logits left by the preceding team_route on the same context, stream and rows. */
+ * logits left by the preceding team_route or team_moe_forward on the same
+ * context, stream and rows. */
 int team_select_experts(team_ctx *ctx, const team_step_state *st, team_routing *out, void *stream);
 
 /* The whole layer step: route, select, dispatch, SwiGLU experts, weighted

@@ -19,6 +19,8 @@ namespace cg = cooperative_groups;
 
 constexpr int kF32Threads = 1024, kF32Warps = kF32Threads / 32;
 constexpr int kF32Rows = 8;
+constexpr int kF32IdleThreads = kF32Threads - kF32Rows * 32;      // of the warps without a row
+static_assert(kF32Rows * TEAM_MAX_EXPERTS <= 8 * kF32IdleThreads, "logit = thread of the smallest cluster");
 static_assert(kF32Threads >= TEAM_MAX_EXPERTS + TEAM_MAX_SHARED, "expert = thread");
 constexpr int kF32Cluster = 16;                       // needs the opt-in beyond the portable 8
 // Expert weights of a call at most.  Below the limit general path and here, us: 3.1 MB (4 rows, hidden 256, 16 experts of 128
@@ -33,6 +35,7 @@ struct F32Args {
   const float* w_gate;           // [E + ns, I, H]
   const float* w_up;
   const float* w_down;           // [E + ns, I/16, H, 16]
+  float* logits;                 // [T, E] left for team_select_experts
   float* act;                    // [T * (k + ns), I]
   float* y;                      // [T, H]
   StepPtrs st;
@@ -110,6 +113,9 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_step_f32(F32Args a) {
       }
   }
   cluster.sync();
+  // The logits are left for team_select_experts, by threads that route no row: 0.05 us of the step (in front of the meeting the
+  // stores cost 0.4, behind the activations 0.05 as well).
+  if (const int i = rank * kF32IdleThreads + tid - kF32Rows * 32; tid >= kF32Rows * 32 && i < T * E) a.logits[i] = s.logits[i];
   // ---- selection, by every CTA; the experts with rows, in ascending order ----
   block_select<kF32Threads>([&](int t, int e) { return s.logits[t * E + e]; }, a.st, a.d, a.p, s.rt, s.bits, 1, a.cls_out, a.status);
   const unsigned act_b = __ballot_sync(0xffffffffu, tid < EN && s.bits[min(tid, EN - 1)] != 0u);
@@ -237,6 +243,7 @@ cudaError_t launch_step_f32(const void* x, const float* w_router, const void* w_
   a.w_gate = static_cast<const float*>(w_gate);
   a.w_up = static_cast<const float*>(w_up);
   a.w_down = static_cast<const float*>(w_down);
+  a.logits = ws.logits;
   a.act = ws.act;
   a.y = y;
   a.st = sel.st;
