@@ -23,10 +23,15 @@ constexpr int kF32IdleThreads = kF32Threads - kF32Rows * 32;      // of the warp
 static_assert(kF32Rows * TEAM_MAX_EXPERTS <= 8 * kF32IdleThreads, "logit = thread of the smallest cluster");
 static_assert(kF32Threads >= TEAM_MAX_EXPERTS + TEAM_MAX_SHARED, "expert = thread");
 constexpr int kF32Cluster = 16;                       // needs the opt-in beyond the portable 8
-// Expert weights of a call at most.  Below the limit general path and here, us: 3.1 MB (4 rows, hidden 256, 16 experts of 128
-// columns) 20.5, 13.6; 2.4 MB (8 rows x 3 choices, hidden 512, 8 of 48) 21.4, 16.7.  Above it 7.6 MB (8 rows x 4, hidden 448, 11
-// of 128) take 22.9 on the general path and took 29.3 here with a slower down product: one cluster's share of L2's rate.
-constexpr size_t kF32MaxBytes = 4 << 20;
+// What one cluster reads at L2's rate to 16 SMs, where the general path has all of them: the weights of a call (its experts' and
+// the router's) at most, and the router's weights times rows (every CTA multiplies its share with all rows out of shared memory).
+// Replayed, general path and here, us: 3.0 MB (4 rows x 2 choices, hidden 256, 16 experts of 128 columns) 14.2, 14.1; 3.8 MB (4 x 2,
+// hidden 512, 80 columns) 14.8, 13.4; 4.0 MB, 1 of them the router's (2 rows x 2, hidden 1024, 256 of 64) 16.5, 15.3.  Above
+// the limit 4.5 MB (4 x 2, hidden 256, 16 of 192) 15.1, 15.9; 6.0 MB (same, 256 columns) 15.3, 17.8; 7.0 MB, 4 of them the
+// router's (4 x 1, hidden 4096, 256 of 16) 25.8, 30.0.  Rows x router of 4 MB and 8 MB: 8 x 1024 x 128 (2 choices) 18.0, 16.9, x
+// 256 experts 18.0, 19.1; 8 x 2048 x 64 (1 choice) 20.6, 20.3, x 128 21.0, 21.2.  (Launched one by one the general path takes 3
+// to 5 us more, the host's time for four launches.)
+constexpr size_t kF32MaxBytes = 4 << 20, kF32MaxRouterRows = 4 << 20;
 constexpr size_t kF32MaxSmem = 200 << 10;
 
 struct F32Args {
@@ -232,7 +237,8 @@ cudaError_t configure_step_f32(int* ctas) {
 
 bool step_f32_supported(const Dims& d) {
   const size_t slots = (size_t)d.T * (d.k + d.ns), experts = slots < (size_t)(d.E + d.ns) ? slots : d.E + d.ns;
-  return d.T <= kF32Rows && experts * d.H * d.I * 12 <= kF32MaxBytes && f32_smem_layout(d, nullptr, nullptr) <= kF32MaxSmem;
+  const size_t router = (size_t)d.E * d.H * 4;
+  return d.T <= kF32Rows && experts * d.H * d.I * 12 + router <= kF32MaxBytes && router * d.T <= kF32MaxRouterRows && f32_smem_layout(d, nullptr, nullptr) <= kF32MaxSmem;
 }
 
 cudaError_t launch_step_f32(const void* x, const float* w_router, const void* w_gate, const void* w_up, const void* w_down, Workspace ws,

@@ -118,6 +118,20 @@ def test_fp32_step_without_tables(name, flags):
         layer.close()
 
 
+@pytest.mark.parametrize("rows,hidden,n_experts,launches", [(4, 4096, 256, 4), (8, 1024, 128, 1), (8, 1024, 129, 4), (1, 2048, 256, 1)])
+def test_fp32_step_router_weights(rows, hidden, n_experts, launches):
+    """The router's weights count, too: the one-cluster step is for calls whose weights one cluster reads faster."""
+    shape = replace(F1, block=rows, hidden=hidden, n_experts=n_experts, top_k=1, inter=16)
+    layer = P.Layer(shape, W.make_weights(shape), 0)
+    try:
+        step = W.make_schedule(shape)[1]
+        y, _, got = _both(layer.ctx, layer.cfg, shape, B.to_device(step["x"], B.TEAM_DTYPE_F32), B.state_to_device(step))
+        assert got == [4, launches]
+        assert ((y[1] - y[0]).abs() <= 1e-5 * y[0].abs().max(dim=1, keepdim=True).values).all()
+    finally:
+        layer.close()
+
+
 @pytest.mark.parametrize("rank", [0, 1])
 def test_fp32_expert_parallel_rank_without_tables(rank):
     from tests.test_gpu_ep import _rank_layer
