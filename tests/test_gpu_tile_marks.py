@@ -21,6 +21,9 @@ CASES = {
     "128_rows_shared": replace(S, block=32, branches=4, n_shared=1),
     "129_rows_shared": replace(S, block=1, seqs=129, n_shared=4, inter=64),
     "300_rows_of_2_experts": replace(S, block=10, seqs=30, n_experts=2, top_k=2, hidden=384),
+    # more pairs of chunks than tiles, every row on every expert; one word more than a warp has lanes, the last with one row
+    "2048_rows_of_2_experts": replace(S, block=32, seqs=64, n_experts=2, top_k=2, inter=128, hidden=128),
+    "1025_rows_shared": replace(S, block=41, seqs=25, n_experts=12, top_k=5, n_shared=1, inter=64, hidden=128),
     "2048_rows": replace(S, block=32, seqs=64, n_experts=9, top_k=3, inter=64, hidden=128),
 }
 
