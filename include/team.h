@@ -254,9 +254,11 @@ int team_select_experts(team_ctx *ctx, const team_step_state *st, team_routing *
 /* The whole layer step: route, select, dispatch, SwiGLU experts, weighted
  * combine.  y: fp32 [T, H]; rows with class TEAM_CLS_SKIP are left untouched
  * (they keep the previous step's output), all other rows are overwritten.
- * `out` may be NULL; tables nobody asked for may not be built at all (with at
+ * `out` may be NULL; tables nobody asked for may not be built at all: with at
  * most 8 rows, and on the tensor-memory kernels, the experts work from the rows'
- * choices alone). */
+ * choices alone, and calls that ask for nothing may be routed inside the expert
+ * kernel (weight-streaming kernel, more than 8 rows) or run as one kernel (fp32,
+ * at most 8 rows and few weights). */
 int team_moe_forward(team_ctx *ctx, const void *x, const team_step_state *st, team_routing *out,
                      float *y, void *stream);
 
@@ -296,11 +298,13 @@ int team_last_launch_count(const team_ctx *ctx);
 
 /* Average device time (ms) of the expert kernel over the launches made since
  * the counters were last reset, measured with CUDA events on the launching
- * stream when timing is enabled.  Synchronises the stream. */
+ * stream when timing is enabled.  It includes whatever that kernel does besides:
+ * the routing of calls that are routed inside it, the whole step where the step
+ * is one kernel.  Synchronises the stream. */
 int team_expert_timing(team_ctx *ctx, int32_t enable, void *stream, float *avg_ms_out, int32_t *launches_out);
 
-/* Name of the expert kernel this context's team_moe_forward launches (static string), e.g. for labelling a
- * measurement.  NULL context: "". */
+/* Name of the expert kernel this context's team_moe_forward launches for max_rows rows and no tables (static
+ * string), e.g. for labelling a measurement.  NULL context: "". */
 const char *team_expert_kernel_name(const team_ctx *ctx);
 
 /* Diagnostic: run the expert FFNs of a bf16 context through the plain-FMA
@@ -365,8 +369,9 @@ int team_block_attention(const team_attn_config *cfg, const team_step_state *st,
                          void *k_block, void *v_block, float *out, int32_t *status, void *stream);
 
 /* Diagnostic knobs of a context (not for production use).
- *   TEAM_KNOB_NO_FUSE (value 0/1): with at most 8 rows and no dispatch table asked for, team_moe_forward runs the
- *     whole step as one kernel; 1 keeps the three-kernel sequence (router, selection, experts) instead.
+ *   TEAM_KNOB_NO_FUSE (value 0/1): 1 keeps router, selection and experts apart where team_moe_forward would run the
+ *     whole step as one kernel (at most 8 rows and no dispatch table asked for; fp32: nothing asked for) or route the
+ *     rows inside the weight-streaming kernel (nothing asked for).
  *   TEAM_KNOB_WAIT_LIMIT_US (1 .. 10,000,000): how long a device-side wait (the one-kernel step's grid barrier) may
  *     last before the kernel gives up, records TEAM_ERR_TIMEOUT in the status word and returns; default about 1 s.
  *   TEAM_KNOB_EXTRA_ARRIVALS (0/1): 1 makes that barrier wait for one arrival that never comes, so that the

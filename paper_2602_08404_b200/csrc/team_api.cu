@@ -25,7 +25,7 @@ struct team_ctx {
   int stream_item_tile, tile_item_tile;
   bool fused_ok;      // at most 8 rows: the whole step can run as one kernel (router and selection in its prologue)
   int f32_ctas;       // fp32: CTAs of the cluster that runs a small step as one kernel (0: never)
-  int no_fuse;        // diagnostic knob: keep the three-kernel sequence
+  int no_fuse;        // diagnostic knob: keep router, selection and experts apart
   int extra_arrivals; // diagnostic knob: arrivals the fused step's barrier waits for beyond the grid's own
   long long spin_cycles;   // limit of device-side waits, in SM clock cycles
   float* ordered;          // ordered combine of the one-kernel step: [SMs][max_rows][H] partial outputs (null: off)
@@ -634,10 +634,16 @@ int team_last_launch_count(const team_ctx* ctx) { return ctx ? ctx->last_launche
 
 const char* team_expert_kernel_name(const team_ctx* ctx) {
   if (ctx == nullptr) return "";
-  if (!use_tensor_path(ctx)) return "k_gate_up + k_down";
+  const team::Dims d = dims_of(ctx->cfg, ctx->cfg.max_rows);
+  if (!use_tensor_path(ctx)) {
+    const bool one = ctx->cfg.dtype == TEAM_DTYPE_F32 && ctx->f32_ctas > 0 && !ctx->no_fuse && team::step_f32_supported(d);
+    return one ? "k_step_f32 (router, selection and experts in one launch)" : "k_gate_up + k_down";
+  }
   if (!ctx->stream_path) return "k_grouped_gemm (tcgen05: gate/up + SwiGLU, then down + combine)";
   const bool fused = ctx->fused_ok && !ctx->no_fuse && !team::experts_stream_gathers(ctx->cfg.max_rows);
-  return fused ? "k_experts_stream (fused step: router, selection and experts in one launch)" : "k_experts_stream";
+  if (fused) return "k_experts_stream (fused step: router, selection and experts in one launch)";
+  const bool routes = !ctx->no_fuse && team::experts_stream_routes(d, ctx->cfg.max_rows, ctx->n_sms);
+  return routes ? "k_experts_stream (selection inside)" : "k_experts_stream";
 }
 
 int team_debug_knob(team_ctx* ctx, int knob, long long value) {

@@ -142,3 +142,16 @@ def test_fp32_expert_parallel_rank_without_tables(rank):
         assert ((y[1] - y[0]).abs() <= 1e-5 * y[0].abs().max(dim=1, keepdim=True).values).all()
     finally:
         B.team_destroy(ctx)
+
+
+@pytest.mark.parametrize("shape,name", [(F1, "k_step_f32"), (F32_CASES["9_rows"], "k_gate_up"), (CASES["31_rows"], "k_experts_stream (selection"),
+                                        (replace(S1, block=8), "k_experts_stream (fused")], ids=["one_cluster", "fp32", "inline", "fused"])
+def test_expert_kernel_name(shape, name):
+    """The kernel that a call of max_rows rows without tables launches; with the knob the general one."""
+    ctx = B.team_create(P.lib_config(shape, 3))
+    try:
+        assert B.team_expert_kernel_name(ctx).startswith(name)
+        B.team_debug_knob(ctx, B.TEAM_KNOB_NO_FUSE, 1)
+        assert B.team_expert_kernel_name(ctx) in ("k_gate_up + k_down", "k_experts_stream")
+    finally:
+        B.team_destroy(ctx)
