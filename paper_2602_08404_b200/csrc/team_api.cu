@@ -272,7 +272,7 @@ int team_create(const team_config* cfg, team_ctx** out) {
     off += (bytes + 255) & ~size_t(255);
     return at;
   };
-  const size_t o_logits = take(T * E * 4), o_idx = take(T * k * 4), o_w = take(T * k * 4), o_margin = take(T * 4);
+  const size_t o_logits = take(T * E * 4), o_idx = take(T * k * 4), o_w = take(T * k * 4);
   const size_t o_cls = take(T), o_gm = take((size_t)cfg->max_groups * ((E + 63) / 64) * 8);
   const size_t o_cnt = take(EN * 4), o_off = take((EN + 1) * 4), o_perm = take(S * 4), o_act_list = take(EN * 4);
   const size_t o_scal = take(64), o_items = take((EN + S / 8 + 2) * sizeof(team::WorkItem));
@@ -295,7 +295,7 @@ int team_create(const team_config* cfg, team_ctx** out) {
   ws.r.probs = nullptr;
   ws.r.topk_idx = reinterpret_cast<int32_t*>(b + o_idx);
   ws.r.topk_w = reinterpret_cast<float*>(b + o_w);
-  ws.r.margin = reinterpret_cast<float*>(b + o_margin);
+  ws.r.margin = nullptr;
   ws.r.tok_class = b + o_cls;
   ws.r.group_mask = reinterpret_cast<uint64_t*>(b + o_gm);
   ws.r.expert_count = reinterpret_cast<int32_t*>(b + o_cnt);

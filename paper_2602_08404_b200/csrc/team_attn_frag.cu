@@ -24,7 +24,6 @@ namespace team {
 constexpr int kAttnDim = 64;            // head size
 constexpr int kAttnPairs = 128;         // (row, head) pairs per CTA
 constexpr int kAttnThreads = 256;
-constexpr int kAttnWarps = 8;
 constexpr int kAttnKeys = 64;          // keys per tile
 constexpr int kAttnStages = 3;
 

@@ -66,7 +66,7 @@ struct WorkItem {
 
 struct Workspace {
   float* logits;        // [max_rows, E]
-  RoutePtrs r;          // context-owned routing tables (probs is null here)
+  RoutePtrs r;          // context-owned routing tables (probs and margin are null here)
   WorkItem* items;      // [E + ns + max_rows*(k+ns)/tile + 1]
   int32_t* n_items;     // [1]
   float* act;           // fp32 path: [max_rows*(k+ns), I] SwiGLU activations

@@ -620,7 +620,6 @@ __global__ void __launch_bounds__(kStThreads, 1) k_experts_stream(StArgs a) {
             if (a.ex.topk_w) a.ex.topk_w[t * k + lane] = w;
           }
           if (lane == 0) {
-            a.r.margin[t] = f_margin;
             if (a.ex.margin) a.ex.margin[t] = f_margin;
             a.r.tok_class[t] = (uint8_t)f_mycls;
             if (a.ex.tok_class) a.ex.tok_class[t] = (uint8_t)f_mycls;

@@ -5,8 +5,8 @@
 //  k_router_logits : more rows, fp32 activations (and hidden sizes the small kernel does not hold).  The work is split
 //                    over experts (one warp per expert, 128-bit loads of the expert's row) and over tiles of 8 rows
 //                    whose activations sit in shared memory.
-//                    Each of them also zeroes the output rows that the streaming expert kernel accumulates into, or the bit matrix
-//                    of the choices for the tensor-memory kernels.
+//  The first two also zero the output rows that the streaming expert kernel accumulates into, or the bit matrix of the choices
+//  for the tensor-memory kernels.
 //  k_router_topk   : one warp per row: softmax over all experts, plain top-k by warp shuffles,
 //                    renormalised weights, decision margin (team_route's outputs).
 #include <mutex>
@@ -26,8 +26,7 @@ __device__ __forceinline__ uint32_t rows_to_zero(const uint8_t* __restrict__ tok
 }
 
 __global__ void __launch_bounds__(kExpertsPerCta * 32)
-k_router_logits(const float* __restrict__ x, const float* __restrict__ w_router, const uint8_t* __restrict__ tok_state,
-                float* __restrict__ logits, float* __restrict__ y_zero, Dims d, int flags) {
+k_router_logits(const float* __restrict__ x, const float* __restrict__ w_router, float* __restrict__ logits, Dims d) {
   extern __shared__ __align__(16) float s_x[];   // [kRowTile][H]
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the selection kernel may stage its inputs meanwhile
   const int t0 = blockIdx.y * kRowTile;
@@ -49,12 +48,6 @@ k_router_logits(const float* __restrict__ x, const float* __restrict__ w_router,
   for (int i = tid; i < nt * H / 4; i += blockDim.x) reinterpret_cast<float4*>(s_x)[i] = __ldg(src + i);
   for (int i = nt * H + tid; i < kRowTile * H; i += blockDim.x) s_x[i] = 0.f;
 
-  // Output rows of computed tokens start from zero (the expert kernel adds partial sums into them);
-  // the CTAs of one row tile share the job.
-  if (y_zero != nullptr) {
-    for (uint32_t m = rows_to_zero(tok_state, t0, nt, lane, flags); m != 0u; m &= m - 1u)
-      for (int i = blockIdx.x * blockDim.x + tid; i < H; i += gridDim.x * blockDim.x) y_zero[(size_t)(t0 + __ffs(m) - 1) * H + i] = 0.f;
-  }
   __syncthreads();
 
   if (e >= d.E) return;
@@ -525,7 +518,7 @@ cudaError_t launch_router_logits(const void* x, int dtype, const float* w_router
   dim3 grid((d.E + kExpertsPerCta - 1) / kExpertsPerCta, (d.T + kRowTile - 1) / kRowTile);
   dim3 block(kExpertsPerCta * 32);
   const size_t smem = (size_t)kRowTile * d.H * sizeof(float);
-  k_router_logits<<<grid, block, smem, s>>>(static_cast<const float*>(x), w_router, tok_state, logits, y_zero, d, flags);
+  k_router_logits<<<grid, block, smem, s>>>(static_cast<const float*>(x), w_router, logits, d);
   return cudaGetLastError();
 }
 

@@ -535,7 +535,7 @@ cudaError_t launch_select(const float* logits, StepPtrs st, Workspace ws, RouteP
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   // Several groups and more rows than one CTA routes at once (one row per warp): the routing rounds run as
-  // one CTA per group (up to 32), the dispatch as a second single-CTA launch.
+  // one CTA per group (up to 128), the dispatch as a second single-CTA launch.
   const int group_ctas = d.G < 128 ? d.G : 128;
   if (d.T > kSelMaxWarps && (d.G == 1 || d.T / group_ctas > kSelMaxWarps)) {
     // one group, or groups of more rows than a CTA routes at once: one cluster, rows split over its CTAs
