@@ -15,10 +15,11 @@
 //   warps 9-12 loaders.  A tile that lies in the prefix is fetched by one thread with TMA boxes of [64 keys][64
 //              elements], swizzled on the way; tiles that reach into the block (prefix, fresh rows and in-block cache mixed)
 //              are stored by all four warps.  Keys are the K-major and values, stored the same way, the MN-major operand.
-// What bounds it: a tile of 64 keys and two M tiles takes 2100 clock cycles, of which the counters show the tensor pipe busy
-// for 1300 (S at N = 64 reads its A operand as long as it computes, and P counts twice) and the softmax needs 1300 (16
-// exponentials per clock and SM); the rest is hand-offs between the two.  Around the tiles: 6000 cycles until the first scores
-// and 5000 to 10000 for the merge, whose reads of distributed shared memory run at about 12 bytes per clock and SM.  Kernel
+// What bounds it (clock stamps at 1850 MHz, head size 128): a tile of 64 keys and two M tiles takes 2450 clock cycles (one M tile:
+// 1530), of which the counters show the tensor pipe busy for 1300 (S at N = 64 reads its A operand as long as it computes, and P
+// counts twice) and the softmax needs 1300 (16 exponentials per clock and SM); the rest is hand-offs between the two.  Around
+// the tiles of a split call with two M tiles: 8200 cycles until the first scores, 1900 to leave the partial result, 13000 for
+// the cluster's barriers and the merge, whose reads of distributed shared memory run at about 12 bytes per clock and SM.  Kernel
 // at 4096 cached tokens, 32 query and 4 key / value heads of 128, block of 32 x 4 branches: 43 us with one M tile per CTA,
 // loads through registers and P in shared memory, 25 now.
 // Every wait is an mbarrier wait with a limit; when one runs out the CTA stops working, reports TEAM_ERR_TIMEOUT and
@@ -759,9 +760,10 @@ static bool use_fragments(const AttnArgs& a, const AttnSetup& st, int tiles_max,
 
 template <int D>
 static cudaError_t launch(AttnArgs a, const AttnSetup& st, cudaStream_t s, bool* inserted) {
-  // One or two M tiles per CTA and how many CTAs split the keys: whatever should end first, by what was measured
-  // (clock cycles): a key tile takes 1500 for one M tile and 2100 for two, everything around the tiles 10000 per wave of
-  // clusters.  A decoded block has a quarter of its rows cached on average when delayed caching is on.  Where the clusters of
+  // One or two M tiles per CTA and how many CTAs split the keys: whatever should end first, at 1500 clock cycles for a key
+  // tile of one M tile, 2100 of two and 10000 around the tiles per wave of clusters, which were fitted to whole calls.  (Clock
+  // stamps inside one CTA give 1530, 2450 and 19000 to 25000, which overlap with the next wave's; with those the choice is
+  // another one for 1 of 80 random calls of up to 512 rows and 8192 cached tokens.)  A decoded block has a quarter of its rows cached on average when delayed caching is on.  Where the clusters of
   // three quarters of the rows just run at once, the first passes of a block take two waves (32 x 4 rows, 32 query and 4 key /
   // value heads of 128, 1500 cached tokens: 35 us in the first pass, 20 to 21 from the third on; 4096 tokens: 51, 27).
   const long long pairs = (long long)a.B * a.L * (a.Hq / a.Hkv), expected = (a.flags & TEAM_F_DCD) ? (3 * pairs + 3) / 4 : pairs;
