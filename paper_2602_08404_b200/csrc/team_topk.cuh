@@ -190,13 +190,10 @@ __device__ __forceinline__ float routing_weight(const TopkResult& r, int k, int 
   return p / s;
 }
 
-// A row routed: v holds its logits (-inf beyond E), of which the first NE per lane exist; `allowed` (null: all) restricts the
-// choice to a set of experts.  Returns lane j's routing weight.  The softmax denominator over all experts is formed only where
-// somebody needs it (`stats`).  Code that a CTA runs once is bound by its instruction fetches, so nothing is unrolled further
-// than the experts at hand need.
+// What a row's routing weights are formed from: its largest logit and, only where somebody needs it (`stats`), the softmax
+// denominator over all experts.  v holds its logits (-inf beyond E), of which the first NE per lane exist.
 template <int NE>
-__device__ __forceinline__ float route_logits(float (&v)[kMaxPerLane], const uint32_t* allowed, int k, int lane, int E, int norm_topk,
-                                              bool stats, bool margin, TopkResult& r, float& row_max, float& denom) {
+__device__ __forceinline__ void row_stats(const float (&v)[kMaxPerLane], int lane, int E, bool stats, float& row_max, float& denom) {
   float m = v[0];
 #pragma unroll
   for (int i = 1; i < NE; ++i) m = fmaxf(m, v[i]);
@@ -209,6 +206,14 @@ __device__ __forceinline__ float route_logits(float (&v)[kMaxPerLane], const uin
       if (i * 32 + lane < E) s += expf(v[i] - row_max);
     denom = warp_sum(s);
   }
+}
+
+// A row routed, from its logits and row_stats: `allowed` (null: all) restricts the choice to a set of experts.  Returns lane j's
+// routing weight.  Code that a CTA runs once is bound by its instruction fetches, so nothing is unrolled further than the
+// experts at hand need.
+template <int NE>
+__device__ __forceinline__ float route_logits(const float (&v)[kMaxPerLane], const uint32_t* allowed, int k, int lane, int norm_topk,
+                                              float row_max, float denom, bool margin, TopkResult& r) {
   float c[kMaxPerLane];
 #pragma unroll
   for (int i = 0; i < NE; ++i) c[i] = allowed == nullptr || ((allowed[i] >> lane) & 1u) ? v[i] : kNegInf;
