@@ -60,9 +60,13 @@ __host__ __device__ inline int padded_rows(int n) { return n / kTileChunk * kTil
 // the CTAs between 108 and 172 us of work.  A few such experts among many of one chunk (a shared expert) keep their CTAs busy
 // longer: half their rows are added then.  Without and with that, us: 185 rows and a shared expert 122.5, 116.5, 486 rows 180,
 // 152, 204 rows 174.5, 153; with it 2048 rows would take 330 in place of 305.
-__device__ __forceinline__ int tile_cost(int n, bool few_large) {
+// The same holds for an expert of one chunk with more than four times the mean (a shared expert of fewer rows): half its rows
+// are what its token tile adds to a step's bytes.  Without and with that, us, with a shared expert: 128 rows of one sequence
+// 131.3, 117.5, of 16 sequences 210.7, 198.7 (256 experts of 512 columns, hidden 2048), of one sequence 139.9, 130.1 (128 of 768).
+__device__ __forceinline__ int tile_cost(int n, bool few_large, int used, int total) {
   const int chunks = (n + kTileChunk - 1) / kTileChunk;
-  return chunks <= 1 ? chunks * 128 : (chunks + 1) / 2 * 256 + (few_large ? padded_rows(n) / 2 : 0);
+  const bool large = chunks <= 1 ? n > 32 && n * used > 4 * total : few_large;
+  return (chunks <= 1 ? chunks * 128 : (chunks + 1) / 2 * 256) + (large ? padded_rows(n) / 2 : 0);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -136,36 +140,38 @@ struct PlanSmem {
 };
 
 __device__ __forceinline__ void block_plan(const PlanSmem& s, const uint32_t* counts, int EN, int I, int H) {
-  __shared__ int2 s_tot[(kMaxExp + 31) / 32];
+  __shared__ int4 s_tot[(kMaxExp + 31) / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int used_warps = (EN + 31) >> 5;
   int n_slots = 0, rows_in = 0, cost_in = 0;
   if (warp < used_warps) {                                      // expert = thread
     n_slots = tid < EN ? (int)__ldcg(counts + tid) : 0;
     const int used = __popc(__ballot_sync(0xffffffffu, n_slots > 0)), large = __popc(__ballot_sync(0xffffffffu, n_slots > kTileChunk));
-    if (lane == 0) s_tot[warp] = make_int2(used, large);
+    const int total = __reduce_add_sync(0xffffffffu, n_slots);
+    if (lane == 0) s_tot[warp] = make_int4(used, large, total, 0);
   }
   __syncthreads();
-  int used = 0, large = 0;
+  int used = 0, large = 0, total = 0;
   for (int w = 0; w < used_warps; ++w) {
     used += s_tot[w].x;
     large += s_tot[w].y;
+    total += s_tot[w].z;
   }
   const bool few_large = 4 * large < used;
   __syncthreads();
   if (warp < used_warps) {
     rows_in = padded_rows(n_slots);
-    cost_in = tile_cost(n_slots, few_large);
+    cost_in = tile_cost(n_slots, few_large, used, total);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int r1 = __shfl_up_sync(0xffffffffu, rows_in, o), c1 = __shfl_up_sync(0xffffffffu, cost_in, o);
       if (lane >= o) { rows_in += r1; cost_in += c1; }
     }
-    if (lane == 31) s_tot[warp] = make_int2(rows_in, cost_in);
+    if (lane == 31) s_tot[warp] = make_int4(rows_in, cost_in, 0, 0);
   }
   __syncthreads();
   if (tid < EN) {
-    int rows = rows_in - padded_rows(n_slots), cost = cost_in - tile_cost(n_slots, few_large);
+    int rows = rows_in - padded_rows(n_slots), cost = cost_in - tile_cost(n_slots, few_large, used, total);
     for (int w = 0; w < warp; ++w) {
       rows += s_tot[w].x;
       cost += s_tot[w].y;
@@ -173,7 +179,7 @@ __device__ __forceinline__ void block_plan(const PlanSmem& s, const uint32_t* co
     s.n[tid] = n_slots;
     s.row0[tid] = rows;
     s.cost[tid] = cost;
-    if (tid == EN - 1) s.cost[EN] = cost + tile_cost(n_slots, few_large);
+    if (tid == EN - 1) s.cost[EN] = cost + tile_cost(n_slots, few_large, used, total);
   }
   __syncthreads();
   if (tid < 2) {
