@@ -140,8 +140,8 @@ __device__ __forceinline__ void route_class(int want, Logit logit, const Dims& d
     fetch(t);
     TopkResult r;
     float row_max, denom;
-    row_stats<NE>(v, lane, E, !p.norm_topk, row_max, denom);
-    const float w = route_logits<NE>(v, want == TEAM_CLS_COLD ? s.mask + g * 8 : nullptr, k, lane, p.norm_topk, row_max, denom, false, r);
+    const float w = route_logits<NE>(v, want == TEAM_CLS_COLD ? s.mask + g * 8 : nullptr, k, lane, E, p.norm_topk, !p.norm_topk, false, false, r,
+                                     row_max, denom);
     if (lane < k) {
       s.idx[cur * k + lane] = (int16_t)r.idx;
       s.w[cur * k + lane] = w;

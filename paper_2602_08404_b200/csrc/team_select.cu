@@ -160,8 +160,9 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
     }
   }
   // at most one row per warp: the row's logits are fetched once, as soon as they are there, and stay in registers through both
-  // rounds, with what the weights are formed from (formed in the rounds, the cold rows' came behind the others' choices:
-  // team_select_experts of 8 and 32 rows of 128 experts 11.2, 12.4 us, this way 10.4, 11.7)
+  // rounds, with the softmax denominators where somebody needs them (formed in the rounds, the cold rows' came behind the others'
+  // choices: team_select_experts of 8 and 32 rows of 128 experts 11.2, 12.4 us, this way 10.4, 11.7; the largest logit alone is
+  // left to the rounds: 11 rows of 199 experts without tables 32.2 us, formed here 32.35)
   if (mode == kSelRounds) __syncthreads();                  // the list of rows is complete
   const int n_mine = mode == kSelRounds ? s.own[T] : t1 - t0;
   const bool one_row_per_warp = mode != kSelDispatch && n_mine <= kSelWarps;
@@ -174,13 +175,12 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
 #pragma unroll
     for (int i = 0; i < kMaxPerLane; ++i) v[i] = i * 32 + lane < E ? __ldcg(logits + (size_t)t * E + i * 32 + lane) : kNegInf;
   };
-  auto stats_of = [&](const float (&v)[kMaxPerLane], float& row_max, float& denom) {
-    if (E <= 128) row_stats<4>(v, lane, E, stats, row_max, denom);
-    else row_stats<kMaxPerLane>(v, lane, E, stats, row_max, denom);
-  };
   if (one_row_per_warp && warp < n_mine) {
     load_logits(mode == kSelRounds ? s.own[warp] : t0 + warp, keep);
-    stats_of(keep, keep_max, keep_denom);
+    if (stats) {
+      if (E <= 128) row_stats<4>(keep, lane, E, true, keep_max, keep_denom);
+      else row_stats<kMaxPerLane>(keep, lane, E, true, keep_max, keep_denom);
+    }
   }
   if (mode == kSelDispatch) {
     // classes and choices were left in the routing tables by the kSelRounds grid
@@ -210,20 +210,18 @@ k_select(const float* __restrict__ logits, StepPtrs st, Workspace ws, RoutePtrs 
       }
       if ((round == 1 && c != TEAM_CLS_FIRST) || (round == 2 && c != TEAM_CLS_COLD)) continue;
       const int g = s.key[t] >> 8;
-      float v[kMaxPerLane], row_max, denom;
+      float v[kMaxPerLane], row_max = keep_max, denom = keep_denom;
       if (one_row_per_warp) {
 #pragma unroll
         for (int i = 0; i < kMaxPerLane; ++i) v[i] = keep[i];
-        row_max = keep_max;
-        denom = keep_denom;
       } else {
         load_logits(t, v);
-        stats_of(v, row_max, denom);
       }
       const uint32_t* allowed = round == 2 ? s.mask + g * n_words32 : nullptr;
+      const bool known = one_row_per_warp && stats;
       TopkResult tr;
-      const float w = E <= 128 ? route_logits<4>(v, allowed, k, lane, p.norm_topk, row_max, denom, ex.margin != nullptr, tr)
-                               : route_logits<kMaxPerLane>(v, allowed, k, lane, p.norm_topk, row_max, denom, ex.margin != nullptr, tr);
+      const float w = E <= 128 ? route_logits<4>(v, allowed, k, lane, E, p.norm_topk, stats, ex.margin != nullptr, known, tr, row_max, denom)
+                               : route_logits<kMaxPerLane>(v, allowed, k, lane, E, p.norm_topk, stats, ex.margin != nullptr, known, tr, row_max, denom);
       if (ex.probs) {
 #pragma unroll
         for (int i = 0; i < kMaxPerLane; ++i) {

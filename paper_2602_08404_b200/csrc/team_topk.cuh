@@ -208,12 +208,13 @@ __device__ __forceinline__ void row_stats(const float (&v)[kMaxPerLane], int lan
   }
 }
 
-// A row routed, from its logits and row_stats: `allowed` (null: all) restricts the choice to a set of experts.  Returns lane j's
-// routing weight.  Code that a CTA runs once is bound by its instruction fetches, so nothing is unrolled further than the
-// experts at hand need.
+// A row routed, from its logits and row_stats (formed here unless they are `known`): `allowed` (null: all) restricts the choice to
+// a set of experts.  Returns lane j's routing weight.  Code that a CTA runs once is bound by its instruction fetches, so nothing
+// is unrolled further than the experts at hand need.
 template <int NE>
-__device__ __forceinline__ float route_logits(const float (&v)[kMaxPerLane], const uint32_t* allowed, int k, int lane, int norm_topk,
-                                              float row_max, float denom, bool margin, TopkResult& r) {
+__device__ __forceinline__ float route_logits(const float (&v)[kMaxPerLane], const uint32_t* allowed, int k, int lane, int E, int norm_topk,
+                                              bool stats, bool margin, bool known, TopkResult& r, float& row_max, float& denom) {
+  if (!known) row_stats<NE>(v, lane, E, stats, row_max, denom);
   float c[kMaxPerLane];
 #pragma unroll
   for (int i = 0; i < NE; ++i) c[i] = allowed == nullptr || ((allowed[i] >> lane) & 1u) ? v[i] : kNegInf;
