@@ -45,8 +45,12 @@ constexpr int kStageBytes = 3 * kTileBytes;
 constexpr int kTileChunk = 128;                // token-slots per chunk at most (N of the MMA)
 constexpr int kTmemCols = 512;                 // two buffers of two accumulators of 128 columns
 constexpr int kEpiWarps = 8;                   // two warpgroups, one per accumulator of a step
+// Rows that a warp of kernel A lists once per expert, where kernel B keeps its slots' tables.  (16 KB more for all 2048 leave the
+// kernel in front no room on the SM: 0.4 us of calls of 270 and 480 rows.)
+constexpr int kListRows = 1024;
+static_assert(kLoadWarps * kListRows * 2 <= kEpiWarps * kTileChunk * 8, "lists in the place of the tables");
 constexpr int kMaxExp = TEAM_MAX_EXPERTS + TEAM_MAX_SHARED;
-constexpr int kTileSmemBytes = 1024 + kTileStages * kStageBytes + kEpiWarps * kTileChunk * 8 + 256 + (3 * kMaxExp + 8) * 4 + kLoadWarps * TEAM_MAX_ROWS * 2;
+constexpr int kTileSmemBytes = 1024 + kTileStages * kStageBytes + kEpiWarps * kTileChunk * 8 + 256 + (3 * kMaxExp + 8) * 4 + 2 * kTileChunk * 2;
 
 enum { kEpiSwiglu = 0, kEpiCombine = 1 };
 
@@ -293,11 +297,35 @@ struct TileWalk {
   __device__ __forceinline__ int n_of(int i) const { return nc == 2 && i ? slots[1] : slots[0]; }
 };
 
-// The rows of an expert's slots [begin, begin + n), by one warp: a slot's number is its row's rank among the expert's.  Two words
-// of 32 rows per lane are fetched and summed up, then every word with a slot of the range is spread over the lanes, one row each.
-// (Every lane its own words, bit by bit, 32 words at a time: 9000 clock cycles where half of 2048 rows chose the expert; 2048 rows
-// x 8 choices of 16 experts, hidden 256, 1024 columns 110.2 -> 101.6 us, 24 experts x 6 choices, hidden 1536, 704 columns 139.4 ->
-// 133.8.  A function of its own: inlined, the loop over the token rows came out slower, 141.2.)
+// The rows of an expert of one chunk, by one warp: a slot's number is its row's rank among the expert's.  Every lane walks the
+// bits of its own words: such an expert has few of a word's rows, or there are few words.
+__device__ __forceinline__ void list_chunk(uint16_t* list, const uint32_t* words, int W) {
+  const int lane = threadIdx.x & 31;
+  int run = 0;
+  __syncwarp();
+  for (int w0 = 0; w0 < W; w0 += 32) {
+    const int w = w0 + lane;
+    const uint32_t word = w < W ? __ldcg(words + w) : 0u;
+    int incl = __popc(word);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    int at = run + incl - __popc(word);
+    for (uint32_t m = word; m != 0u; m &= m - 1u, ++at)
+      if (at < kTileChunk) list[at] = (uint16_t)(w * 32 + __ffs(m) - 1);
+    run += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  __syncwarp();
+}
+
+// The rows of an expert's slots [begin, begin + n) where it has more than one chunk.  Two words of 32 rows per lane are fetched and
+// summed up; then, unless they have few bits each, every word with a slot of the range is spread over the lanes, one row each.
+// (Every lane its own words in any case: 9000 clock cycles where half of 2048 rows chose the expert; 2048 rows x 8 choices of 16
+// experts, hidden 256, 1024 columns 110.2 -> 101.6 us, 24 experts x 6 choices, hidden 1536, 704 columns 139.4 -> 133.8.  This way
+// in any case: 1020 rows and a shared expert 53.6 -> 54.3.  Functions of their own, and only for these experts: inlined, the
+// loop over the token rows came out slower, 141.2; for experts of one chunk 11 rows of 199 experts took 32.7 us in place of 31.7.)
 __device__ __noinline__ void list_rows(uint16_t* list, const uint32_t* words, int W, int begin, int n) {
   static_assert(TEAM_MAX_ROWS <= 64 * 32, "two words per lane");
   const int lane = threadIdx.x & 31;
@@ -317,6 +345,12 @@ __device__ __noinline__ void list_rows(uint16_t* list, const uint32_t* words, in
     before = __shfl_sync(0xffffffffu, end, 31);
     at = end - slots;                                          // rank of the word's first slot
     uint32_t m = __ballot_sync(0xffffffffu, slots > 0 && at < n && end > 0);
+    if ((int)__reduce_max_sync(0xffffffffu, (uint32_t)slots) <= 3 * ((__popc(m) + 3) >> 2)) {      // an exchange takes as long as 3 bits
+      for (uint32_t mine = word; mine != 0u; mine &= mine - 1u, ++at)
+        if (at >= 0 && at < n) list[at] = (uint16_t)(row0 + lane * 32 + __ffs(mine) - 1);
+      m = 0u;
+      __syncwarp();
+    }
 #pragma unroll 1
     while (m != 0u) {
 #pragma unroll
@@ -331,6 +365,32 @@ __device__ __noinline__ void list_rows(uint16_t* list, const uint32_t* words, in
   }
   __syncwarp();
 }
+
+// (output row, routing weight) of n token-slots of expert x (k choices per row, 0: a shared expert), for pass B, by one warp, with
+// the loads of a lane's four slots in flight together.
+__device__ __noinline__ void note_slots(int32_t* row_of, float* w_of, const uint16_t* list, int n, int x, const int32_t* topk_idx,
+                                        const float* topk_w, int k) {
+  constexpr int kPer = kTileChunk / 32;
+  const int lane = threadIdx.x & 31;
+  int row[kPer], choice[kPer];                   // choice -1: a shared expert
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    row[i] = lane + 32 * i < n ? list[lane + 32 * i] : -1;
+    choice[i] = -1;
+  }
+#pragma unroll 4
+  for (int c = 0; c < k; ++c)
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (row[i] >= 0 && __ldcg(topk_idx + row[i] * k + c) == x) choice[i] = c;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i)
+    if (row[i] >= 0) {
+      row_of[lane + 32 * i] = row[i];
+      w_of[lane + 32 * i] = choice[i] >= 0 ? __ldcg(topk_w + row[i] * k + choice[i]) : 1.f;
+    }
+}
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -465,16 +525,22 @@ __global__ void __launch_bounds__(EPI == kEpiSwiglu ? kTileThreadsA : kTileThrea
     // kLag stages later, when this thread's copies have landed and are made visible to the tensor core.
     constexpr int kLag = 2;
     const int lw = warp - 2 - kEpiWarps, piece = lane & 7, W = (a.T + 31) >> 5;
-    uint16_t* tok_list = reinterpret_cast<uint16_t*>(plan.n + 3 * kMaxExp + 8) + lw * TEAM_MAX_ROWS;      // rows of the expert's slots
+    uint16_t* tok_list = reinterpret_cast<uint16_t*>(tab_row) + lw * kListRows;      // rows of the expert's slots
     uint32_t it = 0;
     int cur_x = -1, cur_c = -1, cur_nc = 0;
     const __nv_bfloat16* src[2][8];
     bool ok = true;
     while (ok && wk.next()) {
       if (wk.x != cur_x || wk.c != cur_c || wk.nc != cur_nc) {
-        // every warp makes a list of its own, so that no warp waits for one that has given up; once per expert, although its chunks
-        // come again with every tile
-        if (wk.x != cur_x) list_rows(tok_list, a.bits + (size_t)wk.x * W1, W, 0, wk.n);
+        // every warp makes a list of its own, so that no warp waits for one that has given up; once per expert where it holds all
+        // of its rows, although the chunks come again with every tile
+        const bool all = wk.n <= kListRows;
+        if (wk.n <= kTileChunk) {
+          if (wk.x != cur_x) list_chunk(tok_list, a.bits + (size_t)wk.x * W1, W);
+        } else if (wk.x != cur_x || !all) {
+          list_rows(tok_list, a.bits + (size_t)wk.x * W1, W, all ? 0 : wk.c * kTileChunk, all ? wk.n : wk.nc * kTileChunk);
+        }
+        const uint16_t* chunk = tok_list + (all ? wk.c * kTileChunk : 0);
         cur_x = wk.x;
         cur_c = wk.c;
         cur_nc = wk.nc;
@@ -483,7 +549,7 @@ __global__ void __launch_bounds__(EPI == kEpiSwiglu ? kTileThreadsA : kTileThrea
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const int n = i * 16 + lw * 4 + (lane >> 3);
-            src[q][i] = q < wk.nc && n < wk.slots[q] ? a.x + (size_t)tok_list[(wk.c + q) * kTileChunk + n] * a.H + piece * 8 : nullptr;
+            src[q][i] = q < wk.nc && n < wk.slots[q] ? a.x + (size_t)chunk[q * kTileChunk + n] * a.H + piece * 8 : nullptr;
           }
       }
       for (int kb = 0; kb < NK; ++kb, ++it) {
@@ -532,33 +598,29 @@ __global__ void __launch_bounds__(EPI == kEpiSwiglu ? kTileThreadsA : kTileThrea
       const uint32_t buf = un & 1;
       const bool mine = half < wk.accs();
       const int j = wk.tile(half), first = wk.row(half), n_c = wk.n_of(half), np = pad16(n_c);
-      if (EPI == kEpiSwiglu && wk.j == (wk.c < 2 ? 0 : (wk.c >> 1) % a.tiles) && (ew & 3) == 0 && half < wk.nc) {
+      if (EPI == kEpiSwiglu && (ew & 3) == 0 && half < wk.nc && (wk.n <= kTileChunk ? wk.j == 0 : wk.j == (wk.c >> 1) % a.tiles)) {
         // (output row, routing weight) of the expert's slots for pass B, noted by the CTA of one of its tiles, another one for every
-        // pair of chunks: one warp per chunk, while it waits for the accumulators anyway, with the loads of a lane's four slots in
-        // flight together.  (All pairs at the first tile, one slot after the other: 2048 rows x 8 choices of 16 experts, hidden 256,
-        // 1024 columns 128.7 us, this way 110.2.)
-        uint16_t* list = reinterpret_cast<uint16_t*>(tab_row + ew * kTileChunk);
-        const int n_rows = wk.n_of(half), at = wk.first + half * kTileChunk;
-        list_rows(list, a.bits + (size_t)wk.x * W1, (a.T + 31) >> 5, (wk.c + half) * kTileChunk, n_rows);
-        constexpr int kPer = kTileChunk / 32;
-        int row[kPer], choice[kPer];                   // choice -1: a shared expert
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          row[i] = lane + 32 * i < n_rows ? list[lane + 32 * i] : -1;
-          choice[i] = -1;
-        }
-        if (wk.x < a.E)
+        // pair of chunks: one warp per chunk, while it waits for the accumulators anyway.  (All pairs at the first tile, one slot
+        // after the other: 2048 rows x 8 choices of 16 experts, hidden 256, 1024 columns 128.7 us, this way 110.2.)
+        uint16_t* list = reinterpret_cast<uint16_t*>(plan.n + 3 * kMaxExp + 8) + half * kTileChunk;
+        const uint32_t* bits = a.bits + (size_t)wk.x * W1;
+        const int n_rows = wk.n_of(half), at = wk.first + half * kTileChunk, W = (a.T + 31) >> 5;
+        if (wk.n <= kTileChunk) {
+          list_chunk(list, bits, W);
+          for (int n = lane; n < n_rows; n += 32) {
+            const int row = list[n];
+            int choice = -1;                             // -1: a shared expert
+            if (wk.x < a.E)
 #pragma unroll 4
-          for (int c = 0; c < a.k; ++c)
-#pragma unroll
-            for (int i = 0; i < kPer; ++i)
-              if (row[i] >= 0 && __ldcg(a.topk_idx + row[i] * a.k + c) == wk.x) choice[i] = c;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i)
-          if (row[i] >= 0) {
-            a.row_of[at + lane + 32 * i] = row[i];
-            a.w_of[at + lane + 32 * i] = choice[i] >= 0 ? __ldcg(a.topk_w + row[i] * a.k + choice[i]) : 1.f;
+              for (int i = 0; i < a.k; ++i)
+                if (__ldcg(a.topk_idx + row * a.k + i) == wk.x) choice = i;
+            a.row_of[at + n] = row;
+            a.w_of[at + n] = choice >= 0 ? __ldcg(a.topk_w + row * a.k + choice) : 1.f;
           }
+        } else {
+          list_rows(list, bits, W, (wk.c + half) * kTileChunk, n_rows);
+          note_slots(a.row_of + at, a.w_of + at, list, n_rows, wk.x, a.topk_idx, a.topk_w, wk.x < a.E ? a.k : 0);
+        }
       }
       if (EPI == kEpiCombine && mine && first != tab_first) {
         // (output row, weight) of the chunk's slots: every epilogue warp keeps a copy of its own, refilled at its own pace

@@ -17,6 +17,8 @@ CASES = {
     "100_rows_wide": replace(S, block=20, seqs=5, hidden=384, n_experts=250, top_k=4, inter=192, n_shared=2),
     "128_rows": replace(S, branches=4, inter=512),
     "129_rows": replace(S, block=43, seqs=3, hidden=640, inter=320),
+    # as many rows as a warp lists at once, of an expert with several chunks among small ones
+    "1024_rows": replace(S, seqs=32, n_experts=100, hidden=128, inter=64),
     # nobody has four times the mean
     "128_rows_of_3_experts": replace(S, branches=4, n_experts=3, top_k=1, n_shared=2),
 }
